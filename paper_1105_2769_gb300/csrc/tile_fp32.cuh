@@ -90,12 +90,14 @@ __device__ __forceinline__ bool build_table_entry(TabPair (*tab)[kTile / 2], int
     return bad;
 }
 
-// One row j against the 8 column pairs (16 columns k) held in registers:
+// One row j against the column pairs (8 of them, 16 columns k, unless P says
+// otherwise) held in registers:
 // the 14-operation loop of the header comment. Column pair p of the row is
 // xy[p * stride], zr[p * stride] (float4: (ex_k, ex_k+1, ey_k, ey_k+1) and
 // (ez_k, ez_k+1, rho_k, rho_k+1)). Adds q rho_ij to the column accumulators
 // acc[p] and returns the packed row sum sum_k q rho_ik (the caller multiplies
 // by rho_ij).
+template <int P = kPairs>
 __device__ __forceinline__ float2 row_half(const float4* xy, const float4* zr, int stride,
                                            const float2* vx, const float2* vy, const float2* vz,
                                            const float2* rk, float2* acc, float2 ux, float2 uy,
@@ -103,7 +105,7 @@ __device__ __forceinline__ float2 row_half(const float4* xy, const float4* zr, i
                                            float2 rij2) {
     float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int p = 0; p < kPairs; ++p) {
+    for (int p = 0; p < P; ++p) {
         const float4 t0 = xy[p * stride];
         const float4 t1 = zr[p * stride];
         const float2 wx = make_float2(t0.x, t0.y);
@@ -189,6 +191,73 @@ __device__ __forceinline__ float tile_triples(const TabPair (*tab)[kTile / 2], c
             const float2 c = f2_mul(acc[p], rk[p]);
             redK[kb + 2 * p][lane] = c.x;
             redK[kb + 2 * p + 1][lane] = c.y;
+        }
+    }
+    __syncwarp();
+    return acc_i;
+}
+
+// Triples of 32 particles i (one per lane, from any leaves) against a (J, K)
+// table of leaves of at most 32 points, in n_chunk passes of 2 P columns. A
+// leaf of n points needs n_chunk = 1 or 2 passes of ceil(n / (2 n_chunk))
+// column pairs and n rows, so that 17-point leaves pay for 17 x 20 columns and
+// not for 32 x 32 (the launch picks P). Order mask: points are numbered in the
+// tree's order, i < j is tested per row (i_rel = number of i minus that of
+// row 0), j < k is in the table, and i < k follows.
+//   redJ[jj][lane], redK[kk][lane]: as in tile_triples, rows jj < nJ only.
+template <int P>
+__device__ __forceinline__ float flat_triples(const TabPair (*tab)[kTile / 2], const float4* sJh,
+                                              const float4* sJl, const float4* sKh,
+                                              const float4* sKl, float4 ih, float4 il, bool iv,
+                                              int i_rel, int lane, int nJ, int nK, int n_chunk,
+                                              float (*redJ)[kTile + 1], float (*redK)[kTile + 1]) {
+    float acc_i = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < n_chunk; ++c) {
+        const int kb = c * 2 * P;
+        float2 vx[P], vy[P], vz[P], rk[P], acc[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            float e[2][4];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int kk = kb + 2 * p + q;
+                float s;
+                const PairF pr = pair_unit(ih, il, sKh[kk], sKl[kk], &s);
+                const bool v = iv && kk < nK && s > 0.f;
+                e[q][0] = v ? pr.ex : 0.f;
+                e[q][1] = v ? pr.ey : 0.f;
+                e[q][2] = v ? pr.ez : 0.f;
+                e[q][3] = v ? pr.rho : 0.f;
+            }
+            vx[p] = make_float2(e[0][0], e[1][0]);
+            vy[p] = make_float2(e[0][1], e[1][1]);
+            vz[p] = make_float2(e[0][2], e[1][2]);
+            rk[p] = make_float2(e[0][3], e[1][3]);
+            acc[p] = make_float2(0.f, 0.f);
+        }
+#pragma unroll 2
+        for (int jj = 0; jj < nJ; ++jj) {
+            float s;
+            const PairF pu = pair_unit(ih, il, sJh[jj], sJl[jj], &s);
+            const bool v = iv && i_rel < jj && s > 0.f;
+            const float ex = v ? pu.ex : 0.f, ey = v ? pu.ey : 0.f, ez = v ? pu.ez : 0.f;
+            const float rij = v ? pu.rho : 0.f;
+            const TabPair* row = tab[jj] + (kb >> 1);
+            const float2 s2 = row_half<P>(&row->xy, &row->zr, 2, vx, vy, vz, rk, acc, f2_splat(ex),
+                                          f2_splat(ey), f2_splat(ez), f2_splat(-3.0f * ex),
+                                          f2_splat(-3.0f * ey), f2_splat(-3.0f * ez),
+                                          f2_splat(rij));
+            const float srow = (s2.x + s2.y) * rij;
+            acc_i += srow;
+            if (c == 0) redJ[jj][lane] = srow;
+            else redJ[jj][lane] += srow;
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const float2 t = f2_mul(acc[p], rk[p]);
+            redK[kb + 2 * p][lane] = t.x;
+            redK[kb + 2 * p + 1][lane] = t.y;
         }
     }
     __syncwarp();
@@ -297,6 +366,21 @@ __device__ __forceinline__ float row_sum(const float (*red)[kTile + 1], int r) {
 #pragma unroll 8
     for (int m = 0; m < kTile; ++m) s += red[r][m];
     return s;
+}
+
+// The same sum carried with its rounding error (an exact two-term addition per
+// element), so that it does not depend on which particle sits in which lane.
+__device__ __forceinline__ double row_sum_exact(const float (*red)[kTile + 1], int r) {
+    float s = 0.f, c = 0.f;
+#pragma unroll 8
+    for (int m = 0; m < kTile; ++m) {
+        const float v = red[r][m];
+        const float t = __fadd_rn(s, v);
+        const float b = __fsub_rn(t, s);
+        c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+        s = t;
+    }
+    return (double)s + (double)c;
 }
 
 }  // namespace mbm_tile

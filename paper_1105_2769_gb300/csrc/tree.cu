@@ -312,13 +312,6 @@ seed_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int64_
 constexpr int kBaseWarps = 4;
 constexpr int kPiece = 64;
 
-// First particle of node v (recomputed where keeping it live costs registers).
-__device__ __noinline__ int64_t leaf_first(int64_t v, int64_t N) {
-    int64_t b, e;
-    node_range(v, N, b, e);
-    return b;
-}
-
 __device__ __forceinline__ unsigned leaf_triple_count(int x, int y, int z, unsigned n1,
                                                       unsigned n2, unsigned n3) {
     if (x == y && y == z) return n1 * (n1 - 1) * (n1 - 2) / 6;
@@ -392,13 +385,21 @@ struct BaseSmem {
     float redJ[kBaseWarps][kTile][kTile + 1];
     float redK[kBaseWarps][kTile][kTile + 1];
     double wsum[2][kBaseWarps][kTile];
-    long long b2, b3;  // first particle of the y and z leaves
+    long long b2, b3;        // first particle of the y and z leaves
+    int xfirst[kPiece];      // first particle of every x leaf of the piece
+    int xoff[kPiece + 1];    // particles of the x leaves before it
     int Y, Z, n2, n3, st, en;
 };
 
+// P column pairs per pass, n_chunk passes (2 P n_chunk >= the largest leaf).
+// The particles of a piece's x leaves are numbered through and dealt to lanes
+// 32 at a time, so that lanes are full whatever the leaf size: with one x
+// leaf per sweep, leaves of 17.6 points (N = 9 000) used 18 of 32 lanes and,
+// with 32 rows and 32 columns, one triple slot in six. FP32-pipe bound.
+template <int P>
 __global__ void __launch_bounds__(kBaseWarps * 32, 4)
 base_group_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int64_t N,
-                  int64_t first_leaf, int d, const ull* __restrict__ key,
+                  int64_t first_leaf, int d, int n_chunk, const ull* __restrict__ key,
                   const int* __restrict__ val, const int* __restrict__ heads,
                   const int* __restrict__ n_pieces_p, unsigned* __restrict__ piece_ctr,
                   double* __restrict__ acc, int* __restrict__ flags) {
@@ -438,15 +439,43 @@ base_group_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, 
             const int kk = threadIdx.x - kTile, n3 = sm.n3;
             sm.sKh[kk] = kk < n3 ? xh[sm.b3 + kk] : z4;
             sm.sKl[kk] = kk < n3 ? xl[sm.b3 + kk] : z4;
+        } else if (warp == 2) {
+            // offsets of the piece's x leaves (two per lane, kPiece = 64)
+            const int cnt = sm.en - sm.st;
+            int n[2], first[2];
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+                const int q = 2 * lane + o;
+                n[o] = 0;
+                first[o] = 0;
+                if (q < cnt) {
+                    int64_t b1, e1;
+                    node_range(val[sm.st + q], N, b1, e1);
+                    n[o] = (int)(e1 - b1);
+                    first[o] = (int)b1;
+                }
+            }
+            int incl = n[0] + n[1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int excl = incl - n[0] - n[1];
+            sm.xfirst[2 * lane] = first[0];
+            sm.xfirst[2 * lane + 1] = first[1];
+            sm.xoff[2 * lane] = excl;
+            sm.xoff[2 * lane + 1] = excl + n[0];
+            if (lane == 31) sm.xoff[kPiece] = incl;
         }
         __syncthreads();
         bool bad = false;
         {
             const int n2 = sm.n2, n3 = sm.n3;
             const bool e23 = sm.Y == sm.Z;
-            for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) {
+            for (int e = threadIdx.x; e < n2 * kTile; e += blockDim.x) {
                 const int jj = e >> 5, kk = e & 31;
-                const bool v = jj < n2 && kk < n3 && (!e23 || jj < kk);
+                const bool v = kk < n3 && (!e23 || jj < kk);
                 bad |= mbm_tile::build_table_entry(sm.tab, jj, kk, sm.sJh[jj], sm.sJl[jj],
                                                    sm.sKh[kk], sm.sKl[kk], v);
             }
@@ -455,22 +484,28 @@ base_group_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, 
         __syncthreads();
         sm.wsum[0][warp][lane] = 0.0;
         sm.wsum[1][warp][lane] = 0.0;
-        const int en = sm.en;
-        for (int q = sm.st + warp; q < en; q += kBaseWarps) {
-            const int X = val[q];
-            int64_t b1, e1;
-            node_range(X, N, b1, e1);
-            const int n1 = (int)(e1 - b1);
-            const bool iv = lane < n1;
-            const float4 ih = iv ? xh[b1 + lane] : z4;
-            const float4 il = iv ? xl[b1 + lane] : z4;
-            const float acc_i = mbm_tile::tile_triples(sm.tab, sm.sJh, sm.sJl, sm.sKh, sm.sKl, ih,
-                                                       il, iv, lane, sm.n2, sm.n3, X == sm.Y,
-                                                       X == sm.Z, sm.redJ[warp], sm.redK[warp]);
-            sm.wsum[0][warp][lane] += (double)mbm_tile::row_sum(sm.redJ[warp], lane);
-            sm.wsum[1][warp][lane] += (double)mbm_tile::row_sum(sm.redK[warp], lane);
+        const int total = sm.xoff[kPiece];
+        for (int f0 = warp * 32; f0 < total; f0 += kBaseWarps * 32) {
+            const bool iv = f0 + lane < total;
+            int pos = 0;  // the lane's particle
+            if (iv) {
+                int lo = 0;  // last leaf with xoff <= f (empty slots repeat the total)
+#pragma unroll
+                for (int w = kPiece / 2; w > 0; w >>= 1)
+                    if (sm.xoff[lo + w] <= f0 + lane) lo += w;
+                pos = sm.xfirst[lo] + (f0 + lane - sm.xoff[lo]);
+            }
+            const float4 ih = iv ? xh[pos] : z4;
+            const float4 il = iv ? xl[pos] : z4;
+            const float acc_i = mbm_tile::flat_triples<P>(
+                sm.tab, sm.sJh, sm.sJl, sm.sKh, sm.sKl, ih, il, iv, pos - (int)sm.b2, lane, sm.n2,
+                sm.n3, n_chunk, sm.redJ[warp], sm.redK[warp]);
+            // the lanes hold whatever leaves the list brought together: sums
+            // over them must not depend on that order
+            if (lane < sm.n2) sm.wsum[0][warp][lane] += mbm_tile::row_sum_exact(sm.redJ[warp], lane);
+            if (lane < sm.n3) sm.wsum[1][warp][lane] += mbm_tile::row_sum_exact(sm.redK[warp], lane);
             __syncwarp();
-            if (iv) atomicAdd(&acc[leaf_first(X, N) + lane], (double)acc_i);
+            if (iv) atomicAdd(&acc[pos], (double)acc_i);
         }
         __syncthreads();
         if (warp < 2) {
@@ -482,6 +517,24 @@ base_group_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, 
             if (lane < nn) atomicAdd(&acc[b + lane], tot);
         }
         __syncthreads();
+    }
+}
+
+using BaseGroupFn = void (*)(const float4*, const float4*, int64_t, int64_t, int, int, const ull*,
+                             const int*, const int*, const int*, unsigned*, double*, int*);
+
+// Passes and column pairs per pass for leaves of at most n points.
+BaseGroupFn base_group_for(int n, int& n_chunk) {
+    n_chunk = n > 16 ? 2 : 1;
+    switch ((n + 2 * n_chunk - 1) / (2 * n_chunk)) {
+        case 1: return base_group_kernel<1>;
+        case 2: return base_group_kernel<2>;
+        case 3: return base_group_kernel<3>;
+        case 4: return base_group_kernel<4>;
+        case 5: return base_group_kernel<5>;
+        case 6: return base_group_kernel<6>;
+        case 7: return base_group_kernel<7>;
+        default: return base_group_kernel<8>;
     }
 }
 
@@ -2232,14 +2285,16 @@ static mbm_status tree_solve(mbm_ctx* ctx, const double* X, int64_t N, double ep
     p.pt_acc3 = pt_acc3;
 
     const size_t bsm = sizeof(BaseSmem);
-    MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)base_group_kernel,
+    int n_chunk = 1;
+    const BaseGroupFn base_group = base_group_for((int)((N + n_leaves - 1) / n_leaves), n_chunk);
+    MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)base_group,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm));
     if (F)
         MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)base_forces_kernel,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)(sizeof(ForceWarpSmem) * kForceWarps)));
     int base_per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&base_per_sm, base_group_kernel,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&base_per_sm, base_group,
                                                       kBaseWarps * 32, bsm) != cudaSuccess ||
         base_per_sm < 1)
         base_per_sm = 1;
@@ -2278,8 +2333,8 @@ static mbm_status tree_solve(mbm_ctx* ctx, const double* X, int64_t N, double ep
         MBM_CUDA_TRY(mbm_exclusive_scan_i32(bflag, bpos, n, sort_tmp, s));
         base_piece_heads_kernel<<<grid_of(n, 256), 256, 0, s>>>(bflag, bpos, n, bheads, bmeta);
         MBM_CUDA_TRY(cudaMemsetAsync(bmeta + 1, 0, sizeof(int), s));
-        base_group_kernel<<<base_grid, kBaseWarps * 32, bsm, s>>>(
-            tree->xh, tree->xl, N, first_leaf, d, bkey2, bval2, bheads, bmeta,
+        base_group<<<base_grid, kBaseWarps * 32, bsm, s>>>(
+            tree->xh, tree->xl, N, first_leaf, d, n_chunk, bkey2, bval2, bheads, bmeta,
             reinterpret_cast<unsigned*>(bmeta + 1), pt_acc, ctx->d_flags);
         MBM_CUDA_TRY(cudaGetLastError());
         if (tm.on) {
