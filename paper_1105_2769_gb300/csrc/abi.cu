@@ -6,6 +6,7 @@
 #include <new>
 #include <string>
 
+#include "contract.h"
 #include "mbm_internal.h"
 #include "mbm_tree_api.h"
 
@@ -192,6 +193,18 @@ constexpr int64_t kPairTableMaxN = 65536;
 static mbm_status run_exhaustive(mbm_ctx* ctx, const double* X, int64_t N, int mode, double* phi,
                                  int validate, cudaStream_t s) {
     const size_t hdr = 256;  // work counter
+    if (mode == MBM_EXH_FP32 && N >= kContractMinPhi) {
+        bool done = false;
+        MbmGate g;
+        MBM_TRY(mbm_contract(ctx, X, N, nullptr, MBM_CONTRACT_PHI, 1.0, phi, s, &done, &g));
+        if (done) {
+            MBM_CUDA_TRY(launch_exh_fp32(g.xh, g.xl, N, phi, g.counter, ctx->d_flags, ctx->num_sms,
+                                         s, g.gate));
+            mbm_time_end(ctx, s);
+            if (validate) return mbm_check_flags(ctx, s);
+            return MBM_OK;
+        }
+    }
     if (mode == MBM_EXH_FP32 && N <= kPairTableMaxN) {
         const size_t tb = pair_table_bytes(N);
         const mbm_status rs = mbm_scratch_reserve(ctx, hdr + tb);

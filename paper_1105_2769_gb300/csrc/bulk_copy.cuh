@@ -28,6 +28,11 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long* bar, u
                  : "memory");
 }
 
+// Arrive on the barrier.
+__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // Copy `bytes` (a multiple of 16; both addresses 16-byte aligned) from global
 // to shared memory; completion is counted on `bar`.
 __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, unsigned bytes,

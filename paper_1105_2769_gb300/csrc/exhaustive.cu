@@ -76,7 +76,8 @@ struct Fp32Smem {
 __global__ void __launch_bounds__(kWarps32 * 32, 2)
 exh_fp32_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int NT,
                 long long n_items, unsigned long long* __restrict__ counter,
-                double* __restrict__ phi, int* __restrict__ flags) {
+                double* __restrict__ phi, int* __restrict__ flags, const int* __restrict__ gate) {
+    if (gate && !*gate) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Fp32Smem& sm = *reinterpret_cast<Fp32Smem*>(smem_raw);
     const int lane = threadIdx.x & 31;
@@ -521,7 +522,7 @@ cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* fl
 
 cudaError_t launch_exh_fp32(const float4* xhi, const float4* xlo, int64_t N, double* phi,
                             unsigned long long* counter, int* flags, int num_sms,
-                            cudaStream_t s) {
+                            cudaStream_t s, const int* gate) {
     const int NT = (int)((N + kTile - 1) / kTile);
     const long long items = (long long)NT * (NT + 1) / 2;
     const int threads = kWarps32 * 32;
@@ -530,7 +531,8 @@ cudaError_t launch_exh_fp32(const float4* xhi, const float4* xlo, int64_t N, dou
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = grid_for((const void*)exh_fp32_kernel, threads, smem, num_sms, items);
-    exh_fp32_kernel<<<grid, threads, smem, s>>>(xhi, xlo, (int)N, NT, items, counter, phi, flags);
+    exh_fp32_kernel<<<grid, threads, smem, s>>>(xhi, xlo, (int)N, NT, items, counter, phi, flags,
+                                                gate);
     return cudaGetLastError();
 }
 

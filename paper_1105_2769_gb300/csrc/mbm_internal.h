@@ -83,9 +83,10 @@ cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* fl
 
 // Exhaustive sums (steps a2/a3). phi must be zeroed by the caller.
 // counter: one zeroed unsigned long long of scratch for dynamic scheduling.
+// gate: NULL, or a device word; the kernel runs only if it is set.
 cudaError_t launch_exh_fp32(const float4* xhi, const float4* xlo, int64_t N, double* phi,
                             unsigned long long* counter, int* flags, int num_sms,
-                            cudaStream_t s);
+                            cudaStream_t s, const int* gate = nullptr);
 // Pair table of the FP32-bulk sum (unit vector and r^-3 of every pair, FP64
 // rounded once to FP32): its size, its build from X, and the sum that reads it.
 size_t pair_table_bytes(int64_t N);

@@ -29,6 +29,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "contract.h"
 #include "mbm_internal.h"
 #include "mbm_tree_api.h"
 
@@ -74,11 +75,18 @@ struct Worker {
     unsigned long long* h_stamp = nullptr;  // pinned host copy
 };
 
-size_t estimate_bytes(const mbm_request& r, const mbm_config& c) {
+// The contraction's scratch counts where the budget can hold it; a smaller
+// budget admits the request as before and the solve finds its own room.
+size_t estimate_bytes(const mbm_request& r, const mbm_config& c, size_t budget) {
     const size_t N = (size_t)r.N;
     const size_t io = N * 24 + N * (r.kind == MBM_REQ_FORCES ? 24 : 8);
     const int base = r.mode & 0xff;
-    if (base != MBM_TREE) return io + N * 32 + 4096;
+    if (base != MBM_TREE) {
+        const size_t least = io + N * 32 + 4096;
+        const size_t more =
+            base == MBM_EXH_FP32 ? mbm_contract_bytes(r.N, r.kind == MBM_REQ_FORCES) : 0;
+        return budget && least + more > budget ? least : least + more;
+    }
     return io + mbm_tree_solve_bytes(r.N, c, r.kind == MBM_REQ_FORCES) + (1 << 20);
 }
 
@@ -388,7 +396,7 @@ extern "C" mbm_status mbm_submit(mbm_server* s, const mbm_request* req, uint64_t
     if (req->cfg) job.cfg = *req->cfg;
     else mbm_config_default(&job.cfg);
     job.req.cfg = nullptr;
-    job.est = estimate_bytes(job.req, job.cfg);
+    job.est = estimate_bytes(job.req, job.cfg, s->budget);
     job.submitted = clk::now();
     std::unique_lock<std::mutex> lock(s->mu);
     if (s->budget && job.est > s->budget) {
