@@ -11,8 +11,8 @@
 // G = (u.v)(u.w)(v.w), u = x_j - x_i, v = x_k - x_i, w = x_k - x_j.)
 //
 // FP32 gradients of kContractMinForces and more particles are a tensor-core contraction
-// (contract.cu), 12 times faster at N = 8 192; what follows serves FP64, small N,
-// sets that the contraction's error bound turns away and scratch too small for it.
+// (contract.cu), 20 times faster at N = 8 192; what follows serves FP64, small N
+// and scratch too small for it.
 //
 // Gather form: a lane owns particle i and sums grad_i over every pair j < k
 // of the set (pairs through i drop out: their distance is exactly zero), so

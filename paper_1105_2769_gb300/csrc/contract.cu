@@ -18,59 +18,58 @@
 // solutions the one of least sum_r |l_r|^6 is taken, which keeps the cancellation
 // between the ten terms small.
 //
-// Precision. The tensor cores multiply fp16 exactly and add in FP32 with
-// truncation, which would lose 1e-7 of a sum per 16 terms. Each row of L is
-// therefore cut into three pieces against a power of two a per row and window
-// of 64 columns, |a L| <= 2^15: h, a multiple of 2^7 (8 bits), the rounding m of
-// the rest to fp16 and the rounding l of what is left. Products h h are integers
-// in units of 2^14, so their sums over a window are exact (measured: bit-exact
-// up to 256 columns); the other products but l l go to a second accumulator,
-// whose truncation is 2^-8 smaller where h carries the value. Both are added to
-// FP32 sums (round to nearest) window by window. Median error against 64 bits at
-// N = 2 600 (in brackets the FP32 triple sweep): potentials 4.1e-8 (5.6e-8) on
-// uniform sets, 8.1e-8 (1.0e-7) in the unit cube, 7.9e-8 (9.7e-8) on mixtures;
-// forces 2.7e-7 (3.4e-7), 2.6e-7 (3.3e-7), 2.6e-7 (3.8e-7). Windows of 256 columns
-// were 10 % faster but off by 1.7e-6 on a mixture.
-// Pieces have a floor relative to the largest entry of their window, so a set
-// whose tightest pairs are 50 times closer than everything around them loses
-// digits (isolated dimers at 1/100: 7e-6). The pair pass sums a bound of that
-// error next to the terms' magnitudes; a set over the bound is solved again by
-// the FP32 sweep behind it, decided on the device (gate), and that sweep returns
-// at once otherwise.
+// Precision. Each particle's four nearest neighbours are left out of the matrices
+// and the triples that hold such a pair are summed term by term (near.cu): they
+// carry 90-97 % of a potential and all of its large terms. The rest is smooth. A
+// row of L is cut against a power of two a per row and 256 columns, |a L| <= 2^15,
+// into h = fp16(a L) and l = fp16(2^11 (a L - h)): 22 bits. The tensor cores
+// multiply fp16 exactly and add in FP32 with truncation (8e-8 of a sum per 16
+// terms, measured), so h h is read out every 64 columns, h l + l h (2^-11 smaller)
+// every 256, and both are added in FP32, round to nearest. l l is left out. Median
+// error against 64 bits at N = 2 600 (in brackets the FP32 triple sweep):
+// potentials 1.7e-8 (5.6e-8) on uniform sets, 2.5e-8 (1.0e-7) in the unit cube,
+// 2.8e-8 (9.7e-8) on mixtures; forces 1.6e-7 (3.4e-7), 1.9e-7 (3.3e-7), 2.1e-7
+// (3.8e-7). Without the split, three pieces and eight products were needed for the
+// sweep's accuracy: forces of 8 192 particles took 29 ms against 16.
+// A set with more than 16 near pairs per particle (many equal distances) is left
+// to the FP32 sweep behind, decided on the device (gate); that sweep returns at
+// once otherwise.
 //
-// Kernels: window maxima -> scales; piece table (stored in the operand layout,
-// so a stage is two kinds of bulk copies and no tensor map); contraction
-// (tcgen05.mma 128 x 256, warp-specialised, persistent); pair pass over the
-// tiles' C. Large N runs in slabs of columns k and batches of tiles; all sums
-// are linear in both.
+// Kernels: near pairs (near.cu); block maxima -> scales; piece table (stored in
+// the operand layout, so a stage is two kinds of bulk copies and no tensor map);
+// contraction (tcgen05.mma 128 x 256, warp-specialised, persistent); pair pass
+// over the tiles' C; near triples. Large N runs in slabs of columns k and batches
+// of tiles; all sums are linear in both.
 #include <algorithm>
 #include <cuda_fp16.h>
 
 #include "bulk_copy.cuh"
 #include "contract.h"
 #include "device_math.cuh"
+#include "dfloat.cuh"
+#include "near.h"
 #include "tcgen05.cuh"
 #include "tile_fp32.cuh"
 
 namespace {
 
 constexpr int kForms = 10;
-constexpr int kPieces = 3;
-constexpr int kBlk = 256;      // rows per table block, and columns per scale block
+constexpr int kPieces = 2;
+constexpr int kBlk = 256;      // rows per table block, and columns that share a scale
 constexpr int kBM = 128;       // tile rows
 constexpr int kBN = 256;       // tile columns
 constexpr int kBK = 32;        // columns k per pipeline stage
 constexpr int kKbPerBlk = kBlk / kBK;
-constexpr int kWin = 64;       // columns k that share a scale and an accumulator window
+constexpr int kWin = 64;       // columns k per read-out of h h
 constexpr int kKbPerWin = kWin / kBK;
 constexpr int kWinPerBlk = kBlk / kWin;
-// Factor slots: a window's factors are copied when the MMAs of the window two
-// before it are done, which waited for the accumulators of the one three before.
-constexpr int kFactorSlots = 4;
-constexpr int kFlush = 8;      // windows summed in registers before C takes them
 constexpr int kPieceB = kBN * kBK * 2;  // 16 KB: one piece of 256 rows x 32 columns
 constexpr int kPieceA = kBM * kBK * 2;
-constexpr int kStages = 3;
+constexpr int kStages = 4;
+// Factor slots: a block's factors are copied when at most half a block of MMAs is
+// in flight, which waited for the accumulators of the block before.
+constexpr int kFactorSlots = 4;
+constexpr float kLowScale = 1.0f / 2048.0f;
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 2) * 32;
 constexpr int kGroup = 8;  // J tiles walked together: their rows and 19 I tiles stay in L2
@@ -135,35 +134,6 @@ __device__ __forceinline__ void form_value(const float (&ch)[5], const float (&c
     }
 }
 
-// ----- double-float helpers -----
-struct df {
-    float h, l;
-};
-__device__ __forceinline__ df df_fast(float a, float b) {  // |a| >= |b|
-    const float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ df df_mul(df a, df b) {
-    const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, e);
-    e = __fmaf_rn(a.l, b.h, e);
-    return df_fast(p, e);
-}
-__device__ __forceinline__ df df_add(df a, df b) {
-    const float s = __fadd_rn(a.h, b.h);
-    const float t = __fsub_rn(s, a.h);
-    float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
-    e = __fadd_rn(e, __fadd_rn(a.l, b.l));
-    return df_fast(s, e);
-}
-__device__ __forceinline__ df df_diff(float qh, float ql, float ph, float pl) {
-    const float s = __fsub_rn(qh, ph);
-    const float t = __fsub_rn(s, qh);
-    const float e = __fsub_rn(__fsub_rn(qh, __fsub_rn(s, t)), __fadd_rn(ph, t));
-    return df_fast(s, __fadd_rn(e, __fsub_rn(ql, pl)));
-}
-
 // Pair terms to about 2^-40: v = (Exx - Ezz, Eyy - Ezz, Exy, Exz, Eyz) and
 // rho = r^-3. False if the pair is coincident or not finite (terms then zero).
 struct PairDf {
@@ -178,12 +148,7 @@ __device__ __forceinline__ bool pair_df(float4 ph, float4 pl, float4 qh, float4 
     const df s = df_add(df_add(xx, yy), zz);
     o.s = s.h;
     if (!(s.h > 0.f) || !(s.h < INFINITY)) return false;
-    // 1/r: hardware estimate and one Newton step, kept as a two-term number
-    const float y0 = rsqrtf(s.h);
-    const float p = __fmul_rn(y0, y0), pe = __fmaf_rn(y0, y0, -p);
-    const float q = __fmul_rn(s.h, p), qe = __fmaf_rn(s.h, p, -q);
-    const float res = __fsub_rn(__fsub_rn(1.0f, q), __fmaf_rn(s.l, p, __fmaf_rn(s.h, pe, qe)));
-    const df y = df_fast(y0, __fmul_rn(__fmul_rn(0.5f, y0), res));
+    const df y = df_rsqrt(s);
     const df y2 = df_mul(y, y);
     o.y = y.h;
     o.rho = df_mul(y2, y);
@@ -202,43 +167,40 @@ __device__ __forceinline__ float pow2f(int e) {  // 2^e, 0 below the normal rang
 }
 
 // ---------------------------------------------------------------------------
-// Scales. ea[w][i]: exponent of a(i, w), the power of two with |a l| <= 2^15
-// over the 64 columns k of window w (times |g_k| for the weighted table). A
-// CTA takes 256 rows and one window; its columns are staged in shared memory.
+// Scales. ea[b][i]: exponent of a(i, b), the power of two with |a l| <= 2^15 over
+// the 256 columns k of block b without near pairs (times |g_k| for the weighted
+// table). A CTA takes 256 rows and one block, its columns in shared memory.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlk)
-scale_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int w0,
-             const double* __restrict__ g, int n_pad, int* __restrict__ ea,
-             int* __restrict__ row_ea, int* __restrict__ flags) {
-    __shared__ float4 kh[kWin], kl[kWin];
-    __shared__ float kg[kWin];
-    const int w = blockIdx.y, k0 = (w0 + w) * kWin;
+scale_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int b0,
+             const float* __restrict__ tau, const double* __restrict__ g, int n_pad,
+             int* __restrict__ ea, int* __restrict__ row_ea) {
+    __shared__ float4 kh[kBlk], kl[kBlk];
+    __shared__ float kg[kBlk], kt[kBlk];
+    const int b = blockIdx.y, k0 = (b0 + b) * kBlk;
     const int i = blockIdx.x * kBlk + threadIdx.x;
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (threadIdx.x < kWin) {
-        const int kk = k0 + threadIdx.x;
-        kh[threadIdx.x] = kk < N ? xh[kk] : z4;
-        kl[threadIdx.x] = kk < N ? xl[kk] : z4;
-        kg[threadIdx.x] = g && kk < N ? fabsf((float)g[kk]) : 1.f;
-    }
+    const int kk = k0 + threadIdx.x;
+    kh[threadIdx.x] = kk < N ? xh[kk] : z4;
+    kl[threadIdx.x] = kk < N ? xl[kk] : z4;
+    kt[threadIdx.x] = kk < N ? tau[kk] : 0.f;
+    kg[threadIdx.x] = g && kk < N ? fabsf((float)g[kk]) : 1.f;
     __syncthreads();
     const float4 ih = i < N ? xh[i] : z4, il = i < N ? xl[i] : z4;
-    const int cnt = min(kWin, N - k0);
-    float best = 0.f;  // largest rho (or |g| rho) of the window
-    bool bad = false;
+    const float ti = i < N ? tau[i] : 0.f;
+    const int cnt = min(kBlk, N - k0);
+    float best = 0.f;  // largest rho (or |g| rho) of the block
     if (i < N) {
         float smin = INFINITY;
         for (int q = 0; q < cnt; ++q) {
             const float s = pair_d2_hilo(ih, il, kh[q], kl[q]);
-            const bool self = k0 + q == i;
-            bad |= !self && !(s > 0.f);
-            if (!self && s > 0.f && s < INFINITY) {
-                if (g) {
-                    const float y = rsqrtf(s);
-                    best = fmaxf(best, kg[q] * (y * y * y));
-                } else {
-                    smin = fminf(smin, s);
-                }
+            // (the particle itself has s = 0 <= tau)
+            if (mbm_is_near(s, ti, kt[q]) || !(s < INFINITY)) continue;
+            if (g) {
+                const float y = rsqrtf(s);
+                best = fmaxf(best, kg[q] * (y * y * y));
+            } else {
+                smin = fminf(smin, s);
             }
         }
         if (!g && smin < INFINITY) {
@@ -246,11 +208,10 @@ scale_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
             best = y * y * y;
         }
     }
-    if (bad && !g) atomicOr(flags, MBM_FLAG_COINCIDENT);
-    int e = 127;  // nothing in this window
+    int e = 127;  // nothing in this block
     if (best > 0.f && best < INFINITY) e = 14 - ilogbf(best * (kFormMax * 1.0001f));
     if (best > 0.f) e = max(-120, min(126, e));
-    ea[(size_t)w * n_pad + i] = e;
+    ea[(size_t)b * n_pad + i] = e;
     if (i < N) atomicMin(&row_ea[i], e);
 }
 
@@ -263,26 +224,14 @@ __global__ void ref_kernel(const int* __restrict__ row_ea, int N, int* __restric
     if ((threadIdx.x & 31) == 0) atomicMin(ref, m);
 }
 
-// f[w][i] = 2^(row exponent - window exponent) <= 1; for the error bound its
-// maximum over the four windows of a 256-column block, fb[b][i], and that
-// maximum over 16 rows, fb16[b][i / 16].
+// f[b][i] = 2^(row exponent - block exponent) <= 1.
 __global__ void __launch_bounds__(kBlk)
 factor_kernel(const int* __restrict__ ea, const int* __restrict__ row_ea, int n_pad, int N,
-              float* __restrict__ f, float* __restrict__ fb, float* __restrict__ fb16) {
-    const int b = blockIdx.y, i = blockIdx.x * kBlk + threadIdx.x;
-    const int er = i < N ? row_ea[i] : 0;
-    float m = 0.f;
-    for (int q = 0; q < kWinPerBlk; ++q) {
-        const size_t o = (size_t)(b * kWinPerBlk + q) * n_pad + i;
-        const int e = ea[o];
-        const float v = i < N && e < 127 ? pow2f(er - e) : 0.f;
-        f[o] = v;
-        m = fmaxf(m, v);
-    }
-    fb[(size_t)b * n_pad + i] = m;
-    if (!fb16) return;
-    for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 15) == 0) fb16[(size_t)b * (n_pad / 16) + i / 16] = m;
+              float* __restrict__ f) {
+    const int i = blockIdx.x * kBlk + threadIdx.x;
+    const size_t o = (size_t)blockIdx.y * n_pad + i;
+    const int e = ea[o];
+    f[o] = i < N && e < 127 ? pow2f(row_ea[i] - e) : 0.f;
 }
 
 // ---------------------------------------------------------------------------
@@ -295,11 +244,11 @@ factor_kernel(const int* __restrict__ ea, const int* __restrict__ row_ea, int n_
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlk)
 table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int b0,
-             const double* __restrict__ g, int n_pad, int nb, int nkb, const int* __restrict__ ea,
+             const float* __restrict__ tau, const double* __restrict__ g, int n_pad, int nb, int nkb, const int* __restrict__ ea,
              unsigned char* __restrict__ T) {
     __shared__ FormCoef fc;
     __shared__ float4 kh[kBK], kl[kBK];
-    __shared__ float kg[kBK], kgl[kBK];
+    __shared__ float kg[kBK], kgl[kBK], kt[kBK];
     const int rb = blockIdx.x, kb = blockIdx.y;
     const int k0 = b0 * kBlk + kb * kBK;
     const int row = threadIdx.x, i = rb * kBlk + row;
@@ -312,6 +261,7 @@ table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
         const int k = k0 + threadIdx.x;
         kh[threadIdx.x] = k < N ? xh[k] : z4;
         kl[threadIdx.x] = k < N ? xl[k] : z4;
+        kt[threadIdx.x] = k < N ? tau[k] : 0.f;
         const double gk = g && k < N ? g[k] : 1.0;
         kg[threadIdx.x] = (float)gk;
         kgl[threadIdx.x] = (float)(gk - (double)(float)gk);
@@ -319,10 +269,10 @@ table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
     __syncthreads();
     const float4 ih = i < N ? xh[i] : z4, il = i < N ? xl[i] : z4;
     // two exact factors: one alone may pass the FP32 range
-    const int e = ea[(size_t)(kb / kKbPerWin) * n_pad + i];
+    const float ti = i < N ? tau[i] : 0.f;
+    const int e = ea[(size_t)(kb / kKbPerBlk) * n_pad + i];
     const int e1 = e / 2;
     const float a1 = pow2f(e1), a2 = pow2f(e - e1);
-    constexpr float kMagic = 1.5f * 1073741824.0f;  // rounds to multiples of 2^7
     {
         const int k8 = blockIdx.z;
         float vh[8][5], vl[8][5], rh[8], rl[8];
@@ -330,7 +280,10 @@ table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
         for (int q = 0; q < 8; ++q) {
             const int kk = k8 * 8 + q, k = k0 + kk;
             PairDf p;
-            const bool ok = i < N && k < N && k != i && pair_df(ih, il, kh[kk], kl[kk], p);
+            const bool ok =
+                i < N && k < N && k != i &&
+                !mbm_is_near(pair_d2_hilo(ih, il, kh[kk], kl[kk]), ti, kt[kk]) &&
+                pair_df(ih, il, kh[kk], kl[kk], p);
             df rho = {0.f, 0.f};
             if (ok) {
                 rho = p.rho;
@@ -352,7 +305,7 @@ table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
                 ch[m] = fc.ch[r][m];
                 cl[m] = fc.cl[r][m];
             }
-            __align__(16) __half h8[8], m8[8], l8[8];
+            __align__(16) __half h8[8], l8[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 float H, Lw;
@@ -361,18 +314,15 @@ table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
                 float x = __fmaf_rn(H, rh[q], -p);
                 x = __fmaf_rn(H, rl[q], x);
                 x = __fmaf_rn(Lw, rh[q], x);
-                const float hi = __fsub_rn(__fadd_rn(p, kMagic), kMagic);
-                const float rem = __fadd_rn(__fsub_rn(p, hi), x);
-                const __half mh = __float2half_rn(rem);
-                h8[q] = __float2half_rn(hi);
-                m8[q] = mh;
-                l8[q] = __float2half_rn(__fsub_rn(rem, __half2float(mh)));
+                const df v = df_fast(p, x);  // x holds the form's small part, up to 2^-9 p
+                h8[q] = __float2half_rn(v.h);
+                const float rem = __fadd_rn(__fsub_rn(v.h, __half2float(h8[q])), v.l);
+                l8[q] = __float2half_rn(__fmul_rn(rem, 2048.0f));
             }
             unsigned char* dst =
                 T + (((size_t)r * nb + rb) * nkb + kb) * (size_t)(kPieces * kPieceB) + off;
             *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h8);
-            *reinterpret_cast<uint4*>(dst + kPieceB) = *reinterpret_cast<const uint4*>(m8);
-            *reinterpret_cast<uint4*>(dst + 2 * kPieceB) = *reinterpret_cast<const uint4*>(l8);
+            *reinterpret_cast<uint4*>(dst + kPieceB) = *reinterpret_cast<const uint4*>(l8);
         }
     }
 }
@@ -457,13 +407,10 @@ __device__ __forceinline__ void drain(unsigned addr, const float* fj, float2 fi,
 
 // C[tile][r][column / 4][row][4] = sum over the slab's k of A_ik B_jk, in units
 // of the row scales. One CTA per SM, items (form, tile) dealt round robin,
-// forms outermost. Warps 0-15: accumulator windows to registers every 64
-// columns and to C every 512 (shorter FP32 chains); warp 16: bulk copies
-// (72 KB stages of 32 columns); warp 17: MMAs (8 products of pieces). The
-// accumulators fill TMEM: 256 columns for h h and 256 for the rest; each is
-// drained while the other is computed. (The rest in two halves of 128 columns
-// reads A twice and is bound by shared memory: forces of 8 192 particles took
-// 40.6 ms against 27.1; scale factors read from global memory in the drain: 37.1.)
+// forms outermost. Warps 0-15: read-outs to registers, C at the end; warp 16: bulk
+// copies (48 KB stages of 32 columns); warp 17: MMAs. The accumulators fill
+// TMEM: 256 columns for h h and 256 for h l + l h; each is drained while the
+// other is computed.
 __global__ void __launch_bounds__(kThreads, 1)
 contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __restrict__ TB,
                 const float* __restrict__ fA, const float* __restrict__ fB, int n_pad, int nb,
@@ -514,9 +461,9 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
                         bulk_copy_g2s(sm.a[s] + p * kPieceA, pa + kb * stage_src + p * kPieceB,
                                       kPieceA, &sm.full[s]);
                     bulk_copy_g2s(sm.b[s], pb + kb * stage_src, kPieces * kPieceB, &sm.full[s]);
-                    if (kb % kKbPerWin == 0) {
+                    if (kb % kKbPerBlk == 0) {
                         const int q = win++ % kFactorSlots;
-                        const size_t w = (size_t)(kb / kKbPerWin) * n_pad;
+                        const size_t w = (size_t)(kb / kKbPerBlk) * n_pad;
                         mbar_arrive_expect_tx(&sm.factors[q], (kBM + kBN) * sizeof(float));
                         bulk_copy_g2s(sm.fj[q], fB + w + J * kBN, kBN * sizeof(float),
                                       &sm.factors[q]);
@@ -534,17 +481,12 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
     } else if (warp == kEpiWarps + 1) {
         if (lane == 0) {
             constexpr unsigned idesc = tc_idesc_f16(kBM, kBN);
-            // products but h h, as (piece of A, piece of B), the largest last:
-            // what follows an addition truncates it
-            constexpr int kOther = 7;
-            constexpr int pa[kOther] = {2, 1, 0, 2, 0, 1, 1}, pb[kOther] = {1, 2, 2, 0, 1, 0, 1};
-            unsigned it = 0, win = 0;  // stages used, windows handed over
+            unsigned it = 0, win = 0, blk = 0;  // stages, windows and blocks handed over
             bool ok = true;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 for (int kb = 0; kb < nkb; kb += kKbPerWin, ++win) {
-                    // h h of the whole window, then the rest: the previous window's
-                    // second accumulator is drained under the former, the first
-                    // one under the latter
+                    const bool first = kb % kKbPerBlk == 0;
+                    const bool last = kb % kKbPerBlk == kKbPerBlk - kKbPerWin;
                     if (win && !wait_phase(sm, &sm.acc_empty[0], (win - 1) & 1)) {
                         ok = false;
                         break;
@@ -564,7 +506,7 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
                     }
                     if (!ok) break;
                     tc_commit(smem_u32(&sm.acc_full[0]));
-                    if (win && !wait_phase(sm, &sm.acc_empty[1], (win - 1) & 1)) {
+                    if (first && blk && !wait_phase(sm, &sm.acc_empty[1], (blk - 1) & 1)) {
                         ok = false;
                         break;
                     }
@@ -574,14 +516,17 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
                         const unsigned ab = smem_u32(sm.a[it % kStages]);
                         const unsigned bb = smem_u32(sm.b[it % kStages]);
 #pragma unroll
-                        for (int q = 0; q < kOther; ++q)
-#pragma unroll
-                            for (int k = 0; k < kBK / 16; ++k)
-                                tc_mma_f16(tmem + kBN,
-                                           tc_desc(ab + pa[q] * kPieceA + k * 256, 128, 512),
-                                           tc_desc(bb + pb[q] * kPieceB + k * 256, 128, 512), idesc,
-                                           u + q + k > 0);
-                        if (u == kKbPerWin - 1) tc_commit(smem_u32(&sm.acc_full[1]));
+                        for (int k = 0; k < kBK / 16; ++k) {
+                            tc_mma_f16(tmem + kBN, tc_desc(ab + k * 256, 128, 512),
+                                       tc_desc(bb + kPieceB + k * 256, 128, 512), idesc,
+                                       !(first && u + k == 0));
+                            tc_mma_f16(tmem + kBN, tc_desc(ab + kPieceA + k * 256, 128, 512),
+                                       tc_desc(bb + k * 256, 128, 512), idesc, true);
+                        }
+                        if (last && u == kKbPerWin - 1) {
+                            tc_commit(smem_u32(&sm.acc_full[1]));
+                            ++blk;
+                        }
                         tc_commit(smem_u32(&sm.empty[it % kStages]));
                     }
                 }
@@ -595,53 +540,39 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
         // rows 32 (warp % 4) + lane of the tile, columns 64 (warp / 4) + 0..63
         const int row = (warp & 3) * 32 + lane, col = (warp >> 2) * 64;
         const unsigned base = tmem + ((unsigned)(warp & 3) << 21) + col;
-        const int n_win = nkb / kKbPerWin;
-        unsigned win = 0;
+        unsigned win = 0, blk = 0;
         bool ok = true;
+        // waits for accumulator `a`, adds it and hands it back
+        auto take = [&](int a, unsigned phase, const float* fj, float fi, float2(&acc)[32]) {
+            if (!__all_sync(0xffffffffu, wait_phase(sm, &sm.acc_full[a], phase & 1))) return false;
+            tc_fence_after();
+            drain(base + a * kBN, fj, f2_splat(fi), acc);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.acc_empty[a]);
+            return true;
+        };
         for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-            int I, J;
-            decode_tile(t0 + item % nt, nb, I, J);
-            float4* out = reinterpret_cast<float4*>(C) +
-                          (size_t)((item % nt) * kForms + item / nt) * (kBM * kBN / 4) +
-                          (size_t)(col / 4) * kBM + row;
             float2 acc[32];
 #pragma unroll
             for (int c = 0; c < 32; ++c) acc[c] = make_float2(0.f, 0.f);
-            for (int w = 0; w < n_win; ++w, ++win) {
-                const unsigned slot = win % kFactorSlots;
-                if (!__all_sync(0xffffffffu,
-                                wait_phase(sm, &sm.factors[slot], (win / kFactorSlots) & 1))) {
-                    ok = false;
-                    break;
-                }
-                const float2 fi = f2_splat(sm.fi[slot][row]);
+            for (int b = 0; b < nkb / kKbPerBlk && ok; ++b, ++blk) {
+                const unsigned slot = blk % kFactorSlots;
+                ok = __all_sync(0xffffffffu,
+                                wait_phase(sm, &sm.factors[slot], (blk / kFactorSlots) & 1));
+                const float fi = sm.fi[slot][row];
                 const float* fj = &sm.fj[slot][col];
-#pragma unroll 1
-                for (int a = 0; a < 2; ++a) {
-                    if (!__all_sync(0xffffffffu, wait_phase(sm, &sm.acc_full[a], win & 1))) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    drain(base + a * kBN, fj, fi, acc);
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm.acc_empty[a]);
-                }
-                if (!ok) break;
-                if (w % kFlush == kFlush - 1 || w == n_win - 1) {
+                for (int w = 0; w < kWinPerBlk && ok; ++w, ++win) ok = take(0, win, fj, fi, acc);
+                if (ok) ok = take(1, blk, fj, fi * kLowScale, acc);
+            }
+            if (ok) {
+                float4* out = reinterpret_cast<float4*>(C) +
+                              (size_t)((item % nt) * kForms + item / nt) * (kBM * kBN / 4) +
+                              (size_t)(col / 4) * kBM + row;
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        float4 v = make_float4(acc[2 * c].x, acc[2 * c].y, acc[2 * c + 1].x,
+                for (int c = 0; c < 16; ++c)
+                    out[c * kBM] = make_float4(acc[2 * c].x, acc[2 * c].y, acc[2 * c + 1].x,
                                                acc[2 * c + 1].y);
-                        if (w >= kFlush) {
-                            const float4 u = out[c * kBM];
-                            v = make_float4(v.x + u.x, v.y + u.y, v.z + u.z, v.w + u.w);
-                        }
-                        out[c * kBM] = v;
-                        acc[2 * c] = acc[2 * c + 1] = make_float2(0.f, 0.f);
-                    }
-                }
             }
         }
     }
@@ -654,41 +585,26 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
 
 // ---------------------------------------------------------------------------
 // Pair pass: four CTAs per tile, a thread per row and 32 columns, four columns
-// at a time. Potentials: rho sum_r l_r(E) C^r, the forms as exact as in the table
-// (summing C^r A_r first costs two more roundings where the terms cancel).
-// Gradients: G = sum_r C^r A_r and (rho / r)(2 G e - 5 (e.G e) e). Column sums go
-// through a transposed shared buffer. Next to the result it sums, per particle,
-// the magnitudes of the pair terms and the bound of the slices' error.
+// at a time: G = sum_r C^r A_r (five components), then the pair's potential
+// rho e.G e or its gradient (rho / r)(2 G e - 5 (e.G e) e). Column sums go
+// through a transposed shared buffer. Near pairs have no entry in L.
 // ---------------------------------------------------------------------------
 enum : int { kPhi = 0, kForce = 1, kVjp = 2 };
-
-// Pieces are floating-point down to a floor of 2^-25 in units of |a L| <= 2^15;
-// a block's C is off by at most that times the other factor (2^15), twice, in
-// units of a_i a_j, and ten forms of |l| <= 1.86 rho add up to about four times one.
-constexpr float kSliceErr = 1.0f / 128.0f;
-// Of the summed magnitudes. The bound takes every entry of a window at the floor
-// against the largest of 16 columns, so it is far above the error: mixtures and
-// unit cubes reach 3e-5 with no loss, dimers 20 times closer than their
-// spacing 0.1 with none, 50 times 20 with the first loss (1e-6).
-constexpr double kGateTol = 1.0 / 64.0;
 
 constexpr int kStep = 16;      // columns between two column sums
 constexpr int kPairCols = 64;  // columns of a tile per CTA: 20 tiles alone left SMs idle
 
 template <int Mode>
 __global__ void __launch_bounds__(256)
-pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int n_pad, int nb,
-            int n_blk, int t0, const float* __restrict__ C, const float* __restrict__ Cg,
-            const double* __restrict__ g, const int* __restrict__ row_ea,
-            const int* __restrict__ row_eag, const int* __restrict__ ref,
-            const float* __restrict__ fb, const float* __restrict__ fb16,
-            const float* __restrict__ fbg, double sign, double* __restrict__ out,
-            double* __restrict__ mag, double* __restrict__ err) {
-    constexpr int kVals = Mode == kPhi ? 3 : 5;  // components, magnitude, error bound
+pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int nb, int t0,
+            const float* __restrict__ tau, const float* __restrict__ C,
+            const float* __restrict__ Cg, const double* __restrict__ g,
+            const int* __restrict__ row_ea, const int* __restrict__ row_eag,
+            const int* __restrict__ ref, double sign, double* __restrict__ out) {
+    constexpr int kVals = Mode == kPhi ? 1 : 3;
     __shared__ float4 jh[kBN], jl[kBN];
-    __shared__ float wj[kBN], gj[kBN];
-    __shared__ float coef[kForms][5];  // gradients: A_r
-    __shared__ FormCoef fc;            // potentials
+    __shared__ float wj[kBN], gj[kBN], tj[kBN];
+    __shared__ float coef[kForms][5];  // A_r
     __shared__ float red[8][kStep][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int I, J;
@@ -702,16 +618,15 @@ pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
         jh[threadIdx.x] = j < N ? xh[j] : z4;
         jl[threadIdx.x] = j < N ? xl[j] : z4;
         wj[threadIdx.x] = j < N ? pow2f(eref - row_ea[j]) : 0.f;
+        tj[threadIdx.x] = j < N ? tau[j] : 0.f;
         gj[threadIdx.x] = Mode == kVjp && j < N ? (float)g[j] : 0.f;
-        if (threadIdx.x < kForms * 5) {
-            const int r = threadIdx.x / 5, m = threadIdx.x % 5;
-            coef[r][m] = (float)kFormA[r][m];
-            form_split(r, m, fc.ch[r][m], fc.cl[r][m]);
-        }
+        if (threadIdx.x < kForms * 5)
+            coef[threadIdx.x / 5][threadIdx.x % 5] = (float)kFormA[threadIdx.x / 5][threadIdx.x % 5];
     }
     __syncthreads();
     const bool iv = i < N;
     const float4 ih = iv ? xh[i] : z4, il = iv ? xl[i] : z4;
+    const float ti = iv ? tau[i] : 0.f;
     const int ei = iv ? row_ea[i] : 0;
     const float wi = iv ? pow2f(eref - ei) : 0.f;
     const float gi = Mode == kVjp && iv ? (float)g[i] : 0.f;
@@ -733,41 +648,14 @@ pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
         float part[kVals], col[kVals][kStep];
 #pragma unroll
         for (int d = 0; d < kVals; ++d) part[d] = 0.f;
-        float slice = 0.f, slice_g = 0.f;  // bound of |delta C| in units of A_i A_j
-        if (iv) {
-            const float* mj = fb16 + (J * kBN + c0) / kStep;
-            for (int b = 0; b < n_blk; ++b) {
-                const float m = mj[(size_t)b * (n_pad / kStep)];
-                slice = fmaf(fb[(size_t)b * n_pad + i], m, slice);
-                if (Mode == kVjp) slice_g = fmaf(fbg[(size_t)b * n_pad + i], m, slice_g);
-            }
-            slice *= kSliceErr;
-            slice_g *= kSliceErr * cg_scale;
-        }
 #pragma unroll
         for (int cc = 0; cc < kStep; cc += 4) {
             const int c4 = (c0 + cc) >> 2;
-            float G[4][5];             // gradients: sum_r C^r A_r
-            float T[4];                // potentials: sum_r l_r C^r
-            float vh[4][5], vl[4][5], rho[4];
-            if (Mode == kPhi) {
+            float G[4][5];  // sum_r C^r A_r
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int c = c0 + cc + q, j = J * kBN + c;
-                    PairDf p;
-                    const bool ok = pair_df(ih, il, jh[c], jl[c], p) && iv && j < N && j > i;
-                    T[q] = 0.f;
-                    rho[q] = ok ? p.rho.h * rho_scale1 * rho_scale2 : 0.f;
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-                    for (int m = 0; m < 5; ++m)
-                        comp_split(ok ? p.v[m].h : 0.f, ok ? p.v[m].l : 0.f, vh[q][m], vl[q][m]);
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int m = 0; m < 5; ++m) G[q][m] = 0.f;
-            }
+                for (int m = 0; m < 5; ++m) G[q][m] = 0.f;
 #pragma unroll
             for (int r = 0; r < kForms; ++r) {
                 float4 v = __ldcs(Cp + (size_t)(r * (kBN / 4) + c4) * kBM);
@@ -780,55 +668,40 @@ pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
                     v.w = fmaf(v.w, gi + gj[c + 3], u.w * cg_scale);
                 }
                 const float x[4] = {v.x, v.y, v.z, v.w};
-                if (Mode == kPhi) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float H, Lw;
-                        form_value(fc.ch[r], fc.cl[r], vh[q], vl[q], H, Lw);
-                        T[q] = fmaf(__fadd_rn(H, Lw), x[q], T[q]);
-                    }
-                } else {
+                for (int m = 0; m < 5; ++m) {
+                    const float a = coef[r][m];
 #pragma unroll
-                    for (int m = 0; m < 5; ++m) {
-                        const float a = coef[r][m];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) G[q][m] = fmaf(a, x[q], G[q][m]);
-                    }
+                    for (int q = 0; q < 4; ++q) G[q][m] = fmaf(a, x[q], G[q][m]);
                 }
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int c = c0 + cc + q, j = J * kBN + c;
                 const bool on = iv && j < N && j > i;
-                float val[kVals];  // components, their magnitude, the error bound
-                float bound = slice;
-                if (Mode == kVjp) bound = fmaf(slice, fabsf(gi + gj[c]), slice_g);
+                float val[kVals];
+                const float dx = (jh[c].x - ih.x) + (jl[c].x - il.x);
+                const float dy = (jh[c].y - ih.y) + (jl[c].y - il.y);
+                const float dz = (jh[c].z - ih.z) + (jl[c].z - il.z);
+                const float s = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                float y = rsqrtf(s);
+                y = fmaf(0.5f * y, fmaf(-s * y, y, 1.0f), y);
+                const bool ok = on && s < INFINITY &&
+                                !mbm_is_near(pair_d2_hilo(ih, il, jh[c], jl[c]), ti, tj[c]);
+                const float ex = ok ? dx * y : 0.f, ey = ok ? dy * y : 0.f, ez = ok ? dz * y : 0.f;
+                const float rho = ok ? (y * y * y) * rho_scale1 * rho_scale2 : 0.f;
+                // G is symmetric and traceless: (xx, yy, xy, xz, yz)
+                const float gx = fmaf(G[q][3], ez, fmaf(G[q][2], ey, G[q][0] * ex));
+                const float gy = fmaf(G[q][4], ez, fmaf(G[q][1], ey, G[q][2] * ex));
+                const float gz = fmaf(-(G[q][0] + G[q][1]), ez, fmaf(G[q][4], ey, G[q][3] * ex));
+                const float ege = fmaf(ez, gz, fmaf(ey, gy, ex * gx));
                 if (Mode == kPhi) {
-                    val[0] = T[q] * rho[q];
-                    val[1] = fabsf(val[0]);
-                    val[2] = bound * rho[q];
+                    val[0] = rho * ege;
                 } else {
-                    const float dx = (jh[c].x - ih.x) + (jl[c].x - il.x);
-                    const float dy = (jh[c].y - ih.y) + (jl[c].y - il.y);
-                    const float dz = (jh[c].z - ih.z) + (jl[c].z - il.z);
-                    const float s = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                    float y = rsqrtf(s);
-                    y = fmaf(0.5f * y, fmaf(-s * y, y, 1.0f), y);
-                    const bool ok = on && s > 0.f && s < INFINITY;
-                    const float ex = ok ? dx * y : 0.f, ey = ok ? dy * y : 0.f,
-                                ez = ok ? dz * y : 0.f;
-                    const float k = ok ? (y * y * y) * rho_scale1 * rho_scale2 * y : 0.f;
-                    // G is symmetric and traceless: (xx, yy, xy, xz, yz)
-                    const float gx = fmaf(G[q][3], ez, fmaf(G[q][2], ey, G[q][0] * ex));
-                    const float gy = fmaf(G[q][4], ez, fmaf(G[q][1], ey, G[q][2] * ex));
-                    const float gz =
-                        fmaf(-(G[q][0] + G[q][1]), ez, fmaf(G[q][4], ey, G[q][3] * ex));
-                    const float u = -5.0f * fmaf(ez, gz, fmaf(ey, gy, ex * gx));
+                    const float k = ok ? rho * y : 0.f, u = -5.0f * ege;
                     val[0] = k * fmaf(u, ex, 2.0f * gx);
-                    val[1] = k * fmaf(u, ey, 2.0f * gy);
-                    val[2] = k * fmaf(u, ez, 2.0f * gz);
-                    val[kVals - 2] = fmaxf(fabsf(val[0]), fmaxf(fabsf(val[1]), fabsf(val[2])));
-                    val[kVals - 1] = bound * k;
+                    val[kVals / 2] = k * fmaf(u, ey, 2.0f * gy);
+                    val[kVals - 1] = k * fmaf(u, ez, 2.0f * gz);
                 }
 #pragma unroll
                 for (int d = 0; d < kVals; ++d) {
@@ -854,9 +727,7 @@ pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
             t += __shfl_xor_sync(0xffffffffu, t, 16);
             if (lane < kStep && j < N && t != 0.f) {
                 const double v = unit * (double)t;
-                if (d == kVals - 2) atomicAdd(&mag[j], v);
-                else if (d == kVals - 1) atomicAdd(&err[j], v);
-                else if (Mode == kPhi) atomicAdd(&out[j], 0.5 * v);
+                if (Mode == kPhi) atomicAdd(&out[j], 0.5 * v);
                 else atomicAdd(&out[3 * (size_t)j + d], sign * v);
             }
         }
@@ -867,20 +738,10 @@ pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
         for (int d = 0; d < kVals; ++d) {
             if (sum[d] == 0.0) continue;
             const double v = unit * sum[d];
-            if (d == kVals - 2) atomicAdd(&mag[i], v);
-            else if (d == kVals - 1) atomicAdd(&err[i], v);
-            else if (Mode == kPhi) atomicAdd(&out[i], 0.5 * v);
+            if (Mode == kPhi) atomicAdd(&out[i], 0.5 * v);
             else atomicAdd(&out[3 * (size_t)i + d], -sign * v);
         }
     }
-}
-
-// Gate: some particle's summed error bound passes the tolerance.
-__global__ void __launch_bounds__(kBlk)
-gate_kernel(const double* __restrict__ mag, const double* __restrict__ err, int N,
-            int* __restrict__ gate) {
-    const int i = blockIdx.x * kBlk + threadIdx.x;
-    if (i < N && err[i] > kGateTol * mag[i]) *gate = 1;
 }
 
 __global__ void zero_if_kernel(const int* __restrict__ gate, double* __restrict__ out, int64_t n) {
@@ -910,10 +771,10 @@ Plan make_plan(int64_t N, bool weighted, size_t cap) {
     const int copies = weighted ? 2 : 1;
     const size_t per_blk = (size_t)kForms * p.nb * kKbPerBlk * kPieces * kPieceB * copies;
     const size_t per_tile = (size_t)kForms * kBM * kBN * sizeof(float) * copies;
-    const size_t fixed = up256((size_t)p.n_pad * 32) + 16 * (size_t)p.n_pad +
-                         2 * 4 * (size_t)p.n_pad + 131072;
-    // per 256 columns of a slab: ea and f per window, fb (and the weighted ones), fb16
-    const size_t per_blk_f = (size_t)p.n_pad * (8 * kWinPerBlk + 4) * copies + (size_t)p.n_pad / 4;
+    const size_t fixed =
+        up256((size_t)p.n_pad * 32) + 8 * (size_t)p.n_pad + mbm_near_bytes(N) + 131072;
+    // per 256 columns of a slab: ea and f (and the weighted ones)
+    const size_t per_blk_f = (size_t)p.n_pad * 8 * copies;
     if (cap < fixed) return Plan{};
     const size_t room = cap - fixed;
     int n_blk = (int)std::min<size_t>(std::min(p.nb, 16),
@@ -975,18 +836,14 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     auto* counter = reinterpret_cast<unsigned long long*>(head + 16);
     auto* xh = reinterpret_cast<float4*>(take((size_t)N * 16));
     auto* xl = reinterpret_cast<float4*>(take((size_t)N * 16));
-    auto* mag = reinterpret_cast<double*>(take((size_t)n_pad * 8));
-    auto* err = reinterpret_cast<double*>(take((size_t)n_pad * 8));
+    char* near_mem = take(mbm_near_bytes(N));
     auto* row_ea = reinterpret_cast<int*>(take((size_t)n_pad * 4));
     auto* row_eag = reinterpret_cast<int*>(take((size_t)n_pad * 4));
-    const size_t per_w = (size_t)n_pad * 4 * kWinPerBlk * p.n_blk, per_b = (size_t)n_pad * 4 * p.n_blk;
-    auto* ea = reinterpret_cast<int*>(take(per_w));
-    auto* f = reinterpret_cast<float*>(take(per_w));
-    auto* fb = reinterpret_cast<float*>(take(per_b));
-    auto* fb16 = reinterpret_cast<float*>(take(per_b / 16));
-    int* eag = weighted ? reinterpret_cast<int*>(take(per_w)) : nullptr;
-    float* fg = weighted ? reinterpret_cast<float*>(take(per_w)) : nullptr;
-    float* fbg = weighted ? reinterpret_cast<float*>(take(per_b)) : nullptr;
+    const size_t per_b = (size_t)n_pad * 4 * p.n_blk;
+    auto* ea = reinterpret_cast<int*>(take(per_b));
+    auto* f = reinterpret_cast<float*>(take(per_b));
+    int* eag = weighted ? reinterpret_cast<int*>(take(per_b)) : nullptr;
+    float* fg = weighted ? reinterpret_cast<float*>(take(per_b)) : nullptr;
     auto* T = reinterpret_cast<unsigned char*>(take(p.table));
     auto* Tg = weighted ? reinterpret_cast<unsigned char*>(take(p.table)) : nullptr;
     auto* C = reinterpret_cast<float*>(take(p.cbuf));
@@ -996,7 +853,6 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
     MBM_CUDA_TRY(cudaMemsetAsync(head, 0, 256, s));
     MBM_CUDA_TRY(cudaMemsetAsync(ref, 0x7f, 4, s));
-    MBM_CUDA_TRY(cudaMemsetAsync(mag, 0, up256((size_t)n_pad * 8) * 2, s));
     MBM_CUDA_TRY(cudaMemsetAsync(row_ea, 0x7f, up256((size_t)n_pad * 4) * 2, s));
     MBM_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)N * n_out * sizeof(double), s));
     MBM_CUDA_TRY(launch_pack_hilo(X, N, xh, xl, ctx->d_flags, s));
@@ -1005,16 +861,18 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(ContractSmem)));
     mbm_time_begin(ctx, s);
+    MbmNear near;
+    MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
     // Row exponents come from all columns: with several slabs a first pass over
     // them finds the row exponents before any table is built.
     const int slabs = (p.nb + p.n_blk - 1) / p.n_blk;
     auto scales = [&](int b0, int nblk) {
-        const dim3 grid(p.nb, nblk * kWinPerBlk);
-        scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0 * kWinPerBlk, nullptr, n_pad, ea,
-                                           row_ea, ctx->d_flags);
+        const dim3 grid(p.nb, nblk);
+        scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, nullptr, n_pad, ea,
+                                           row_ea);
         if (weighted)
-            scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0 * kWinPerBlk, g, n_pad, eag,
-                                               row_eag, ctx->d_flags);
+            scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, g, n_pad, eag,
+                                               row_eag);
     };
     if (slabs > 1)
         for (int b0 = 0; b0 < p.nb; b0 += p.n_blk) scales(b0, std::min(p.n_blk, p.nb - b0));
@@ -1023,14 +881,12 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
         scales(b0, nblk);
         if (b0 == 0)
             ref_kernel<<<std::min(p.nb, 64), kBlk, 0, s>>>(row_ea, (int)N, ref);
-        factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(ea, row_ea, n_pad, (int)N, f, fb, fb16);
-        table_kernel<<<dim3(p.nb, nkb, kBK / 8), kBlk, 0, s>>>(xh, xl, (int)N, b0, nullptr, n_pad, p.nb, nkb,
+        factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(ea, row_ea, n_pad, (int)N, f);
+        table_kernel<<<dim3(p.nb, nkb, kBK / 8), kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, nullptr, n_pad, p.nb, nkb,
                                                       ea, T);
         if (weighted) {
-            // fb16 keeps the unweighted maxima: the weighted rows meet unweighted columns
-            factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(eag, row_eag, n_pad, (int)N, fg, fbg,
-                                                            nullptr);
-            table_kernel<<<dim3(p.nb, nkb, kBK / 8), kBlk, 0, s>>>(xh, xl, (int)N, b0, g, n_pad, p.nb, nkb,
+            factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(eag, row_eag, n_pad, (int)N, fg);
+            table_kernel<<<dim3(p.nb, nkb, kBK / 8), kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, g, n_pad, p.nb, nkb,
                                                           eag, Tg);
         }
         MBM_CUDA_TRY(cudaGetLastError());
@@ -1042,22 +898,20 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
             if (weighted)
                 contract_kernel<<<grid, kThreads, sizeof(ContractSmem), s>>>(
                     Tg, T, fg, f, n_pad, p.nb, nkb, t0, nt, Cg, ctx->d_flags);
-            if (what == MBM_CONTRACT_PHI)
-                pair_kernel<kPhi><<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, n_pad, p.nb, nblk, t0, C, Cg,
-                                                     g, row_ea, row_eag, ref, fb, fb16, fbg, sign, out,
-                                                     mag, err);
-            else if (what == MBM_CONTRACT_FORCES)
-                pair_kernel<kForce><<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, n_pad, p.nb, nblk, t0, C,
-                                                       Cg, g, row_ea, row_eag, ref, fb, fb16, fbg,
-                                                       sign, out, mag, err);
-            else
-                pair_kernel<kVjp><<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, n_pad, p.nb, nblk, t0, C, Cg,
-                                                     g, row_ea, row_eag, ref, fb, fb16, fbg, sign, out,
-                                                     mag, err);
+            auto pass = [&](auto kernel) {
+                kernel<<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, p.nb, t0, near.tau,
+                                                                 C, Cg, g, row_ea, row_eag, ref,
+                                                                 sign, out);
+            };
+            if (what == MBM_CONTRACT_PHI) pass(pair_kernel<kPhi>);
+            else if (what == MBM_CONTRACT_FORCES) pass(pair_kernel<kForce>);
+            else pass(pair_kernel<kVjp>);
             MBM_CUDA_TRY(cudaGetLastError());
         }
     }
-    gate_kernel<<<p.nb, kBlk, 0, s>>>(mag, err, (int)N, gate);
+    MBM_CUDA_TRY(launch_near_triples(xh, xl, nullptr, N, near, g,
+                                     what == MBM_CONTRACT_PHI ? MBM_NEAR_PHI : MBM_NEAR_GRAD, sign,
+                                     out, ctx->num_sms, s));
     const int64_t n_val = N * n_out;
     zero_if_kernel<<<(unsigned)((n_val + 255) / 256), 256, 0, s>>>(gate, out, n_val);
     MBM_CUDA_TRY(cudaGetLastError());

@@ -5,9 +5,9 @@
 
 enum : int { MBM_CONTRACT_PHI = 0, MBM_CONTRACT_FORCES = 1, MBM_CONTRACT_VJP = 2 };
 
-// Smallest N that goes to the contraction: its chain of small kernels costs 0.15
+// Smallest N that goes to the contraction: its chain of small kernels costs 0.2
 // ms. Potentials: the pair-table sweep of N = 1 000 takes 0.27 ms, of 2 500 1.72
-// (contraction 1.28). Gradients: the gather form of N = 64 takes 0.12 ms (0.19),
+// (contraction 1.0). Gradients: the gather form of N = 64 takes 0.12 ms (0.19),
 // of 100 0.30 (0.19); VJP 0.31 against 0.25.
 constexpr int64_t kContractMinPhi = 1280;
 constexpr int64_t kContractMinForces = 96;

@@ -1,7 +1,8 @@
 """The tensor-core contraction behind the FP32 exhaustive modes (csrc/contract.cu)
 against the FP64 oracle, at the edges of its tiles (128 rows, 256 columns),
 windows (64) and blocks (256), with scratch that forces slabs and batches, and
-on sets that its error bound must turn away.
+on sets whose closest pairs dwarf the rest or tie (the pairs that are summed
+term by term).
 
 Bars: the FP32 ones of the exhaustive tests, 3e-6 sum|phi| for potentials and
 3e-5 sum|grad phi| for gradients."""
@@ -65,8 +66,8 @@ def test_slabs_and_batches_agree_with_one_piece():
 
 @pytest.mark.parametrize("ratio", [10.0, 300.0])
 def test_isolated_dimers(ratio):
-    """Pairs `ratio` times closer than their spacing: far past the point where
-    the pieces' floor shows, the solve has to notice and use the sweep."""
+    """Pairs `ratio` times closer than their spacing: their terms must not set the
+    scale that the others are cut against."""
     n = 1400
     rng = np.random.default_rng(3)
     c = inputs.uniform_cube(n // 2, (n // 2) ** (1 / 3), 0.5, 5)
@@ -94,3 +95,15 @@ def test_invalid_points_are_reported():
         assert getattr(e.value, "status", None) == -1
     good = api.potential(_dev(X), mode="fp32").cpu().numpy()
     assert np.all(np.isfinite(good))
+
+
+def test_lattice_ties():
+    """Six nearest neighbours at one distance: all of them are near pairs."""
+    g = np.arange(11, dtype=np.float64)
+    X = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3) * 0.75
+    idx = inputs.sample_indices(len(X), 32, 2)
+    ref, ref_abs = oracle.phi(X, idx, with_abs=True)
+    got = api.potential(_dev(X), mode="fp32").cpu().numpy()[idx]
+    assert np.all(np.abs(got - ref) <= 3e-6 * ref_abs)
+    F, S = oracle.forces(X, with_norm=True)
+    assert np.all(np.abs(api.forces(_dev(X), mode="fp32").cpu().numpy() - F).max(axis=1) <= 3e-5 * S)
