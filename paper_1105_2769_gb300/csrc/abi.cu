@@ -225,6 +225,18 @@ static mbm_status run_exhaustive(mbm_ctx* ctx, const double* X, int64_t N, int m
         if (rs != MBM_EBUDGET && rs != MBM_ENOMEM) return rs;
         cudaGetLastError();  // clear a failed allocation; take the path without a table
     }
+    if (mode == MBM_EXH_FP64 && N >= kContract64MinPhi) {
+        bool done = false;
+        MbmGate64 g;
+        MBM_TRY(mbm_contract64(ctx, X, N, MBM_CONTRACT_PHI, 1.0, phi, s, &done, &g));
+        if (done) {
+            MBM_CUDA_TRY(launch_exh_fp64(g.x4, N, phi, g.counter, ctx->d_flags, ctx->num_sms, s,
+                                         g.gate));
+            mbm_time_end(ctx, s);
+            if (validate) return mbm_check_flags(ctx, s);
+            return MBM_OK;
+        }
+    }
     const size_t pack = mode == MBM_EXH_FP32 ? (size_t)N * 2 * sizeof(float4)
                                              : (size_t)N * sizeof(double4_32a);
     MBM_TRY(mbm_scratch_reserve(ctx, hdr + pack));

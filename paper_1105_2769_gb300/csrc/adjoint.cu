@@ -299,12 +299,13 @@ cudaError_t launch_adjoint(Pts pts, int64_t N, const double* g, double* grad, do
     const int NT = (int)((N + kTile - 1) / kTile);
     const long long n_pairs = (long long)NT * (NT + 1) / 2;
     const int groups = (NT + kWarps - 1) / kWarps;
-    // enough items for ~4 waves; at least 64 pairs per chunk to amortise the table
+    // enough items for ~4 waves, down to 4 pairs per chunk: 64 left N = 700 with 12
+    // CTAs
     const long long want_items = (long long)(num_sms > 0 ? num_sms : 1) * 4;
     long long n_chunks = (want_items + groups - 1) / groups;
     if (n_chunks < 1) n_chunks = 1;
     long long ppc = (n_pairs + n_chunks - 1) / n_chunks;
-    if (ppc < 64) ppc = 64;
+    if (ppc < 4) ppc = 4;
     n_chunks = (n_pairs + ppc - 1) / ppc;
     const size_t smem = sizeof(AdjSmem<Real>);
     auto kern = adjoint_kernel<Real, KSUB, Pts>;
@@ -332,6 +333,17 @@ mbm_status run_adjoint(mbm_ctx* ctx, const double* X, int64_t N, const double* g
         if (done) {
             MBM_CUDA_TRY((launch_adjoint<float, 16>(Pts32{gt.xh, gt.xl}, N, g, out, sign,
                                                     ctx->num_sms, s, gt.gate)));
+            mbm_time_end(ctx, s);
+            return MBM_OK;
+        }
+    }
+    if (mode == MBM_EXH_FP64 && !g && N >= kContract64MinForces) {
+        bool done = false;
+        MbmGate64 gt;
+        MBM_TRY(mbm_contract64(ctx, X, N, MBM_CONTRACT_FORCES, sign, out, s, &done, &gt));
+        if (done) {
+            MBM_CUDA_TRY((launch_adjoint<double, 8>(Pts64{gt.x4}, N, g, out, sign, ctx->num_sms, s,
+                                                    gt.gate)));
             mbm_time_end(ctx, s);
             return MBM_OK;
         }

@@ -47,13 +47,13 @@
 #include "contract.h"
 #include "device_math.cuh"
 #include "dfloat.cuh"
+#include "forms.cuh"
 #include "near.h"
 #include "tcgen05.cuh"
 #include "tile_fp32.cuh"
 
 namespace {
 
-constexpr int kForms = 10;
 constexpr int kPieces = 2;
 constexpr int kBlk = 256;      // rows per table block, and columns that share a scale
 constexpr int kBM = 128;       // tile rows
@@ -75,39 +75,10 @@ constexpr int kThreads = (kEpiWarps + 2) * 32;
 constexpr int kGroup = 8;  // J tiles walked together: their rows and 19 I tiles stay in L2
 constexpr long long kWaitLimit = 4000000000LL;
 
-// A_r of l_r(B) = A_r : B, symmetric traceless: xx, yy, xy, xz, yz.
-__constant__ double kFormA[kForms][5] = {
-    {0.81051314900914676226, -1.0137444298135470439, 0.69187178704706466114, 0.10879332789123717943,
-     -0.60113244553623436798},
-    {0.29033471318095339961, -0.0037013574801380397359, -0.72945247235092144289,
-     -0.48361735206812446962, -1.2002939641387707073},
-    {0.56687761555815049061, -0.73198503004752586383, 0.77502100982572152509,
-     -0.52554704820191995188, 1.1260055012436281024},
-    {0.32794829997931705277, -1.1326061797678746186, -0.75463606268664968689,
-     -0.21929916513785778691, 0.2800933877523261306},
-    {-0.97297445172993803997, 0.29341922256285760709, 0.90751192347309499305,
-     0.32759516889683504779, 0.19146086840943790974},
-    {-0.67316138985808209333, 0.46260916239411561729, -0.054408203924041754195, -1.1509903099773033,
-     0.17733809272697340492},
-    {-0.017877295745476926793, 0.72594943548244305062, 0.18789931162397575175,
-     1.0813915903289111131, -0.75562451530097259604},
-    {0.13857796836323824696, 0.19482576157814381221, -0.26028666636158319084,
-     0.78643885767995610097, 0.97182503734766801594},
-    {-1.3260688300585429969, 0.63825499910587256587, -0.89891222534809540828,
-     0.37904860109016530897, -0.13692011279071057931},
-    {0.9208917500732497988, 0.48297899581067608991, 0.22434594372376326752,
-     -0.36411353209625681955, 0.076469687931274560653}};
-// largest |l_r(E)| over unit vectors and forms (the largest |eigenvalue| of an A_r)
-constexpr float kFormMax = 1.8573f;
-
 // Coefficients of l_r on (Exx - Ezz, Eyy - Ezz, Exy, Exz, Eyz).
 struct FormCoef {
     float ch[kForms][5], cl[kForms][5];
 };
-__device__ __forceinline__ double form_coef(int r, int m) {
-    return m < 2 ? kFormA[r][m] : 2.0 * kFormA[r][m];
-}
-
 // Split of the coefficients for exact chains: ch a multiple of 2^-10, cl the rest.
 __device__ __forceinline__ void form_split(int r, int m, float& ch, float& cl) {
     const double c = form_coef(r, m);

@@ -29,3 +29,14 @@ struct MbmGate {
 // then zeroed). sign multiplies the gradient; g: VJP only.
 mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* g, int what,
                         double sign, double* out, cudaStream_t s, bool* done, MbmGate* gate);
+
+// The same in FP64 (contract64.cu), potentials and forces.
+struct MbmGate64 {
+    const int* gate = nullptr;
+    unsigned long long* counter = nullptr;  // zeroed
+    const double4_32a* x4 = nullptr;        // packed points
+};
+constexpr int64_t kContract64MinPhi = 320;
+constexpr int64_t kContract64MinForces = 96;
+mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, double sign,
+                          double* out, cudaStream_t s, bool* done, MbmGate64* gate);

@@ -317,7 +317,8 @@ struct Fp64Smem {
 __global__ void __launch_bounds__(kWarps64 * 32, 1)
 exh_fp64_kernel(const double4_32a* __restrict__ x4, int N, int NT, long long n_items,
                 unsigned long long* __restrict__ counter, double* __restrict__ phi,
-                int* __restrict__ flags) {
+                int* __restrict__ flags, const int* __restrict__ gate) {
+    if (gate && !*gate) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Fp64Smem& sm = *reinterpret_cast<Fp64Smem*>(smem_raw);
     const int lane = threadIdx.x & 31;
@@ -567,7 +568,7 @@ cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
 }
 
 cudaError_t launch_exh_fp64(const double4_32a* x4, int64_t N, double* phi, unsigned long long* counter,
-                            int* flags, int num_sms, cudaStream_t s) {
+                            int* flags, int num_sms, cudaStream_t s, const int* gate) {
     const int NT = (int)((N + kTile - 1) / kTile);
     const long long items = (long long)NT * (NT + 1) / 2;
     const int threads = kWarps64 * 32;
@@ -576,7 +577,7 @@ cudaError_t launch_exh_fp64(const double4_32a* x4, int64_t N, double* phi, unsig
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = grid_for((const void*)exh_fp64_kernel, threads, smem, num_sms, items);
-    exh_fp64_kernel<<<grid, threads, smem, s>>>(x4, (int)N, NT, items, counter, phi, flags);
+    exh_fp64_kernel<<<grid, threads, smem, s>>>(x4, (int)N, NT, items, counter, phi, flags, gate);
     return cudaGetLastError();
 }
 

@@ -95,7 +95,7 @@ cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
                                   unsigned long long* counter, int* flags, int num_sms,
                                   cudaStream_t s);
 cudaError_t launch_exh_fp64(const double4_32a* x4, int64_t N, double* phi, unsigned long long* counter,
-                            int* flags, int num_sms, cudaStream_t s);
+                            int* flags, int num_sms, cudaStream_t s, const int* gate = nullptr);
 // Exact FP32-bulk Phi of sampled particles idx[0..n_idx) (out zeroed by the caller).
 cudaError_t launch_sampled_fp32(const float4* xhi, const float4* xlo, int64_t N,
                                 const int64_t* idx, int64_t n_idx, double* out, int* flags,
