@@ -1664,8 +1664,10 @@ seed_scale_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, 
 // partner pairs (b, c) the canonical case allows, and credits -grad. The
 // partner pairs' terms (unit vector, r^-3) are built once per slot in the
 // warp's shared table; a's terms to 8 columns c are held in registers and
-// its term to row b is formed once per row, so the inner loop is the
-// gradient alone. Masked pairs have zero terms and contribute exactly 0.
+// its term to row b is formed once per row, so the inner loop is the gradient
+// alone: 29 packed operations per two columns, the e_ab and e_ac terms summed
+// per row and column before the vectors, FP64 sums per leaf and 8 columns (per
+// row they kept the FP64 pipe half busy). Masked pairs have zero terms and contribute exactly 0.
 constexpr int kForceWarps = 4;
 constexpr int kForceCols = 8;
 // Largest seed level of the force criterion's A^l: the seed pass costs the
@@ -1674,30 +1676,15 @@ constexpr int kForceCols = 8;
 // 11.3 s at 6 levels, 12.7 s at 7, 21.2 s at 8).
 constexpr int kForceSeedMax = 6;
 
-// The partner table holds half of the c columns at a time (8 KB per warp), so
-// that five 4-warp CTAs (96 registers a thread) fit an SM: 20 warps.
+// The partner table holds half of the c columns at a time (8 KB per warp); four
+// 4-warp CTAs fit an SM at 128 registers a thread (five at 96 spilled).
 constexpr int kForceHalf = kTile / 2;
 struct ForceWarpSmem {
-    float4 ph[3][kTile], pl[3][kTile];  // the three leaves (hi/lo)
-    float4 tab[kTile][kForceHalf];      // partner pair (b, c): (e_bc, rho_bc), c in this half
+    float4 ph[3][kTile], pl[3][kTile];             // the three leaves (hi/lo)
+    mbm_tile::TabPair tab[kTile][kForceHalf / 2];  // partner pairs (b, c): (e_bc, rho_bc)
 };
 
-__device__ __forceinline__ float3 grad_from_terms(const PairFY& ab, const PairFY& ac, float4 bc) {
-    const float p1 = ab.ex * ac.ex + ab.ey * ac.ey + ab.ez * ac.ez;
-    const float p2 = ab.ex * bc.x + ab.ey * bc.y + ab.ez * bc.z;
-    const float p3 = ac.ex * bc.x + ac.ey * bc.y + ac.ez * bc.z;
-    const float q = fmaf(5.0f, p1 * p2 * p3, -1.0f);
-    const float R3 = 3.0f * (ab.rho * ac.rho * bc.w);
-    const float su = R3 * ab.y, sv = R3 * ac.y;
-    const float p23 = p2 * p3, p13 = p1 * p3, p12 = p1 * p2;
-    float3 g;
-    g.x = -su * (q * ab.ex - p23 * ac.ex - p13 * bc.x) - sv * (q * ac.ex - p23 * ab.ex - p12 * bc.x);
-    g.y = -su * (q * ab.ey - p23 * ac.ey - p13 * bc.y) - sv * (q * ac.ey - p23 * ab.ey - p12 * bc.y);
-    g.z = -su * (q * ab.ez - p23 * ac.ez - p13 * bc.z) - sv * (q * ac.ez - p23 * ab.ez - p12 * bc.z);
-    return g;
-}
-
-__global__ void __launch_bounds__(kForceWarps * 32, 5)
+__global__ void __launch_bounds__(kForceWarps * 32, 4)
 base_forces_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int64_t N,
                    const int4* __restrict__ items, int64_t n_items, double* __restrict__ acc3) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1731,44 +1718,88 @@ base_forces_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
             for (int e = lane; e < kTile * kForceHalf; e += 32) {
                 const int bi = e / kForceHalf, cr = e % kForceHalf, ci = h0 + cr;
                 const bool v = bi < n[o1] && ci < n[o2] && (!same || bi < ci);
-                float4 ent = z4;
-                if (v) {
-                    const PairFY bc = pair_sample_y(sm.ph[o1][bi], sm.pl[o1][bi], sm.ph[o2][ci],
-                                                    sm.pl[o2][ci]);
-                    ent = make_float4(bc.ex, bc.ey, bc.ez, bc.rho);
-                }
-                sm.tab[bi][cr] = ent;
+                const PairFY bc = pair_sample_y_or_zero(sm.ph[o1][bi], sm.pl[o1][bi],
+                                                        sm.ph[o2][ci & 31], sm.pl[o2][ci & 31], v);
+                float* ent = reinterpret_cast<float*>(&sm.tab[bi][cr >> 1]) + (cr & 1);
+                ent[0] = bc.ex;
+                ent[2] = bc.ey;
+                ent[4] = bc.ez;
+                ent[6] = bc.rho;
             }
             __syncwarp();
             const int h1 = h0 + kForceHalf < n[o2] ? h0 + kForceHalf : n[o2];
             for (int cb = h0; cb < h1; cb += kForceCols) {
-                PairFY ac[kForceCols];
+                constexpr int kP = kForceCols / 2;
+                float2 vx[kP], vy[kP], vz[kP], rv[kP], iv[kP], a2[kP];
 #pragma unroll
-                for (int q = 0; q < kForceCols; ++q) {
-                    const int ci = cb + q;
-                    const bool v = act && ci < n[o2] && !(ex2 && ci == lane);
-                    ac[q] = pair_sample_y(ah, al, sm.ph[o2][ci & 31], sm.pl[o2][ci & 31]);
-                    if (!v) ac[q] = PairFY{0.f, 0.f, 0.f, 0.f, 0.f};
+                for (int q = 0; q < kP; ++q) {
+                    const int c0 = cb + 2 * q, c1 = c0 + 1;
+                    const PairFY p0 = pair_sample_y_or_zero(
+                        ah, al, sm.ph[o2][c0 & 31], sm.pl[o2][c0 & 31],
+                        act && c0 < n[o2] && !(ex2 && c0 == lane));
+                    const PairFY p1 = pair_sample_y_or_zero(
+                        ah, al, sm.ph[o2][c1 & 31], sm.pl[o2][c1 & 31],
+                        act && c1 < n[o2] && !(ex2 && c1 == lane));
+                    vx[q] = make_float2(p0.ex, p1.ex);
+                    vy[q] = make_float2(p0.ey, p1.ey);
+                    vz[q] = make_float2(p0.ez, p1.ez);
+                    rv[q] = make_float2(p0.rho, p1.rho);
+                    iv[q] = make_float2(p0.y, p1.y);
+                    a2[q] = make_float2(0.f, 0.f);
                 }
+                // -grad = sum c1 e_ab + sum c2 e_ac - sum c3 e_bc: the first summed per
+                // row, the second per column, before the vectors come in
+                float g1x = 0.f, g1y = 0.f, g1z = 0.f;
+                float2 g3x = make_float2(0.f, 0.f), g3y = g3x, g3z = g3x;
+#pragma unroll 1
                 for (int bi = 0; bi < n[o1]; ++bi) {
-                    PairFY ab = pair_sample_y(ah, al, sm.ph[o1][bi], sm.pl[o1][bi]);
-                    if (!act || (ex1 && bi == lane)) ab = PairFY{0.f, 0.f, 0.f, 0.f, 0.f};
-                    float rx = 0.f, ry = 0.f, rz = 0.f;
+                    const PairFY ab = pair_sample_y_or_zero(ah, al, sm.ph[o1][bi], sm.pl[o1][bi],
+                                                            act && !(ex1 && bi == lane));
+                    const float2 ux = f2_splat(ab.ex), uy = f2_splat(ab.ey), uz = f2_splat(ab.ez);
+                    const float2 r3 = f2_splat(3.0f * ab.rho), iu = f2_splat(ab.y);
+                    float2 a1 = make_float2(0.f, 0.f);
+                    const mbm_tile::TabPair* tr = sm.tab[bi] + ((cb - h0) >> 1);
 #pragma unroll
-                    for (int q = 0; q < kForceCols; ++q) {
-                        const float3 g = grad_from_terms(ab, ac[q], sm.tab[bi][cb - h0 + q]);
-                        rx += g.x;
-                        ry += g.y;
-                        rz += g.z;
+                    for (int q = 0; q < kP; ++q) {
+                        const float4 t0 = tr[q].xy, t1 = tr[q].zr;
+                        const float2 wx = make_float2(t0.x, t0.y), wy = make_float2(t0.z, t0.w);
+                        const float2 wz = make_float2(t1.x, t1.y), rw = make_float2(t1.z, t1.w);
+                        const float2 p1 = f2_fma(uz, vz[q], f2_fma(uy, vy[q], f2_mul(ux, vx[q])));
+                        const float2 p2 = f2_fma(uz, wz, f2_fma(uy, wy, f2_mul(ux, wx)));
+                        const float2 p3 = f2_fma(vz[q], wz, f2_fma(vy[q], wy, f2_mul(vx[q], wx)));
+                        const float2 p12 = f2_mul(p1, p2), p13 = f2_mul(p1, p3);
+                        const float2 p23 = f2_mul(p2, p3);
+                        const float2 qf = f2_fma(f2_splat(5.f), f2_mul(p12, p3), f2_splat(-1.f));
+                        const float2 R3 = f2_mul(f2_mul(r3, rv[q]), rw);
+                        const float2 su = f2_mul(R3, iu), sv = f2_mul(R3, iv[q]);
+                        const float2 np23 = f2_mul(p23, f2_splat(-1.f));
+                        a1 = f2_add(a1, f2_fma(su, qf, f2_mul(sv, np23)));
+                        a2[q] = f2_add(a2[q], f2_fma(sv, qf, f2_mul(su, np23)));
+                        const float2 c3 = f2_fma(su, p13, f2_mul(sv, p12));
+                        g3x = f2_fma(c3, wx, g3x);
+                        g3y = f2_fma(c3, wy, g3y);
+                        g3z = f2_fma(c3, wz, g3z);
                     }
-                    gx += (double)rx;
-                    gy += (double)ry;
-                    gz += (double)rz;
+                    const float c1 = a1.x + a1.y;
+                    g1x = fmaf(c1, ab.ex, g1x);
+                    g1y = fmaf(c1, ab.ey, g1y);
+                    g1z = fmaf(c1, ab.ez, g1z);
                 }
+                float2 g2x = make_float2(0.f, 0.f), g2y = g2x, g2z = g2x;
+#pragma unroll
+                for (int q = 0; q < kP; ++q) {
+                    g2x = f2_fma(a2[q], vx[q], g2x);
+                    g2y = f2_fma(a2[q], vy[q], g2y);
+                    g2z = f2_fma(a2[q], vz[q], g2z);
+                }
+                gx += (double)((g3x.x + g3x.y) - g1x - (g2x.x + g2x.y));
+                gy += (double)((g3y.x + g3y.y) - g1y - (g2y.x + g2y.y));
+                gz += (double)((g3z.x + g3z.y) - g1z - (g2z.x + g2z.y));
             }
         }
         if (act) {
             const int64_t a = b[s] + lane;
+            // the sums above are grad phi; the force is its negative
             atomicAdd(&acc3[3 * a], -gx);
             atomicAdd(&acc3[3 * a + 1], -gy);
             atomicAdd(&acc3[3 * a + 2], -gz);
