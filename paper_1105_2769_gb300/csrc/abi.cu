@@ -207,14 +207,16 @@ static mbm_status run_exhaustive(mbm_ctx* ctx, const double* X, int64_t N, int m
     }
     if (mode == MBM_EXH_FP32 && N <= kPairTableMaxN) {
         const size_t tb = pair_table_bytes(N);
-        const mbm_status rs = mbm_scratch_reserve(ctx, hdr + tb);
+        const mbm_status rs = mbm_scratch_reserve(ctx, hdr + tb + (size_t)N * 2 * sizeof(float4));
         if (rs == MBM_OK) {
             char* base = static_cast<char*>(ctx->scratch);
             auto* counter = reinterpret_cast<unsigned long long*>(base);
             MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
             MBM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s));
             MBM_CUDA_TRY(cudaMemsetAsync(phi, 0, (size_t)N * sizeof(double), s));
-            MBM_CUDA_TRY(launch_pair_table(X, N, base + hdr, ctx->d_flags, s));
+            auto* xh = reinterpret_cast<float4*>(base + hdr + tb);
+            MBM_CUDA_TRY(launch_pack_hilo(X, N, xh, xh + N, ctx->d_flags, s));
+            MBM_CUDA_TRY(launch_pair_table(X, xh, xh + N, N, base + hdr, ctx->d_flags, s));
             mbm_time_begin(ctx, s);
             MBM_CUDA_TRY(launch_exh_fp32_table(base + hdr, N, phi, counter, ctx->d_flags,
                                                ctx->num_sms, s));

@@ -25,6 +25,7 @@
 
 #include "bulk_copy.cuh"
 #include "device_math.cuh"
+#include "dfloat.cuh"
 #include "mbm_internal.h"
 #include "tile_fp32.cuh"
 
@@ -145,10 +146,12 @@ exh_fp32_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, in
 // ---------------------------------------------------------------------------
 // Step a3 with a pair table. Every pair term the FP32 sweep uses -- the unit
 // vector e_ab = (x_b - x_a)/r_ab and rho_ab = r_ab^-3 of each pair a < b -- is
-// computed once per solve in FP64 from the FP64 input and rounded once to
-// FP32, so each is correctly rounded (the in-kernel FP32 set-up carries a few
-// ulp), and the sweep no longer spends FP32 pipe time or MUFU work on pair
-// set-up. Layout: one 16 KB mbm_tile::PairBlock per tile pair (A, B),
+// computed once per solve to about 2^-40 and rounded once to FP32, so each is
+// as good as correctly rounded (the in-kernel FP32 set-up carries a few ulp),
+// and the sweep no longer spends FP32 pipe time or MUFU work on pair set-up.
+// The terms are formed in two-term FP32 numbers from the points' FP64 values
+// split in two: in FP64, with its square root and division at 1/64 of the FP32
+// rate, the table of N = 1 000 took 34 us. Layout: one 16 KB mbm_tile::PairBlock per tile pair (A, B),
 // A <= B, blocks of row A contiguous; a block holds the pair terms from
 // particle A*32 + r to B*32 + c in two planes indexed [c / 2][r]. Entries of
 // pairs that are absent (beyond N) or not ordered (A == B, r >= c) are zero.
@@ -157,8 +160,26 @@ __host__ __device__ __forceinline__ long long pt_block(int A, int B, int NT) {
     return (long long)A * NT - (long long)A * (A - 1) / 2 + (B - A);
 }
 
+// The terms in FP64: distances whose square leaves the FP32 range, and what has
+// to be reported.
+__device__ __noinline__ int pair_terms_f64(const double* __restrict__ X, int a, int b, float v[4]) {
+    const double dx = X[3 * (int64_t)b] - X[3 * (int64_t)a];
+    const double dy = X[3 * (int64_t)b + 1] - X[3 * (int64_t)a + 1];
+    const double dz = X[3 * (int64_t)b + 2] - X[3 * (int64_t)a + 2];
+    const double s2 = dx * dx + dy * dy + dz * dz;
+    if (!isfinite(s2)) return MBM_FLAG_NONFINITE;
+    if (!(s2 > 0.0)) return MBM_FLAG_COINCIDENT;
+    const double y = 1.0 / sqrt(s2);
+    v[0] = (float)(dx * y);
+    v[1] = (float)(dy * y);
+    v[2] = (float)(dz * y);
+    v[3] = (float)(y * y * y);
+    return 0;
+}
+
 __global__ void __launch_bounds__(256)
-pair_table_kernel(const double* __restrict__ X, int N, int NT,
+pair_table_kernel(const double* __restrict__ X, const float4* __restrict__ xh,
+                  const float4* __restrict__ xl, int N, int NT,
                   mbm_tile::PairBlock* __restrict__ pt, int* __restrict__ flags) {
     const int A = blockIdx.y;
     const long long per_row = (long long)(NT - A) * (kTile * kTile / 2);
@@ -175,20 +196,18 @@ pair_table_kernel(const double* __restrict__ X, int N, int NT,
             const int col = 2 * p + c, b = B * kTile + col;
             v[c][0] = v[c][1] = v[c][2] = v[c][3] = 0.f;
             if (a < N && b < N && (A < B || r < col)) {
-                const double dx = X[3 * (int64_t)b] - X[3 * (int64_t)a];
-                const double dy = X[3 * (int64_t)b + 1] - X[3 * (int64_t)a + 1];
-                const double dz = X[3 * (int64_t)b + 2] - X[3 * (int64_t)a + 2];
-                const double s2 = dx * dx + dy * dy + dz * dz;
-                if (!isfinite(s2)) {
-                    bad |= MBM_FLAG_NONFINITE;
-                } else if (!(s2 > 0.0)) {
-                    bad |= MBM_FLAG_COINCIDENT;
+                const float4 ph = xh[a], pl = xl[a], qh = xh[b], ql = xl[b];
+                const df d[3] = {df_diff(qh.x, ql.x, ph.x, pl.x), df_diff(qh.y, ql.y, ph.y, pl.y),
+                                 df_diff(qh.z, ql.z, ph.z, pl.z)};
+                const df s2 = df_dot(d, d);
+                if (s2.h > 1e-30f && s2.h < 1e30f) {
+                    const df y = df_rsqrt(s2);
+                    v[c][0] = df_mul(d[0], y).h;
+                    v[c][1] = df_mul(d[1], y).h;
+                    v[c][2] = df_mul(d[2], y).h;
+                    v[c][3] = df_mul(df_mul(y, y), y).h;
                 } else {
-                    const double y = 1.0 / sqrt(s2);
-                    v[c][0] = (float)(dx * y);
-                    v[c][1] = (float)(dy * y);
-                    v[c][2] = (float)(dz * y);
-                    v[c][3] = (float)(y * y * y);
+                    bad |= pair_terms_f64(X, a, b, v[c]);
                 }
             }
         }
@@ -209,13 +228,26 @@ struct PtSmem {
     long long item;
 };
 
+// Items are (tile pair, chunk of `per` I tiles), n_chunk chunks numbered for
+// every pair; those past J hold nothing and are skipped here.
+__device__ __forceinline__ long long next_item(unsigned long long* counter, long long n_items,
+                                               int NT, int n_chunk, int per) {
+    for (;;) {
+        const long long t = (long long)atomicAdd(counter, 1ULL);
+        if (t >= n_items) return t;
+        int J, K;
+        decode_pair_item(t / n_chunk, NT, J, K);
+        if ((int)(t % n_chunk) * per <= J) return t;
+    }
+}
+
 // An item's (j, k) table is block (J, K) of the pair table: one 16 KB bulk
 // copy, issued by thread 0 as soon as the previous item's warps are done
 // with the buffer.
-__device__ __forceinline__ void issue_item_table(PtSmem& sm, long long t, int NT,
+__device__ __forceinline__ void issue_item_table(PtSmem& sm, long long t, int NT, int n_chunk,
                                                  const mbm_tile::PairBlock* pt) {
     int J, K;
-    decode_pair_item(t, NT, J, K);
+    decode_pair_item(t / n_chunk, NT, J, K);
     const unsigned bytes = (unsigned)sizeof(mbm_tile::PairBlock);
     mbar_arrive_expect_tx(&sm.bar, bytes);
     bulk_copy_g2s(&sm.tab, pt + pt_block(J, K, NT), bytes, &sm.bar);
@@ -225,7 +257,7 @@ constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz: a copy that n
 
 __global__ void __launch_bounds__(kWarps32 * 32, 2)
 exh_fp32_pt_kernel(const mbm_tile::PairBlock* __restrict__ pt, int N, int NT, long long n_items,
-                   unsigned long long* __restrict__ counter, double* __restrict__ phi,
+                   int n_chunk, int per, unsigned long long* __restrict__ counter, double* __restrict__ phi,
                    int* __restrict__ flags) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     PtSmem& sm = *reinterpret_cast<PtSmem*>(smem_raw);
@@ -235,10 +267,10 @@ exh_fp32_pt_kernel(const mbm_tile::PairBlock* __restrict__ pt, int N, int NT, lo
     if (threadIdx.x == 0) {
         mbar_init(&sm.bar, 1);
         mbar_fence_init();
-        const long long t = (long long)atomicAdd(counter, 1ULL);
+        const long long t = next_item(counter, n_items, NT, n_chunk, per);
         sm.item = t;
         if (t < n_items) {
-            issue_item_table(sm, t, NT, pt);
+            issue_item_table(sm, t, NT, n_chunk, pt);
             pending = true;
         }
     }
@@ -257,12 +289,13 @@ exh_fp32_pt_kernel(const mbm_tile::PairBlock* __restrict__ pt, int N, int NT, lo
             break;
         }
         int J, K;
-        decode_pair_item(t, NT, J, K);
+        decode_pair_item(t / n_chunk, NT, J, K);
+        const int i_beg = (int)(t % n_chunk) * per, i_end = min(J, i_beg + per - 1);
         double run_j = 0.0, run_k = 0.0;
-        for (int I = warp; I <= J; I += kWarps32) {
+        for (int I = i_beg + warp; I <= i_end; I += kWarps32) {
             const int i = I * kTile + lane;
             // the warp's next (I, K) block is streamed from memory: ask L2 for it now
-            if (I + kWarps32 <= J) {
+            if (I + kWarps32 <= i_end) {
                 const char* nb = reinterpret_cast<const char*>(pt + pt_block(I + kWarps32, K, NT));
                 for (int o = lane * 128; o < (int)sizeof(mbm_tile::PairBlock); o += 32 * 128)
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(nb + o));
@@ -279,10 +312,10 @@ exh_fp32_pt_kernel(const mbm_tile::PairBlock* __restrict__ pt, int N, int NT, lo
         sm.wsum[1][warp][lane] = run_k;
         __syncthreads();  // every warp is done with the table buffer
         if (threadIdx.x == 0) {
-            const long long tn = (long long)atomicAdd(counter, 1ULL);
+            const long long tn = next_item(counter, n_items, NT, n_chunk, per);
             sm.item = tn;
             if (tn < n_items) {
-                issue_item_table(sm, tn, NT, pt);
+                issue_item_table(sm, tn, NT, n_chunk, pt);
                 pending = true;
             }
         }
@@ -542,11 +575,12 @@ size_t pair_table_bytes(int64_t N) {
     return (size_t)(NT * (NT + 1) / 2) * sizeof(mbm_tile::PairBlock);
 }
 
-cudaError_t launch_pair_table(const double* X, int64_t N, void* table, int* flags, cudaStream_t s) {
+cudaError_t launch_pair_table(const double* X, const float4* xh, const float4* xl, int64_t N,
+                              void* table, int* flags, cudaStream_t s) {
     const int NT = (int)((N + kTile - 1) / kTile);
     const long long per_row0 = (long long)NT * (kTile * kTile / 2);
     const int gx = (int)std::min<long long>((per_row0 + 255) / 256, 1024);
-    pair_table_kernel<<<dim3(gx, NT), 256, 0, s>>>(X, (int)N, NT,
+    pair_table_kernel<<<dim3(gx, NT), 256, 0, s>>>(X, xh, xl, (int)N, NT,
                                                    static_cast<mbm_tile::PairBlock*>(table), flags);
     return cudaGetLastError();
 }
@@ -555,7 +589,12 @@ cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
                                   unsigned long long* counter, int* flags, int num_sms,
                                   cudaStream_t s) {
     const int NT = (int)((N + kTile - 1) / kTile);
-    const long long items = (long long)NT * (NT + 1) / 2;
+    // One I tile per warp and item while whole items are too few to fill two CTAs
+    // per SM several times: N = 1 000 has 528 of them, of up to 32 I tiles.
+    const long long pairs = (long long)NT * (NT + 1) / 2;
+    const int per = pairs < 32LL * (num_sms > 0 ? num_sms : 1) ? kWarps32 : NT;
+    const int n_chunk = (NT + per - 1) / per;
+    const long long items = pairs * n_chunk;
     const int threads = kWarps32 * 32;
     const size_t smem = sizeof(PtSmem);
     cudaError_t e = cudaFuncSetAttribute((const void*)exh_fp32_pt_kernel,
@@ -563,7 +602,8 @@ cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
     if (e != cudaSuccess) return e;
     const int grid = grid_for((const void*)exh_fp32_pt_kernel, threads, smem, num_sms, items);
     exh_fp32_pt_kernel<<<grid, threads, smem, s>>>(
-        static_cast<const mbm_tile::PairBlock*>(table), (int)N, NT, items, counter, phi, flags);
+        static_cast<const mbm_tile::PairBlock*>(table), (int)N, NT, items, n_chunk, per, counter, phi,
+        flags);
     return cudaGetLastError();
 }
 

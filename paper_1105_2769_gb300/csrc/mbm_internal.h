@@ -88,9 +88,11 @@ cudaError_t launch_exh_fp32(const float4* xhi, const float4* xlo, int64_t N, dou
                             unsigned long long* counter, int* flags, int num_sms,
                             cudaStream_t s, const int* gate = nullptr);
 // Pair table of the FP32-bulk sum (unit vector and r^-3 of every pair, FP64
-// rounded once to FP32): its size, its build from X, and the sum that reads it.
+// rounded once to FP32): its size, its build from X and its packed form, and the
+// sum that reads it.
 size_t pair_table_bytes(int64_t N);
-cudaError_t launch_pair_table(const double* X, int64_t N, void* table, int* flags, cudaStream_t s);
+cudaError_t launch_pair_table(const double* X, const float4* xh, const float4* xl, int64_t N,
+                              void* table, int* flags, cudaStream_t s);
 cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
                                   unsigned long long* counter, int* flags, int num_sms,
                                   cudaStream_t s);
