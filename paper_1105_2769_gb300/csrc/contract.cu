@@ -18,9 +18,9 @@
 // solutions the one of least sum_r |l_r|^6 is taken, which keeps the cancellation
 // between the ten terms small.
 //
-// Precision. Each particle's four nearest neighbours are left out of the matrices
+// Precision. Each particle's three nearest neighbours are left out of the matrices
 // and the triples that hold such a pair are summed term by term (near.cu): they
-// carry 90-97 % of a potential and all of its large terms. The rest is smooth. A
+// carry 86-96 % of a potential and all of its large terms. The rest is smooth. A
 // row of L is cut against a power of two a per row and 256 columns, |a L| <= 2^15,
 // into h = fp16(a L) and l = fp16(2^11 (a L - h)): 22 bits. The tensor cores
 // multiply fp16 exactly and add in FP32 with truncation (8e-8 of a sum per 16
@@ -46,7 +46,6 @@
 #include "bulk_copy.cuh"
 #include "contract.h"
 #include "device_math.cuh"
-#include "dfloat.cuh"
 #include "forms.cuh"
 #include "near.h"
 #include "tcgen05.cuh"
@@ -74,64 +73,6 @@ constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 2) * 32;
 constexpr int kGroup = 8;  // J tiles walked together: their rows and 19 I tiles stay in L2
 constexpr long long kWaitLimit = 4000000000LL;
-
-// Coefficients of l_r on (Exx - Ezz, Eyy - Ezz, Exy, Exz, Eyz).
-struct FormCoef {
-    float ch[kForms][5], cl[kForms][5];
-};
-// Split of the coefficients for exact chains: ch a multiple of 2^-10, cl the rest.
-__device__ __forceinline__ void form_split(int r, int m, float& ch, float& cl) {
-    const double c = form_coef(r, m);
-    ch = rintf((float)(c * 1024.0)) / 1024.0f;
-    cl = (float)(c - (double)ch);
-}
-// The same for a component |v| <= 1: vh a multiple of 2^-11, so that the five
-// products ch vh are multiples of 2^-21 whose sum stays below 8: exact in FP32.
-__device__ __forceinline__ void comp_split(float h, float l, float& vh, float& vl) {
-    constexpr float kGrid = 1.5f * 4096.0f;
-    vh = __fsub_rn(__fadd_rn(h, kGrid), kGrid);
-    vl = __fadd_rn(__fsub_rn(h, vh), l);
-}
-__device__ __forceinline__ void form_value(const float (&ch)[5], const float (&cl)[5],
-                                           const float (&vh)[5], const float (&vl)[5], float& H,
-                                           float& Lw) {
-    H = 0.f;
-    Lw = 0.f;
-#pragma unroll
-    for (int m = 0; m < 5; ++m) {
-        H = __fmaf_rn(ch[m], vh[m], H);
-        Lw = __fmaf_rn(ch[m], vl[m], Lw);
-        Lw = __fmaf_rn(cl[m], __fadd_rn(vh[m], vl[m]), Lw);
-    }
-}
-
-// Pair terms to about 2^-40: v = (Exx - Ezz, Eyy - Ezz, Exy, Exz, Eyz) and
-// rho = r^-3. False if the pair is coincident or not finite (terms then zero).
-struct PairDf {
-    df v[5], rho;
-    float s, y;  // r^2 and 1/r to FP32
-};
-__device__ __forceinline__ bool pair_df(float4 ph, float4 pl, float4 qh, float4 ql, PairDf& o) {
-    const df dx = df_diff(qh.x, ql.x, ph.x, pl.x);
-    const df dy = df_diff(qh.y, ql.y, ph.y, pl.y);
-    const df dz = df_diff(qh.z, ql.z, ph.z, pl.z);
-    const df xx = df_mul(dx, dx), yy = df_mul(dy, dy), zz = df_mul(dz, dz);
-    const df s = df_add(df_add(xx, yy), zz);
-    o.s = s.h;
-    if (!(s.h > 0.f) || !(s.h < INFINITY)) return false;
-    const df y = df_rsqrt(s);
-    const df y2 = df_mul(y, y);
-    o.y = y.h;
-    o.rho = df_mul(y2, y);
-    const df ez = df_mul(zz, y2);
-    const df nez = {-ez.h, -ez.l};
-    o.v[0] = df_add(df_mul(xx, y2), nez);
-    o.v[1] = df_add(df_mul(yy, y2), nez);
-    o.v[2] = df_mul(df_mul(dx, dy), y2);
-    o.v[3] = df_mul(df_mul(dx, dz), y2);
-    o.v[4] = df_mul(df_mul(dy, dz), y2);
-    return true;
-}
 
 __device__ __forceinline__ float pow2f(int e) {  // 2^e, 0 below the normal range
     return e < -126 ? 0.f : __int_as_float((min(e, 127) + 127) << 23);
@@ -209,33 +150,29 @@ factor_kernel(const int* __restrict__ ea, const int* __restrict__ row_ea, int n_
 // Piece table, in the contraction's operand layout: T[r][row block][kb][piece]
 // is 256 rows x 32 columns as core matrices of 8 rows x 8 columns (128 bytes),
 // [row group][column group][row][column]. A CTA writes all forms and pieces of
-// 256 rows x 8 columns; a thread owns a row (16-byte stores, 128 contiguous bytes per 8 rows). FP32-pipe bound: ~140 operations
-// per pair and ~30 per form; the form is an exact FMA chain on the leading
-// bits plus a small one on the rest.
+// 256 rows x 8 columns; a thread owns a row (16-byte stores, 128 contiguous bytes
+// per 8 rows). FP32 pair terms: what they lose (2^-23) is weighed by the
+// contraction's small share of a result; two-term numbers took 2.4 times as long.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlk)
 table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int b0,
-             const float* __restrict__ tau, const double* __restrict__ g, int n_pad, int nb, int nkb, const int* __restrict__ ea,
-             unsigned char* __restrict__ T) {
-    __shared__ FormCoef fc;
-    __shared__ float4 kh[kBK], kl[kBK];
-    __shared__ float kg[kBK], kgl[kBK], kt[kBK];
-    const int rb = blockIdx.x, kb = blockIdx.y;
-    const int k0 = b0 * kBlk + kb * kBK;
+             const float* __restrict__ tau, const double* __restrict__ g, int n_pad, int nb,
+             int nkb, const int* __restrict__ ea, unsigned char* __restrict__ T) {
+    __shared__ float coef[kForms][5];
+    __shared__ float4 kh[8], kl[8];
+    __shared__ float kg[8], kt[8];
+    const int rb = blockIdx.x, kb = blockIdx.y, k8 = blockIdx.z;
+    const int k0 = b0 * kBlk + kb * kBK + k8 * 8;
     const int row = threadIdx.x, i = rb * kBlk + row;
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (threadIdx.x < kForms * 5) {
-        const int r = threadIdx.x / 5, m = threadIdx.x % 5;
-        form_split(r, m, fc.ch[r][m], fc.cl[r][m]);
-    }
-    if (threadIdx.x < kBK) {
+    if (threadIdx.x < kForms * 5)
+        coef[threadIdx.x / 5][threadIdx.x % 5] = (float)form_coef(threadIdx.x / 5, threadIdx.x % 5);
+    if (threadIdx.x < 8) {
         const int k = k0 + threadIdx.x;
         kh[threadIdx.x] = k < N ? xh[k] : z4;
         kl[threadIdx.x] = k < N ? xl[k] : z4;
         kt[threadIdx.x] = k < N ? tau[k] : 0.f;
-        const double gk = g && k < N ? g[k] : 1.0;
-        kg[threadIdx.x] = (float)gk;
-        kgl[threadIdx.x] = (float)(gk - (double)(float)gk);
+        kg[threadIdx.x] = g && k < N ? (float)g[k] : 1.f;
     }
     __syncthreads();
     const float4 ih = i < N ? xh[i] : z4, il = i < N ? xl[i] : z4;
@@ -244,57 +181,42 @@ table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
     const int e = ea[(size_t)(kb / kKbPerBlk) * n_pad + i];
     const int e1 = e / 2;
     const float a1 = pow2f(e1), a2 = pow2f(e - e1);
-    {
-        const int k8 = blockIdx.z;
-        float vh[8][5], vl[8][5], rh[8], rl[8];
+    float v[8][5];  // (Exx - Ezz, Eyy - Ezz, Exy, Exz, Eyz) a rho
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float dx = (kh[q].x - ih.x) + (kl[q].x - il.x);
+        const float dy = (kh[q].y - ih.y) + (kl[q].y - il.y);
+        const float dz = (kh[q].z - ih.z) + (kl[q].z - il.z);
+        const float s = pair_d2_hilo(ih, il, kh[q], kl[q]);
+        const bool ok = i < N && k0 + q < N && k0 + q != i && s < INFINITY &&
+                        !mbm_is_near(s, ti, kt[q]);
+        float y = rsqrtf(s);
+        y = fmaf(0.5f * y, fmaf(-s * y, y, 1.0f), y);
+        const float ex = dx * y, ey = dy * y, ez = dz * y;
+        const float rho = (y * y * y) * kg[q] * a1 * a2;
+        const float tx = ex * rho, ty = ey * rho, tz = ez * rho, zz = ez * tz;
+        v[q][0] = ok ? fmaf(ex, tx, -zz) : 0.f;
+        v[q][1] = ok ? fmaf(ey, ty, -zz) : 0.f;
+        v[q][2] = ok ? ex * ty : 0.f;
+        v[q][3] = ok ? ex * tz : 0.f;
+        v[q][4] = ok ? ey * tz : 0.f;
+    }
+    const size_t off = (size_t)(row >> 3) * 512 + k8 * 128 + (row & 7) * 16;
+#pragma unroll 1
+    for (int r = 0; r < kForms; ++r) {
+        __align__(16) __half h8[8], l8[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const int kk = k8 * 8 + q, k = k0 + kk;
-            PairDf p;
-            const bool ok =
-                i < N && k < N && k != i &&
-                !mbm_is_near(pair_d2_hilo(ih, il, kh[kk], kl[kk]), ti, kt[kk]) &&
-                pair_df(ih, il, kh[kk], kl[kk], p);
-            df rho = {0.f, 0.f};
-            if (ok) {
-                rho = p.rho;
-                if (g) rho = df_mul(rho, df{kg[kk], kgl[kk]});
-                rho = {rho.h * a1 * a2, rho.l * a1 * a2};
-            }
-            rh[q] = rho.h;
-            rl[q] = rho.l;
+            float x = coef[r][0] * v[q][0];
 #pragma unroll
-            for (int m = 0; m < 5; ++m)
-                comp_split(ok ? p.v[m].h : 0.f, ok ? p.v[m].l : 0.f, vh[q][m], vl[q][m]);
+            for (int m = 1; m < 5; ++m) x = fmaf(coef[r][m], v[q][m], x);
+            h8[q] = __float2half_rn(x);
+            l8[q] = __float2half_rn((x - __half2float(h8[q])) * 2048.0f);
         }
-        const size_t off = (size_t)(row >> 3) * 512 + k8 * 128 + (row & 7) * 16;
-#pragma unroll 1
-        for (int r = 0; r < kForms; ++r) {
-            float ch[5], cl[5];
-#pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                ch[m] = fc.ch[r][m];
-                cl[m] = fc.cl[r][m];
-            }
-            __align__(16) __half h8[8], l8[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                float H, Lw;
-                form_value(ch, cl, vh[q], vl[q], H, Lw);
-                const float p = __fmul_rn(H, rh[q]);
-                float x = __fmaf_rn(H, rh[q], -p);
-                x = __fmaf_rn(H, rl[q], x);
-                x = __fmaf_rn(Lw, rh[q], x);
-                const df v = df_fast(p, x);  // x holds the form's small part, up to 2^-9 p
-                h8[q] = __float2half_rn(v.h);
-                const float rem = __fadd_rn(__fsub_rn(v.h, __half2float(h8[q])), v.l);
-                l8[q] = __float2half_rn(__fmul_rn(rem, 2048.0f));
-            }
-            unsigned char* dst =
-                T + (((size_t)r * nb + rb) * nkb + kb) * (size_t)(kPieces * kPieceB) + off;
-            *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h8);
-            *reinterpret_cast<uint4*>(dst + kPieceB) = *reinterpret_cast<const uint4*>(l8);
-        }
+        unsigned char* dst =
+            T + (((size_t)r * nb + rb) * nkb + kb) * (size_t)(kPieces * kPieceB) + off;
+        *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h8);
+        *reinterpret_cast<uint4*>(dst + kPieceB) = *reinterpret_cast<const uint4*>(l8);
     }
 }
 

@@ -6,8 +6,8 @@
 enum : int { MBM_CONTRACT_PHI = 0, MBM_CONTRACT_FORCES = 1, MBM_CONTRACT_VJP = 2 };
 
 // Smallest N that goes to the contraction: its chain of small kernels costs 0.2
-// ms. Potentials: the pair-table sweep of N = 1 000 takes 0.27 ms, of 2 500 1.72
-// (contraction 1.0). Gradients: the gather form of N = 64 takes 0.12 ms (0.19),
+// ms. Potentials: the pair-table sweep of N = 1 000 takes 0.21 ms, of 2 500 1.72
+// (contraction 0.90). Gradients: the gather form of N = 64 takes 0.12 ms (0.19),
 // of 100 0.30 (0.19); VJP 0.31 against 0.25.
 constexpr int64_t kContractMinPhi = 1280;
 constexpr int64_t kContractMinForces = 96;
@@ -36,6 +36,8 @@ struct MbmGate64 {
     unsigned long long* counter = nullptr;  // zeroed
     const double4_32a* x4 = nullptr;        // packed points
 };
+// (FP64: the sweep of N = 300 takes 0.8 ms and the contraction 0.4; forces of
+// N = 100 took 3 ms in gather form and take 0.5.)
 constexpr int64_t kContract64MinPhi = 320;
 constexpr int64_t kContract64MinForces = 96;
 mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, double sign,

@@ -230,7 +230,9 @@ __device__ __forceinline__ void read_out(unsigned addr, unsigned long long (&t)[
 // (form, tile) dealt round robin. Warps 0-15: read-outs, a group of products of
 // one weight at a time, onto 32 sums per thread; warp 16: bulk copies (112 KB
 // stages); warp 17: MMAs, 28 products a stage. Four accumulators let the MMAs
-// run three groups ahead of the read-out.
+// run three groups ahead of the read-out, which bounds it: 10.5 ms at N = 3 001,
+// three times the products' time. (Two groups as one 32-bit integer per 64-bit
+// addition spilled at 96 registers: 11.4.)
 template <int Stages>  // stages per block
 __global__ void __launch_bounds__(kThreads, 1)
 contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, int nt,
@@ -379,10 +381,12 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
 }
 
 // ---------------------------------------------------------------------------
-// Pair pass in FP64: four CTAs per tile, a thread per row and 16 columns, two at a
-// time: C^r = sum over blocks of the scaled 64-bit sums, G = sum_r C^r A_r, then
+// Pair pass in FP64: 16 CTAs per tile, a thread per row and 4 columns, two at a
+// time (ten tiles at N = 512 need that many to fill the chip): C^r = sum over blocks of the scaled 64-bit sums, G = sum_r C^r A_r, then
 // rho e.G e or (rho / r)(2 G e - 5 (e.G e) e).
 // ---------------------------------------------------------------------------
+constexpr int kPairCols = 4;  // columns per thread
+
 template <bool Grad>
 __global__ void __launch_bounds__(256)
 pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
@@ -391,17 +395,17 @@ pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
               const longlong2* __restrict__ C, double sign, double* __restrict__ out) {
     constexpr int kVals = Grad ? 3 : 1;
     __shared__ double coef[kForms][5];
-    __shared__ double red[8][16][33];
+    __shared__ double red[8][kPairCols][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int I, J;
     decode_tile(t0 + blockIdx.x, I, J);
     const int row = (warp & 3) * 32 + lane;
-    const int c0 = blockIdx.y * 32 + (warp >> 2) * 16;
+    const int c0 = (blockIdx.y * 2 + (warp >> 2)) * kPairCols;
     const int i = I * kRows + row;
     if (threadIdx.x < kForms * 5)
         coef[threadIdx.x / 5][threadIdx.x % 5] = kFormA[threadIdx.x / 5][threadIdx.x % 5];
     __syncthreads();
-    if (J * kRows + c0 + 15 <= I * kRows + (warp & 3) * 32) return;  // no j > i (warp-uniform)
+    if (J * kRows + c0 + kPairCols - 1 <= I * kRows + (warp & 3) * 32) return;  // no j > i (warp-uniform)
     const bool iv = i < N;
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     const float4 ih = iv ? xh[i] : z4, il = iv ? xl[i] : z4;
@@ -410,9 +414,9 @@ pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
     double sum[kVals];
 #pragma unroll
     for (int d = 0; d < kVals; ++d) sum[d] = 0.0;
-    double col[kVals][16];
+    double col[kVals][kPairCols];
 #pragma unroll
-    for (int cc = 0; cc < 16; cc += 2) {
+    for (int cc = 0; cc < kPairCols; cc += 2) {
         const int j0 = J * kRows + c0 + cc;
         double G[2][5];
 #pragma unroll
@@ -478,18 +482,18 @@ pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
             }
         }
     }
-    const int j = J * kRows + c0 + (lane & 15);
+    const int j = J * kRows + c0 + (lane & 3);
 #pragma unroll
     for (int d = 0; d < kVals; ++d) {
         __syncwarp();
 #pragma unroll
-        for (int cc = 0; cc < 16; ++cc) red[warp][cc][lane] = col[d][cc];
+        for (int cc = 0; cc < kPairCols; ++cc) red[warp][cc][lane] = col[d][cc];
         __syncwarp();
-        double t = 0.0;  // 16 of the column's 32 rows
+        double t = 0.0;  // 4 of the column's 32 rows
 #pragma unroll
-        for (int q = 0; q < 16; ++q) t += red[warp][lane & 15][(lane >> 4) * 16 + q];
-        t += __shfl_xor_sync(0xffffffffu, t, 16);
-        if (lane < 16 && j < N && t != 0.0) {
+        for (int q = 0; q < 4; ++q) t += red[warp][lane & 3][(lane >> 2) * 4 + q];
+        for (int o = 16; o >= 4; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane < 4 && j < N && t != 0.0) {
             if constexpr (Grad) atomicAdd(&out[3 * (size_t)j + d], sign * t);
             else atomicAdd(&out[j], t);
         }
@@ -582,7 +586,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
         kernel<<<std::min(nt * kForms, std::max(1, ctx->num_sms)), kThreads, sizeof(ContractSmem),
                  s>>>(T, nb, nkb, t0, nt, C, ctx->d_flags);
         auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
-        pass<<<dim3(nt, kRows / 32), 256, 0, s>>>(x4, xh, xl, (int)N, n_pad, n_blk,
+        pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(x4, xh, xl, (int)N, n_pad, n_blk,
                                                   base_shift(stages), t0, near.tau, ea, C, sign,
                                                   out);
         MBM_CUDA_TRY(cudaGetLastError());

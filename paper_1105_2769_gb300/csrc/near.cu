@@ -2,10 +2,11 @@
 //
 // The contraction (contract.cu) multiplies matrices of pair terms r^-3 whose
 // largest entries are a few close pairs. Those carry most of every sum and set
-// the scale that the others are cut against. So each particle's four nearest
+// the scale that the others are cut against. So each particle's three nearest
 // neighbours are taken out of the matrices, and the triples with at least one
-// such pair (about 7.5 N of N^2 / 6 per particle) are summed directly here. What
-// is left to the contraction is 3-10 % of a potential and smooth.
+// such pair (about 2 N of N^2 / 6 per particle) are summed directly here. What
+// is left to the contraction is 4-14 % of a potential and smooth. (Two neighbours
+// double the contraction's error, four cost a third more triples here.)
 //
 // A triple with several near pairs is met once from each of them and counts
 // 1/2 or 1/3 each time.
@@ -21,7 +22,7 @@ namespace {
 
 constexpr int kRowWarps = 8;
 
-// One warp per particle: the four smallest r^2 of each lane, then of the warp.
+// One warp per particle: the smallest r^2 of each lane, then of the warp.
 __global__ void __launch_bounds__(kRowWarps * 32)
 knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
            float* __restrict__ tau, int* __restrict__ flags) {
@@ -39,7 +40,7 @@ knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
         bad |= !(s > 0.f);
         if (!(s > 0.f)) continue;
 #pragma unroll
-        for (int k = 0; k < kNearK; ++k) {  // insertion into the sorted four
+        for (int k = 0; k < kNearK; ++k) {  // insertion into the sorted list
             const float lo = fminf(s, t[k]);
             s = fmaxf(s, t[k]);
             t[k] = lo;
@@ -160,7 +161,7 @@ __device__ __forceinline__ float phi_df(const EdgeDf& u, const EdgeDf& a, const 
     return f.h;
 }
 
-constexpr int kChunk = 64;      // near pairs staged at a time
+constexpr int kChunk = 32;      // near pairs staged at a time
 constexpr int kNearWarps = 4;   // 128 particles j per CTA
 
 template <typename R>
@@ -387,8 +388,8 @@ cudaError_t launch_near_triples(const float4* xh, const float4* xl, const double
                                 int64_t N, const MbmNear& near, const double* g, int what,
                                 double sign, double* out, int num_sms, cudaStream_t s) {
     const unsigned bx = (unsigned)((N + kNearWarps * 32 - 1) / (kNearWarps * 32));
-    // about 3 N pairs; enough CTAs for eight per SM, at least one chunk each
-    const int64_t chunks = (3 * N + kChunk - 1) / kChunk;
+    // about 2 N pairs; enough CTAs for eight per SM, at least one chunk each
+    const int64_t chunks = (2 * N + kChunk - 1) / kChunk;
     int64_t by = (8 * (int64_t)(num_sms > 0 ? num_sms : 1) + bx - 1) / bx;
     if (by > chunks) by = chunks;
     const dim3 grid(bx, (unsigned)(by < 1 ? 1 : by));

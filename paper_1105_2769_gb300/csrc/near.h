@@ -3,9 +3,9 @@
 
 #include "mbm_internal.h"
 
-// tau[i]: r^2 (FP32, pair_d2_hilo) of particle i's fourth-nearest neighbour. A
+// tau[i]: r^2 (FP32, pair_d2_hilo) of particle i's third-nearest neighbour. A
 // pair is near if r^2 <= max(tau_i, tau_j): both members see the same answer.
-constexpr int kNearK = 4;
+constexpr int kNearK = 3;
 constexpr int kNearMax = 16;  // list capacity per particle; more sets the overflow word
 
 size_t mbm_near_bytes(int64_t N);
