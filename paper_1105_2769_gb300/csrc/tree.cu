@@ -65,6 +65,8 @@ struct mbm_tree {
     double* nphil = nullptr;  // per node
     double* pphil = nullptr;  // per sorted particle: |S(x)|
     int* weak = nullptr;      // per node: up to 32 sorted positions of smallest Phi^l(x)
+    float4* box32 = nullptr;  // per node: box lo, box hi, centre in FP32 (3 entries)
+    float* slack = nullptr;   // bound of what the FP32 rounding moves a difference by
 };
 
 namespace {
@@ -231,6 +233,26 @@ __global__ void node_finish_kernel(int64_t N, int64_t n_nodes, const double* nlo
     const double dz = __dsub_rn(nhi[3 * v + 2], nlo[3 * v + 2]);
     ndiam2[v] = cnt > 0 ? __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz))
                         : 0.0;
+}
+
+// FP32 boxes and centres, and a bound on the error of a difference of two of
+// their coordinates: each is rounded by 2^-24 of the largest coordinate, and so
+// is the difference; four times their sum.
+__global__ void box32_kernel(int64_t n_nodes, const double* __restrict__ nlo,
+                             const double* __restrict__ nhi, const double* __restrict__ ncen,
+                             float4* __restrict__ box, float* __restrict__ slack) {
+    const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (v >= n_nodes) return;
+    box[3 * v] = make_float4((float)nlo[3 * v], (float)nlo[3 * v + 1], (float)nlo[3 * v + 2], 0.f);
+    box[3 * v + 1] =
+        make_float4((float)nhi[3 * v], (float)nhi[3 * v + 1], (float)nhi[3 * v + 2], 0.f);
+    box[3 * v + 2] =
+        make_float4((float)ncen[3 * v], (float)ncen[3 * v + 1], (float)ncen[3 * v + 2], 0.f);
+    if (v == 0) {
+        double m = 0.0;
+        for (int k = 0; k < 3; ++k) m = fmax(m, fmax(fabs(nlo[k]), fabs(nhi[k])));
+        *slack = (float)(m * 7.2e-7);  // 12 x 2^-24
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -634,6 +656,8 @@ struct Trav {
     int64_t N, n_nodes, n_leaves;
     const double *nlo, *nhi, *ncen, *ndiam2, *nphil, *pphil;
     const int* weak;
+    const float4* box32;
+    const float* slack;
     const double* xs;
     const float4 *xh, *xl;
     double eps, tau, troot, zeta, z, alpha;
@@ -876,6 +900,61 @@ __device__ void triple_counts(const Trav& p, const int64_t P[3], double n[3], do
 
 enum : int { kActNone = 0, kActDet = 1, kActMC = 2, kActBase = 3, kActSplit = 4 };
 
+// Whether the p = 0 rule of the potential certainly fails, from FP32 boxes: true
+// only if the FP64 rule below would not prune either. Its interval contains phi
+// at every factor and cosine the boxes allow, so its width is at least
+// |n_c| (1/R3_lo - 1/R3_hi), n_c = 1 + 3 cos cos cos at the centres and R3 from
+// the nearest and farthest distances; its budget is at most that of the
+// smallest Phi^l. All roundings are taken against the claim (`slack` on every
+// coordinate difference, 1e-4 on the rest); what remains unclear goes to FP64.
+// Nearly every triple ends here: FP64 bounds on all of them were two thirds of
+// the traversal's kernels (N = 9 000: 41.7 million triples, 260 prunes).
+__device__ __forceinline__ bool surely_kept(const Trav& p, const int64_t P[3],
+                                            const bool first[3]) {
+    const float dl = *p.slack;
+    float smin_up = 1.f, smax_dn = 1.f;  // products over the three pairs
+    float4 c[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) c[s] = p.box32[3 * P[s] + 2];
+    float d[3][3], d2[3];  // centre differences of pairs 01, 02, 12
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int a = q == 2 ? 1 : 0, b = q == 0 ? 1 : 2;
+        const float4 la = p.box32[3 * P[a]], ha = p.box32[3 * P[a] + 1];
+        const float4 lb = p.box32[3 * P[b]], hb = p.box32[3 * P[b] + 1];
+        const float gx = fmaxf(lb.x - ha.x, la.x - hb.x), gy = fmaxf(lb.y - ha.y, la.y - hb.y),
+                    gz = fmaxf(lb.z - ha.z, la.z - hb.z);
+        if (fmaxf(gx, fmaxf(gy, gz)) + dl <= 0.f) return true;  // the boxes touch: no bound
+        const float ux = fmaxf(gx + dl, 0.f), uy = fmaxf(gy + dl, 0.f), uz = fmaxf(gz + dl, 0.f);
+        smin_up *= ux * ux + uy * uy + uz * uz;
+        const float fx = fmaxf(fmaxf(hb.x - la.x, ha.x - lb.x) - dl, 0.f);
+        const float fy = fmaxf(fmaxf(hb.y - la.y, ha.y - lb.y) - dl, 0.f);
+        const float fz = fmaxf(fmaxf(hb.z - la.z, ha.z - lb.z) - dl, 0.f);
+        smax_dn *= fx * fx + fy * fy + fz * fz;
+        d[q][0] = c[b].x - c[a].x;
+        d[q][1] = c[b].y - c[a].y;
+        d[q][2] = c[b].z - c[a].z;
+        d2[q] = d[q][0] * d[q][0] + d[q][1] * d[q][1] + d[q][2] * d[q][2];
+    }
+    const float r0 = rsqrtf(d2[0]), r1 = rsqrtf(d2[1]), r2 = rsqrtf(d2[2]);
+    const float p1 = (d[0][0] * d[1][0] + d[0][1] * d[1][1] + d[0][2] * d[1][2]) * r0 * r1;
+    const float p2 = (d[0][0] * d[2][0] + d[0][1] * d[2][1] + d[0][2] * d[2][2]) * r0 * r2;
+    const float p3 = (d[1][0] * d[2][0] + d[1][1] * d[2][1] + d[1][2] * d[2][2]) * r1 * r2;
+    // a centre difference is off by at most slack per coordinate: each cosine by at
+    // most 4 slack / r per edge
+    const float nc = fabsf(1.0f - 3.0f * (p1 * p2 * p3)) - 1e-3f -
+                     24.0f * 2.0f * dl * fmaxf(r0, fmaxf(r1, r2));
+    const float il = rsqrtf(smin_up), ih = rsqrtf(smax_dn);
+    const float width = nc * (il * il * il * 0.9999f - ih * ih * ih * 1.0001f);
+    double ph = INFINITY;
+#pragma unroll
+    for (int s = 0; s < 3; ++s)
+        if (first[s]) ph = fmin(ph, p.nphil[P[s]]);
+    const float budget = (float)((p.eps * fmax(ph, 0.0) + p.tau) * p.inv_troot) * 1.0001f;
+    // out of FP32's range (an overflowed or vanished power): FP64 decides
+    return nc > 0.f && width > budget && width > 1e-30f && width < 1e38f;
+}
+
 // F = false: the potential (p = 0 interval of phi, credit T_i phi(c1, c2, c3)).
 // F = true : the forces (bound M_s on |grad phi|_2 over the boxes, prune iff
 //            2 M_s <= (eps A^l(P_s) + tau) / T^root for every distinct slot;
@@ -893,10 +972,12 @@ __global__ void classify_kernel(const int4* __restrict__ front, int64_t n_front,
         double n[3], T[3];
         bool first[3];
         triple_counts(p, P, n, T, first);
-        double sl[3], sh[3];
-        box_d2(p, P[0], P[1], sl[0], sh[0]);
-        box_d2(p, P[0], P[2], sl[1], sh[1]);
-        box_d2(p, P[1], P[2], sl[2], sh[2]);
+        double sl[3] = {0.0, 0.0, 0.0}, sh[3];
+        if (F || !surely_kept(p, P, first)) {
+            box_d2(p, P[0], P[1], sl[0], sh[0]);
+            box_d2(p, P[0], P[2], sl[1], sh[1]);
+            box_d2(p, P[1], P[2], sl[2], sh[2]);
+        }
         // Touching boxes (d^l = 0, e.g. a repeated node) leave phi_hi = +inf:
         // the width is infinite and the rule cannot prune; skip its arithmetic.
         bool prune = false;
@@ -1892,7 +1973,7 @@ std::vector<size_t> tree_parts(int64_t N, int64_t n_nodes) {
     return {(size_t)N * 8, (size_t)N * 24, (size_t)N * 16, (size_t)N * 16,   // perm xs xh xl
             (size_t)n_nodes * 24, (size_t)n_nodes * 24, (size_t)n_nodes * 24,  // lo hi cen
             (size_t)n_nodes * 8, (size_t)n_nodes * 8, (size_t)N * 8,           // diam2 phil pphil
-            (size_t)n_nodes * 32 * 4};                                          // weak
+            (size_t)n_nodes * 32 * 4, (size_t)n_nodes * 48, 4};                 // weak box32 slack
 }
 
 // Buffer capacities of one traversal and its scratch layout.
@@ -1998,6 +2079,8 @@ static mbm_status build_tree(mbm_ctx* ctx, const double* X, int64_t N, const mbm
     t->nphil = cv.take<double>(n_nodes);
     t->pphil = cv.take<double>(N);
     t->weak = cv.take<int>((size_t)n_nodes * 32);
+    t->box32 = cv.take<float4>((size_t)n_nodes * 3);
+    t->slack = cv.take<float>(1);
 
     // Temporary scratch: box partials, keys/indices (double-buffered), sort temp, seed sums.
     const int nb = 256;
@@ -2054,6 +2137,8 @@ static mbm_status build_tree(mbm_ctx* ctx, const double* X, int64_t N, const mbm
     }
     node_finish_kernel<<<grid_of(n_nodes, 256), 256, 0, s>>>(N, n_nodes, t->nlo, t->nhi, t->ncen,
                                                              t->ndiam2);
+    box32_kernel<<<grid_of(n_nodes, 256), 256, 0, s>>>(n_nodes, t->nlo, t->nhi, t->ncen, t->box32,
+                                                       t->slack);
     TRY_LAUNCH();
 
     // Phi^l seed: exact sums over triples inside each seed node.
@@ -2281,6 +2366,8 @@ static mbm_status tree_solve(mbm_ctx* ctx, const double* X, int64_t N, double ep
     p.nphil = tree->nphil;
     p.pphil = tree->pphil;
     p.weak = tree->weak;
+    p.box32 = tree->box32;
+    p.slack = tree->slack;
     p.xs = tree->xs;
     p.xh = tree->xh;
     p.xl = tree->xl;
