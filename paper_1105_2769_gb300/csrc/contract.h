@@ -36,9 +36,9 @@ struct MbmGate64 {
     unsigned long long* counter = nullptr;  // zeroed
     const double4_32a* x4 = nullptr;        // packed points
 };
-// (FP64: the sweep of N = 300 takes 0.8 ms and the contraction 0.4; forces of
+// (FP64: the sweep of N = 300 takes 1.3 ms and the contraction 0.4; forces of
 // N = 100 took 3 ms in gather form and take 0.5.)
-constexpr int64_t kContract64MinPhi = 320;
+constexpr int64_t kContract64MinPhi = 192;
 constexpr int64_t kContract64MinForces = 96;
 mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, double sign,
                           double* out, cudaStream_t s, bool* done, MbmGate64* gate);

@@ -18,7 +18,7 @@ def _dev(X):
     return torch.from_numpy(np.ascontiguousarray(X)).cuda()
 
 
-@pytest.mark.parametrize("n", [320, 383, 384, 385, 512, 513, 769, 2048, 2049, 2561])
+@pytest.mark.parametrize("n", [192, 257, 320, 383, 384, 385, 512, 513, 769, 2048, 2049, 2561])
 def test_potential_at_tile_edges(n):
     X = inputs.uniform_cube(n, n ** (1 / 3), 0.3, 600 + n)
     idx = np.unique(np.concatenate([inputs.sample_indices(n, 40, n), [0, n - 1]]))
