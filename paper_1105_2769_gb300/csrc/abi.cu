@@ -184,10 +184,11 @@ void mbm_time_end(mbm_ctx* ctx, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // Exhaustive solves (steps a1 + a2/a3).
 // ---------------------------------------------------------------------------
-// Largest N whose FP32-bulk solve reads a pair table (NT(NT+1)/2 blocks of
-// 16 KB: 8.6 GB at N = 32 768, 34 GB at 65 536). Larger sets, or a table that
-// does not fit the context's budget or the device, form pair terms in the
-// kernel instead (FP32 set-up, a few ulp per pair term).
+// FP32 bulk from kContractMinPhi particles is a contraction (contract.cu). Below, or
+// if its scratch does not fit the context's budget or the device, the triple sweep
+// reads a pair table (NT(NT+1)/2 blocks of 16 KB: 13 MB at N = 1 279, 34 GB at
+// 65 536). Larger sets, or a table that does not fit either, form pair terms in
+// the kernel instead (FP32 set-up, a few ulp per pair term).
 constexpr int64_t kPairTableMaxN = 65536;
 
 static mbm_status run_exhaustive(mbm_ctx* ctx, const double* X, int64_t N, int mode, double* phi,

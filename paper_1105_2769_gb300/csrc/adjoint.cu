@@ -10,9 +10,9 @@
 // (From phi = L^-3/2 - 3 G L^-5/2 with L = |u|^2 |v|^2 |w|^2 and
 // G = (u.v)(u.w)(v.w), u = x_j - x_i, v = x_k - x_i, w = x_k - x_j.)
 //
-// FP32 gradients of kContractMinForces and more particles are a tensor-core contraction
-// (contract.cu), 20 times faster at N = 8 192; what follows serves FP64, small N
-// and scratch too small for it.
+// Forces of 96 and more particles, and FP32 VJPs, are tensor-core contractions
+// (contract.cu, 20 times faster at N = 8 192; contract64.cu, 160 times at N = 700).
+// What follows serves FP64 VJPs, smaller sets and scratch too small for those.
 //
 // Gather form: a lane owns particle i and sums grad_i over every pair j < k
 // of the set (pairs through i drop out: their distance is exactly zero), so

@@ -49,7 +49,6 @@
 #include "forms.cuh"
 #include "near.h"
 #include "tcgen05.cuh"
-#include "tile_fp32.cuh"
 
 namespace {
 
@@ -775,12 +774,13 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
         if (b0 == 0)
             ref_kernel<<<std::min(p.nb, 64), kBlk, 0, s>>>(row_ea, (int)N, ref);
         factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(ea, row_ea, n_pad, (int)N, f);
-        table_kernel<<<dim3(p.nb, nkb, kBK / 8), kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, nullptr, n_pad, p.nb, nkb,
-                                                      ea, T);
+        const dim3 tgrid(p.nb, nkb, kBK / 8);
+        table_kernel<<<tgrid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, nullptr, n_pad, p.nb,
+                                            nkb, ea, T);
         if (weighted) {
             factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(eag, row_eag, n_pad, (int)N, fg);
-            table_kernel<<<dim3(p.nb, nkb, kBK / 8), kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, g, n_pad, p.nb, nkb,
-                                                          eag, Tg);
+            table_kernel<<<tgrid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, g, n_pad, p.nb, nkb,
+                                                eag, Tg);
         }
         MBM_CUDA_TRY(cudaGetLastError());
         for (int t0 = 0; t0 < p.tiles; t0 += p.batch) {

@@ -6,6 +6,10 @@
 // three members, which is the same sum (each triple appears in exactly the
 // three slices Phi(x_a), Phi(x_b), Phi(x_c)).
 //
+// These sweeps serve small sets (below kContractMinPhi and kContract64MinPhi),
+// scratch too small for the contractions of contract.cu and contract64.cu, and
+// sets that those give back on the device (gate).
+//
 // FP32 bulk evaluates each triple in the direction-cosine form (see
 // tile_fp32.cuh: unit edge vectors and r^-3 per pair, 14 FP32 operations and
 // 23 FLOPs per triple). FP64 evaluates the law-of-cosines form on squared

@@ -250,46 +250,46 @@ near_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
                             part[0] = t;
                             row[0] = f;
                         } else {
-                        Edge<R> a, b;
-                        if constexpr (sizeof(R) == 8) {
-                            a = edge64(x64[n.i], kd);
-                            b = edge64(x64[n.j], kd);
-                        } else {
-                            a = edge32(ah[p], al[p], kh, kl);
-                            b = edge32(bh[p], bl[p], kh, kl);
-                        }
-                        const R ux = n.e.x, uy = n.e.y, uz = n.e.z;
-                        const R p1 = ux * a.x + uy * a.y + uz * a.z;
-                        const R p2 = ux * b.x + uy * b.y + uz * b.z;
-                        const R p3 = a.x * b.x + a.y * b.y + a.z * b.z;
-                        const R rr = n.e.rho * a.rho * b.rho;
-                        if constexpr (!Grad) {
-                            const R f = w * (rr - (R)3 * (p1 * p2 * p3) * rr);
-                            part[0] += f;
-                            row[0] = f;
-                        } else {
-                            w *= g ? n.w + gk : (R)1;
-                            const R qf = (R)5 * (p1 * p2 * p3) - (R)1;
-                            const R t3 = (R)3 * rr * w;
-                            const R su = t3 * n.e.inv, sa3 = t3 * a.inv, sb3 = t3 * b.inv;
-                            const R p23 = p2 * p3, p13 = p1 * p3, p12 = p1 * p2;
-                            // grad_a = -c1 u - c2 e_ak + c3 e_bk
-                            R c1 = su * qf - sa3 * p23, c2 = sa3 * qf - su * p23,
-                              c3 = su * p13 + sa3 * p12;
-                            row[0] = c3 * b.x - c1 * ux - c2 * a.x;
-                            row[1] = c3 * b.y - c1 * uy - c2 * a.y;
-                            row[2] = c3 * b.z - c1 * uz - c2 * a.z;
-                            // grad_b = c1' u - c2' e_bk + c3' e_ak
-                            c1 = su * qf + sb3 * p13;
-                            c2 = sb3 * qf + su * p13;
-                            c3 = sb3 * p12 - su * p23;
-                            row[kRow - 3] = c1 * ux - c2 * b.x + c3 * a.x;
-                            row[kRow - 2] = c1 * uy - c2 * b.y + c3 * a.y;
-                            row[kRow - 1] = c1 * uz - c2 * b.z + c3 * a.z;
-                            part[0] -= row[0] + row[kRow - 3];
-                            part[kCol / 2] -= row[1] + row[kRow - 2];
-                            part[kCol - 1] -= row[2] + row[kRow - 1];
-                        }
+                            Edge<R> a, b;
+                            if constexpr (sizeof(R) == 8) {
+                                a = edge64(x64[n.i], kd);
+                                b = edge64(x64[n.j], kd);
+                            } else {
+                                a = edge32(ah[p], al[p], kh, kl);
+                                b = edge32(bh[p], bl[p], kh, kl);
+                            }
+                            const R ux = n.e.x, uy = n.e.y, uz = n.e.z;
+                            const R p1 = ux * a.x + uy * a.y + uz * a.z;
+                            const R p2 = ux * b.x + uy * b.y + uz * b.z;
+                            const R p3 = a.x * b.x + a.y * b.y + a.z * b.z;
+                            const R rr = n.e.rho * a.rho * b.rho;
+                            if constexpr (!Grad) {
+                                const R f = w * (rr - (R)3 * (p1 * p2 * p3) * rr);
+                                part[0] += f;
+                                row[0] = f;
+                            } else {
+                                w *= g ? n.w + gk : (R)1;
+                                const R qf = (R)5 * (p1 * p2 * p3) - (R)1;
+                                const R t3 = (R)3 * rr * w;
+                                const R su = t3 * n.e.inv, sa3 = t3 * a.inv, sb3 = t3 * b.inv;
+                                const R p23 = p2 * p3, p13 = p1 * p3, p12 = p1 * p2;
+                                // grad_a = -c1 u - c2 e_ak + c3 e_bk
+                                R c1 = su * qf - sa3 * p23, c2 = sa3 * qf - su * p23,
+                                  c3 = su * p13 + sa3 * p12;
+                                row[0] = c3 * b.x - c1 * ux - c2 * a.x;
+                                row[1] = c3 * b.y - c1 * uy - c2 * a.y;
+                                row[2] = c3 * b.z - c1 * uz - c2 * a.z;
+                                // grad_b = c1' u - c2' e_bk + c3' e_ak
+                                c1 = su * qf + sb3 * p13;
+                                c2 = sb3 * qf + su * p13;
+                                c3 = sb3 * p12 - su * p23;
+                                row[kRow - 3] = c1 * ux - c2 * b.x + c3 * a.x;
+                                row[kRow - 2] = c1 * uy - c2 * b.y + c3 * a.y;
+                                row[kRow - 1] = c1 * uz - c2 * b.z + c3 * a.z;
+                                part[0] -= row[0] + row[kRow - 3];
+                                part[kCol / 2] -= row[1] + row[kRow - 2];
+                                part[kCol - 1] -= row[2] + row[kRow - 1];
+                            }
                         }
                     }
                 }
