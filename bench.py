@@ -39,16 +39,15 @@ sys.path.insert(0, ROOT)
 METRIC = "AT triples/s (exhaustive) & particles/s at eps=1e-2 vs plain FP64; p50/p99 ms"
 WORKLOAD = "exh32_n32768"
 N_MAIN = 32768
-FLOPS_PER_TRIPLE_FP32 = 23   # counted from the inner loop (FMA = 2), see csrc/tile_fp32.cuh
-# adjoint (gather form): 43 FLOPs per evaluation of grad_i phi (9 dot-product
-# operations = 15 FLOPs, products and coefficients 22, accumulations 6; FMA = 2,
-# csrc/adjoint.cu), three evaluations per unordered triple
-FLOPS_PER_TRIPLE_ADJOINT = 3 * 43
+# fp16 tensor-core FLOPs of the contraction (csrc/contract.cu) per unordered triple:
+# ten matrix products, three products of pieces each, one half (the matrices are
+# symmetric) of N^3 multiply-adds: 10 * 3 * N^3 FLOPs over N^3 / 6 triples. The
+# same for potentials and forces.
+FLOPS_PER_TRIPLE_CONTRACT = 180
 FP32_LANES_PER_SM = 128
-# dram__bytes_read.sum + dram__bytes_write.sum of one exh_fp32_pt_kernel launch on
-# the N = 32 768 set (ncu, one pass; the command is in
-# profiles/exh_fp32_n32768_launches.md). Valid for the kernel as committed with it.
-EXH_FP32_TRAFFIC_BYTES = 4088735832064 + 14698218240
+# Kernels of one FP32-bulk solve of N_MAIN particles (launch list in
+# profiles/contract_n32768_launches.md).
+LAUNCHES_PER_STEP = 220
 N_CONFIG3 = 1 << 20
 
 
@@ -259,12 +258,14 @@ def fp32_peak_tflops(torch, dev):
     return props.multi_processor_count * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
 
 
-def forces_roofline(rate, torch, dev):
-    peak = fp32_peak_tflops(torch, dev)
-    achieved = rate * FLOPS_PER_TRIPLE_ADJOINT / 1e12
-    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-            "frac": achieved / peak, "kernel": "adjoint_kernel<float>",
-            "flops_per_triple": FLOPS_PER_TRIPLE_ADJOINT, "traffic": None}
+def contract_roofline(rate):
+    peak = _peaks().get("bf16_tflops_sustained")
+    achieved = rate * FLOPS_PER_TRIPLE_CONTRACT / 1e12
+    return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak if peak else None, "kernel": "contract_kernel",
+            "flops_per_triple": FLOPS_PER_TRIPLE_CONTRACT, "traffic": None,
+            "peak_note": "measured cuBLAS bf16 GEMM, sustained; time is the whole solve's kernels "
+                         "(near triples, tables, contraction, pair pass)"}
 
 
 def bench_forces(api, inputs, torch, dev):
@@ -278,8 +279,8 @@ def bench_forces(api, inputs, torch, dev):
     torch.cuda.synchronize()
     dt = time.perf_counter() - t0
     return {"n": n, "triples_per_s": triples(n) / dt, "s": dt,
-            "roofline": forces_roofline(triples(n) / dt, torch, dev),
-            "note": "gather form: each unordered triple evaluated once per member"}
+            "roofline": contract_roofline(triples(n) / dt),
+            "note": "contraction: ten products of N x N matrices in fp16 pieces"}
 
 
 def bench_serving(api, inputs, np, duration=6.0, rate=200.0):
@@ -447,7 +448,7 @@ def run_forces_only(args):
     torch.cuda.synchronize()
     dt = time.perf_counter() - t0
     rep["exhaustive_fp32"] = {"s": dt, "triples_per_s": triples(n) / dt,
-                              "roofline": forces_roofline(triples(n) / dt, torch, dev)}
+                              "roofline": contract_roofline(triples(n) / dt)}
     print(json.dumps({"progress": rep}), flush=True)
     Fe = F.cpu().numpy()
     for eps in (1e-2,):
@@ -716,25 +717,12 @@ def main():
     n_trip = triples(len(X))
     value, tot_ms = aggregate(tot_ms, float(n_trip * args.steps), dist if world > 1 else None)
 
-    props = torch.cuda.get_device_properties(dev)
-    sm_max = float(_peaks().get("sm_max_mhz", 2070.0))
-    peak_tflops = props.multi_processor_count * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     k_ms = sum(kernel_ms) / len(kernel_ms)
-    achieved = FLOPS_PER_TRIPLE_FP32 * n_trip / (k_ms / 1e3) / 1e12
-    roofline = {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
-                "frac": achieved / peak_tflops,
-                "traffic": EXH_FP32_TRAFFIC_BYTES if len(X) == N_MAIN else None,
-                "traffic_note": ("ncu dram bytes per launch of the sweep (read 4.089e12, write "
-                                 "1.47e10): it streams the pair table's (i,k) blocks, 16 B per "
-                                 "pair term (0.7 B per triple), by design: the table replaces "
-                                 "FP32 pair set-up in the sweep; algorithmic input+output is "
-                                 "1.0 MB"),
-                "peak_note": (f"derived: {props.multi_processor_count} SMs x 128 FP32 lanes x 2 "
-                              f"x {sm_max:.0f} MHz (maximum SM clock)"),
-                "kernel": "exh_fp32_pt_kernel", "flops_per_triple": FLOPS_PER_TRIPLE_FP32,
-                "kernel_ms": k_ms}
-    if clocks.get("sm_mhz"):
-        roofline["frac_at_sampled_clock"] = achieved / (peak_tflops * clocks["sm_mhz"] / sm_max)
+    roofline = contract_roofline(n_trip / (k_ms / 1e3))
+    roofline["kernel_ms"] = k_ms
+    if clocks.get("sm_mhz") and roofline["frac"]:
+        sm_max = float(_peaks().get("sm_max_mhz", 2070.0))
+        roofline["frac_at_sampled_clock"] = roofline["frac"] * sm_max / clocks["sm_mhz"]
 
     # end to end through the host-buffer entry point (pinned host memory)
     Xh = torch.from_numpy(X).pin_memory().numpy()
@@ -755,11 +743,12 @@ def main():
         "data": "synthetic",
         "config": {"workload": WORKLOAD, "n": len(X), "triples_per_step": n_trip,
                    "distribution": "uniform [0,32]^3, d_min 0.5, seed 2",
-                   "precision": "FP32 triple arithmetic, FP64 accumulation",
+                   "precision": "FP32-bulk: terms to FP32 accuracy (two fp16 pieces, near "
+                                "triples in two-term FP32), FP64 accumulation",
                    "l2": "flushed between steps (256 MiB write)", "parallelism": f"replicas x{world}"},
         "roofline": roofline,
         "e2e": e2e,
-        "gpu_launches": 2 * args.steps,
+        "gpu_launches": LAUNCHES_PER_STEP * args.steps,
         "clocks": clocks,
     }
     if not args.no_extras and rank == 0:
