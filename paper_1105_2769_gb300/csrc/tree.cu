@@ -418,8 +418,11 @@ struct BaseSmem {
 // 32 at a time, so that lanes are full whatever the leaf size: with one x
 // leaf per sweep, leaves of 17.6 points (N = 9 000) used 18 of 32 lanes and,
 // with 32 rows and 32 columns, one triple slot in six. FP32-pipe bound.
+// A row's (i, j) terms are formed in every pass (about 40 operations against
+// 14 P packed ones), so up to 24 points take one pass, with fewer CTAs per SM
+// where the columns' registers need it (rule in base_group_for).
 template <int P>
-__global__ void __launch_bounds__(kBaseWarps * 32, 4)
+__global__ void __launch_bounds__(kBaseWarps * 32, P > 9 ? 3 : 4)
 base_group_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int64_t N,
                   int64_t first_leaf, int d, int n_chunk, const ull* __restrict__ key,
                   const int* __restrict__ val, const int* __restrict__ heads,
@@ -545,9 +548,13 @@ base_group_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, 
 using BaseGroupFn = void (*)(const float4*, const float4*, int64_t, int64_t, int, int, const ull*,
                              const int*, const int*, const int*, unsigned*, double*, int*);
 
-// Passes and column pairs per pass for leaves of at most n points.
+// Passes and column pairs per pass for leaves of at most n points. One pass
+// against two, base cases of mixtures in 512 leaves: 17 points 72.6 ->
+// 61.2 ms, 18 80.2 -> 67.2, 19 89.9 -> 82.7, 20 101.0 -> 92.4, 22 129.5 -> 115.3, 24
+// 129.1 -> 123.3. Three CTAs per SM from P = 10: at four, 19 points take 85.7 ms and
+// 22 144.5 (spills); at three, 18 points (P = 9) take 70.5.
 BaseGroupFn base_group_for(int n, int& n_chunk) {
-    n_chunk = n > 16 ? 2 : 1;
+    n_chunk = n > 24 ? 2 : 1;
     switch ((n + 2 * n_chunk - 1) / (2 * n_chunk)) {
         case 1: return base_group_kernel<1>;
         case 2: return base_group_kernel<2>;
@@ -556,7 +563,11 @@ BaseGroupFn base_group_for(int n, int& n_chunk) {
         case 5: return base_group_kernel<5>;
         case 6: return base_group_kernel<6>;
         case 7: return base_group_kernel<7>;
-        default: return base_group_kernel<8>;
+        case 8: return base_group_kernel<8>;
+        case 9: return base_group_kernel<9>;
+        case 10: return base_group_kernel<10>;
+        case 11: return base_group_kernel<11>;
+        default: return base_group_kernel<12>;
     }
 }
 
