@@ -62,10 +62,20 @@ knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
 }
 
 // Near pairs (i, j > i) of a particle: their number (pairs == NULL) or the pairs.
+// The numbers are 32-bit and many ties can pass that (points on a few sites: N^2 / 4
+// pairs), so what a particle holds beyond kNearMax is also added up in 64 bits
+// (`excess`, rarely touched). The list fits only if the excess is at most its
+// capacity, and then the 32-bit offsets cannot have wrapped: they are below
+// kNearMax N + cap.
+__device__ __forceinline__ bool list_overflows(const int* off, int N, int cap,
+                                               const unsigned long long* excess) {
+    return *excess > (unsigned long long)cap || off[N] > cap;
+}
+
 __global__ void __launch_bounds__(kRowWarps * 32)
 pairs_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
              const float* __restrict__ tau, int* __restrict__ cnt, const int* __restrict__ off,
-             int cap, int2* __restrict__ pairs) {
+             int cap, unsigned long long* __restrict__ excess, int2* __restrict__ pairs) {
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
     if (i > N) return;
@@ -73,7 +83,7 @@ pairs_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
         if (!pairs && lane == 0) cnt[N] = 0;
         return;
     }
-    if (pairs && off[N] > cap) return;
+    if (pairs && list_overflows(off, N, cap, excess)) return;
     const float4 ih = xh[i], il = xl[i];
     const float ti = tau[i];
     int at = pairs ? off[i] : 0;
@@ -88,12 +98,16 @@ pairs_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N
         if (pairs && near) pairs[at + __popc(m & ((1u << lane) - 1u))] = make_int2(i, j);
         at += __popc(m);
     }
-    if (!pairs && lane == 0) cnt[i] = at;
+    if (!pairs && lane == 0) {
+        cnt[i] = at;
+        if (at > kNearMax) atomicAdd(excess, (unsigned long long)(at - kNearMax));
+    }
 }
 
-__global__ void total_kernel(const int* __restrict__ off, int N, int cap, int* __restrict__ count,
-                             int* __restrict__ overflow) {
-    const bool over = off[N] > cap;
+__global__ void total_kernel(const int* __restrict__ off, int N, int cap,
+                             const unsigned long long* __restrict__ excess,
+                             int* __restrict__ count, int* __restrict__ overflow) {
+    const bool over = list_overflows(off, N, cap, excess);
     *count = over ? 0 : off[N];
     if (over) *overflow = 1;
 }
@@ -370,20 +384,23 @@ cudaError_t launch_near_list(const float4* xh, const float4* xl, int64_t N, void
     int* cnt = reinterpret_cast<int*>(take((size_t)(N + 1) * 4));
     int* off = reinterpret_cast<int*>(take((size_t)(N + 1) * 4));
     out->count = reinterpret_cast<int*>(take(256));
+    auto* excess = reinterpret_cast<unsigned long long*>(out->count + 16);
     out->pairs = reinterpret_cast<int2*>(take((size_t)N * kNearMax * sizeof(int2)));
     void* tmp = take(mbm_scan_temp_bytes_i32(N + 1));
     const int cap = (int)(N * kNearMax);
     const unsigned rows = (unsigned)((N + kRowWarps) / kRowWarps);
+    cudaError_t e = cudaMemsetAsync(excess, 0, sizeof(*excess), s);
+    if (e != cudaSuccess) return e;
     knn_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->tau, flags);
     pairs_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->tau, cnt, nullptr, cap,
-                                                 nullptr);
-    cudaError_t e = cudaGetLastError();
+                                                 excess, nullptr);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = mbm_exclusive_scan_i32(cnt, off, N + 1, tmp, s);
     if (e != cudaSuccess) return e;
     pairs_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->tau, cnt, off, cap,
-                                                 out->pairs);
-    total_kernel<<<1, 1, 0, s>>>(off, (int)N, cap, out->count, overflow);
+                                                 excess, out->pairs);
+    total_kernel<<<1, 1, 0, s>>>(off, (int)N, cap, excess, out->count, overflow);
     return cudaGetLastError();
 }
 
