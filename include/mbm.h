@@ -120,6 +120,11 @@ mbm_status mbm_ctx_destroy(mbm_ctx* ctx);
 /* Library-owned device bytes currently held by the context. */
 size_t mbm_ctx_bytes_in_use(const mbm_ctx* ctx);
 
+/* Clock cycles after which a wait inside the tensor-core kernels gives up
+ * (default 4e9, about 2 s; 0 = at once, which makes the wait run out on purpose).
+ * No wait of a healthy solve comes near the default. */
+mbm_status mbm_ctx_set_wait_cycles(mbm_ctx* ctx, int64_t cycles);
+
 /* Enable (1) or disable (0) CUDA-event timing of each solve's dominant
  * kernel (the exhaustive kernel, or the tree path's base-case kernels).
  * Events are recorded on the solve's stream. */

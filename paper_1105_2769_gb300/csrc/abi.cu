@@ -139,6 +139,14 @@ extern "C" mbm_status mbm_ctx_destroy(mbm_ctx* ctx) {
 
 extern "C" size_t mbm_ctx_bytes_in_use(const mbm_ctx* ctx) { return ctx ? ctx->in_use : 0; }
 
+extern "C" mbm_status mbm_ctx_set_wait_cycles(mbm_ctx* ctx, int64_t cycles) {
+    if (!ctx) return mbm_fail(MBM_EINVAL, "ctx is NULL");
+    if (cycles < 0) return mbm_fail(MBM_EINVAL, "cycles < 0");
+    std::lock_guard<std::mutex> lock(ctx->mu);
+    ctx->wait_cycles = cycles;
+    return MBM_OK;
+}
+
 extern "C" mbm_status mbm_ctx_set_timing(mbm_ctx* ctx, int enable) {
     if (!ctx) return mbm_fail(MBM_EINVAL, "ctx is NULL");
     MBM_CUDA_TRY(cudaSetDevice(ctx->device));

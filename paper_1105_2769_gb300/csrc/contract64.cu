@@ -37,7 +37,7 @@ constexpr int kStages = 2;
 constexpr int kBufs = 4;     // TMEM accumulators of 128 columns
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 2) * 32;
-constexpr long long kWaitLimit = 4000000000LL;
+constexpr long long kDrainLimit = 4000000000LL;  // for work in flight after an expired wait
 
 // Block of S stages: its 64-bit sums hold the weight-0 products, below 2^19 a
 // stage, at 2^base: 2^62 at most.
@@ -171,6 +171,8 @@ struct ContractSmem {
     unsigned char b[kStages][kStageBytes];
     unsigned long long full[kStages], empty[kStages];
     unsigned long long acc_full[kBufs], acc_empty[kBufs];
+    unsigned long long done;  // the MMAs have ended
+    long long wait_limit;
     unsigned tmem;
     volatile int abort;
 };
@@ -178,12 +180,12 @@ struct ContractSmem {
 // Bounded wait; the first one to give up tells every role to stop.
 __device__ __forceinline__ bool wait_phase(ContractSmem& sm, unsigned long long* bar,
                                            unsigned parity) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_test_wait(bar, parity)) return true;
     const long long t0 = clock64();
     for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (sm.wait_limit > 0 && mbar_try_wait(bar, parity)) return true;
         if (sm.abort) return false;
-        if (clock64() - t0 > kWaitLimit) {
+        if (clock64() - t0 > sm.wait_limit) {
             sm.abort = 1;
             return false;
         }
@@ -236,7 +238,7 @@ __device__ __forceinline__ void read_out(unsigned addr, unsigned long long (&t)[
 template <int Stages>  // stages per block
 __global__ void __launch_bounds__(kThreads, 1)
 contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, int nt,
-                  longlong2* __restrict__ C, int* __restrict__ flags) {
+                  longlong2* __restrict__ C, int* __restrict__ flags, long long wait_limit) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ContractSmem& sm = *reinterpret_cast<ContractSmem*>(smem_raw);
     constexpr int kBase = base_shift(Stages);
@@ -250,6 +252,8 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
             mbar_init(&sm.acc_full[a], 1);
             mbar_init(&sm.acc_empty[a], kEpiWarps);
         }
+        mbar_init(&sm.done, 1);
+        sm.wait_limit = wait_limit;
         sm.abort = 0;
         mbar_fence_init();
     }
@@ -283,7 +287,7 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
             }
             // copies in flight land before shared memory is released
             for (unsigned q = it > kStages ? it - kStages : 0; q < it; ++q)
-                mbar_wait_bounded(&sm.full[q % kStages], (q / kStages) & 1, kWaitLimit);
+                mbar_wait_bounded(&sm.full[q % kStages], (q / kStages) & 1, kDrainLimit);
         }
     } else if (warp == kEpiWarps + 1) {
         if (lane == 0) {
@@ -321,10 +325,10 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
                     if (ok) tc_commit(smem_u32(&sm.empty[s]));
                 }
             }
-            // MMAs in flight end before TMEM and shared memory are released
-            if (grp > 0)
-                mbar_wait_bounded(&sm.acc_full[(grp - 1) % kBufs], ((grp - 1) / kBufs) & 1,
-                                  kWaitLimit);
+            // MMAs in flight end before TMEM and shared memory are released, also those
+            // that an expired wait left without a commit
+            tc_commit(smem_u32(&sm.done));
+            mbar_wait_bounded(&sm.done, 0, kDrainLimit);
         }
     } else {
         // rows 32 (warp % 4) + lane of the tile, columns 32 (warp / 4) + 0..31
@@ -584,7 +588,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     for (int t0 = 0; t0 < tiles; t0 += batch) {
         const int nt = std::min(batch, tiles - t0);
         kernel<<<std::min(nt * kForms, std::max(1, ctx->num_sms)), kThreads, sizeof(ContractSmem),
-                 s>>>(T, nb, nkb, t0, nt, C, ctx->d_flags);
+                 s>>>(T, nb, nkb, t0, nt, C, ctx->d_flags, ctx->wait_cycles);
         auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
         pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(x4, xh, xl, (int)N, n_pad, n_blk,
                                                   base_shift(stages), t0, near.tau, ea, C, sign,
