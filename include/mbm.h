@@ -122,7 +122,8 @@ size_t mbm_ctx_bytes_in_use(const mbm_ctx* ctx);
 
 /* Clock cycles after which a wait inside the tensor-core kernels gives up
  * (default 4e9, about 2 s; 0 = at once, which makes the wait run out on purpose).
- * No wait of a healthy solve comes near the default. */
+ * No wait of a healthy solve comes near the default. A solve whose wait ran out is
+ * done again on the device by the triple sweep: its result is right, and late. */
 mbm_status mbm_ctx_set_wait_cycles(mbm_ctx* ctx, int64_t cycles);
 
 /* Enable (1) or disable (0) CUDA-event timing of each solve's dominant

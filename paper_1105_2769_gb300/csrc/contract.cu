@@ -32,8 +32,8 @@
 // (3.8e-7). Without the split, three pieces and eight products were needed for the
 // sweep's accuracy: forces of 8 192 particles took 29 ms against 16.
 // A set with more than 16 near pairs per particle (many equal distances) is left
-// to the FP32 sweep behind, decided on the device (gate); that sweep returns at
-// once otherwise.
+// to the FP32 sweep behind, decided on the device (gate), and so is one where a
+// bounded wait ran out; that sweep returns at once otherwise.
 //
 // Kernels: near pairs (near.cu); block maxima -> scales; piece table (stored in
 // the operand layout, so a stage is two kinds of bulk copies and no tensor map);
@@ -308,7 +308,7 @@ __device__ __forceinline__ void drain(unsigned addr, const float* fj, float2 fi,
 __global__ void __launch_bounds__(kThreads, 1)
 contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __restrict__ TB,
                 const float* __restrict__ fA, const float* __restrict__ fB, int n_pad, int nb,
-                int nkb, int t0, int nt, float* __restrict__ C, int* __restrict__ flags,
+                int nkb, int t0, int nt, float* __restrict__ C, int* __restrict__ gate,
                 long long wait_limit) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ContractSmem& sm = *reinterpret_cast<ContractSmem*>(smem_raw);
@@ -476,7 +476,7 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (threadIdx.x == 0 && sm.abort) atomicOr(flags, MBM_FLAG_TIMEOUT);
+    if (threadIdx.x == 0 && sm.abort) *gate = 1;  // C is not whole
     if (warp == 0) tc_free(tmem, 512);
 }
 
@@ -792,10 +792,10 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
             const int nt = std::min(p.batch, p.tiles - t0);
             const int grid = std::min(nt * kForms, std::max(1, ctx->num_sms));
             contract_kernel<<<grid, kThreads, sizeof(ContractSmem), s>>>(
-                T, T, f, f, n_pad, p.nb, nkb, t0, nt, C, ctx->d_flags, ctx->wait_cycles);
+                T, T, f, f, n_pad, p.nb, nkb, t0, nt, C, gate, ctx->wait_cycles);
             if (weighted)
                 contract_kernel<<<grid, kThreads, sizeof(ContractSmem), s>>>(
-                    Tg, T, fg, f, n_pad, p.nb, nkb, t0, nt, Cg, ctx->d_flags, ctx->wait_cycles);
+                    Tg, T, fg, f, n_pad, p.nb, nkb, t0, nt, Cg, gate, ctx->wait_cycles);
             auto pass = [&](auto kernel) {
                 kernel<<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, p.nb, t0, near.tau,
                                                                  C, Cg, g, row_ea, row_eag, ref,

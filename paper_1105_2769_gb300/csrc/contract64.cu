@@ -238,7 +238,7 @@ __device__ __forceinline__ void read_out(unsigned addr, unsigned long long (&t)[
 template <int Stages>  // stages per block
 __global__ void __launch_bounds__(kThreads, 1)
 contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, int nt,
-                  longlong2* __restrict__ C, int* __restrict__ flags, long long wait_limit) {
+                  longlong2* __restrict__ C, int* __restrict__ gate, long long wait_limit) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ContractSmem& sm = *reinterpret_cast<ContractSmem*>(smem_raw);
     constexpr int kBase = base_shift(Stages);
@@ -380,7 +380,7 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (threadIdx.x == 0 && sm.abort) atomicOr(flags, MBM_FLAG_TIMEOUT);
+    if (threadIdx.x == 0 && sm.abort) *gate = 1;  // C is not whole: the sweep solves the set
     if (warp == 0) tc_free(tmem, 512);
 }
 
@@ -588,7 +588,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     for (int t0 = 0; t0 < tiles; t0 += batch) {
         const int nt = std::min(batch, tiles - t0);
         kernel<<<std::min(nt * kForms, std::max(1, ctx->num_sms)), kThreads, sizeof(ContractSmem),
-                 s>>>(T, nb, nkb, t0, nt, C, ctx->d_flags, ctx->wait_cycles);
+                 s>>>(T, nb, nkb, t0, nt, C, gate, ctx->wait_cycles);
         auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
         pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(x4, xh, xl, (int)N, n_pad, n_blk,
                                                   base_shift(stages), t0, near.tau, ea, C, sign,

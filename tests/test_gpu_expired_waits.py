@@ -1,5 +1,6 @@
 """Waits of the tensor-core kernels that run out (a limit of 0 cycles makes them):
-the kernels end on their own, with nothing in flight, and the context stays usable."""
+the kernels end on their own, with nothing in flight, the context stays usable, and the
+solve is done again by the triple sweep."""
 import numpy as np
 import pytest
 import torch
@@ -38,4 +39,18 @@ def test_context_stays_usable(name):
         ctx.set_wait_cycles(4000000000)
         got = call(X, g, ctx).cpu().numpy()
         assert np.linalg.norm(got - want) <= 1e-12 * np.linalg.norm(want)
+    ctx.close()
+
+
+@pytest.mark.parametrize("name", sorted(CALLS))
+def test_result_is_right(name):
+    """Whatever the contraction left behind: the sweep's own accuracy."""
+    X, g, call = _case(name)
+    want = call(X, g, None).cpu().numpy()
+    ctx = api.Context(0)
+    for cycles in (0, 1, 20000):
+        ctx.set_wait_cycles(cycles)
+        got = call(X, g, ctx).cpu().numpy()
+        tol = 1e-12 if name.endswith("64") else 3e-6
+        assert np.linalg.norm(got - want) <= tol * np.linalg.norm(want)
     ctx.close()
