@@ -303,9 +303,15 @@ near_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
                                 row[kRow - 3] = c1 * ux - c2 * b.x + c3 * a.x;
                                 row[kRow - 2] = c1 * uy - c2 * b.y + c3 * a.y;
                                 row[kRow - 1] = c1 * uz - c2 * b.z + c3 * a.z;
-                                part[0] -= row[0] + row[kRow - 3];
-                                part[kCol / 2] -= row[1] + row[kRow - 2];
-                                part[kCol - 1] -= row[2] + row[kRow - 1];
+                                // grad_k by itself: as minus the sum of the other two it
+                                // would carry their rounding, which for a pair far
+                                // closer than k is 1 / r_ab against grad_k's 1 / r_ak
+                                c1 = sa3 * qf - sb3 * p12;
+                                c2 = sb3 * qf - sa3 * p12;
+                                c3 = sa3 * p23 + sb3 * p13;
+                                part[0] += c1 * a.x + c2 * b.x - c3 * ux;
+                                part[kCol / 2] += c1 * a.y + c2 * b.y - c3 * uy;
+                                part[kCol - 1] += c1 * a.z + c2 * b.z - c3 * uz;
                             }
                         }
                     }
