@@ -13,6 +13,13 @@
 // the pair pass. Error of the contraction: 4e-17 of a potential (norm, N = 300);
 // with the near triples the result is as close to 64 bits as the FP64 sweep's.
 //
+// Range. FP32 carries the near test and the exponents, so the points are brought to
+// a common unit first (frame.h): |x - x_0| < 2^10. With r >= 2^-20 there, every FP32
+// quantity is in range, and r^2 from the two FP32 parts of a point (2^-49 of it) is
+// within 2^-17: inside the exponents' margin. A set with a closer pair goes to the
+// FP64 sweep, decided on the device (gate); so does one with more than 16 near
+// pairs per particle.
+//
 // Kernels: near pairs; block maxima -> exponents; digit table (operand layout);
 // contraction (tcgen05.mma 128 x 128); pair pass in FP64; near triples in FP64.
 #include <algorithm>
@@ -23,6 +30,7 @@
 #include "contract.h"
 #include "device_math.cuh"
 #include "forms.cuh"
+#include "frame.h"
 #include "near.h"
 #include "tcgen05.cuh"
 
@@ -80,7 +88,7 @@ exponent_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, in
         const float y = rsqrtf(smin);
         e = 6 - ilogbf(y * y * y * (kFormMax * 1.0001f));
     }
-    if (i < n_pad) ea[(size_t)b * n_pad + i] = max(-140, min(140, e));
+    if (i < n_pad) ea[(size_t)b * n_pad + i] = e;
 }
 
 // ---------------------------------------------------------------------------
@@ -508,15 +516,12 @@ pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
     }
 }
 
-__global__ void zero_if_kernel(const int* __restrict__ gate, double* __restrict__ out, int64_t n) {
-    if (!*gate) return;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = 0.0;
-}
-
 size_t up256(size_t b) { return mbm_align_up(b, 256); }
 
 }  // namespace
+
+// r^2 of the closest pair that the two FP32 parts of a point resolve, in the frame.
+constexpr float kMinDist2 = 9.094947e-13f;  // 2^-40
 
 // Largest N: its digit table (140 N^2 bytes) has to fit the device.
 constexpr int64_t kMaxN64 = 24576;
@@ -558,6 +563,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     };
     int* gate = reinterpret_cast<int*>(take(256));
     auto* counter = reinterpret_cast<unsigned long long*>(gate + 16);
+    auto* frame = reinterpret_cast<MbmFrame*>(gate + 32);
     auto* x4 = reinterpret_cast<double4_32a*>(take((size_t)N * 32));
     auto* xh = reinterpret_cast<float4*>(take((size_t)N * 16));
     auto* xl = reinterpret_cast<float4*>(take((size_t)N * 16));
@@ -571,14 +577,15 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
     MBM_CUDA_TRY(cudaMemsetAsync(gate, 0, 256, s));
     MBM_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)n_val * sizeof(double), s));
-    MBM_CUDA_TRY(launch_pack_hilo(X, N, xh, xl, ctx->d_flags, s));
-    MBM_CUDA_TRY(launch_pack_f64(X, N, x4, ctx->d_flags, s));
+    MBM_CUDA_TRY(launch_frame(X, N, frame, xh, xl, x4, gate, ctx->d_flags, s));
     auto kernel = stages == 8 ? contract64_kernel<8> : contract64_kernel<16>;
     MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(ContractSmem)));
     mbm_time_begin(ctx, s);
     MbmNear near;
+    near.X = X;
+    near.min_d2 = kMinDist2;
     MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
     exponent_kernel<<<dim3(n_pad / 256, n_blk), 256, 0, s>>>(xh, xl, (int)N, cols, near.tau, n_pad,
                                                             ea);
@@ -598,8 +605,8 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     MBM_CUDA_TRY(launch_near_triples(xh, xl, x4, N, near, nullptr,
                                      grad ? MBM_NEAR_GRAD : MBM_NEAR_PHI, sign, out, ctx->num_sms,
                                      s));
-    zero_if_kernel<<<(unsigned)((n_val + 255) / 256), 256, 0, s>>>(gate, out, n_val);
-    MBM_CUDA_TRY(cudaGetLastError());
+    MBM_CUDA_TRY(launch_unframe(frame, grad ? 10 : 9, gate, out, n_val, s));
+    MBM_CUDA_TRY(launch_pack_f64(X, N, x4, ctx->d_flags, s, gate));  // the sweep's points
     gate_out->gate = gate;
     gate_out->counter = counter;
     gate_out->x4 = x4;

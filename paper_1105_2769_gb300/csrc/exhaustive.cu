@@ -56,7 +56,8 @@ __global__ void pack_hilo_kernel(const double* __restrict__ X, int64_t N, float4
 }
 
 __global__ void pack_f64_kernel(const double* __restrict__ X, int64_t N, double4_32a* __restrict__ x4,
-                                int* __restrict__ flags) {
+                                int* __restrict__ flags, const int* __restrict__ gate) {
+    if (gate && !*gate) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double x = X[3 * i], y = X[3 * i + 1], z = X[3 * i + 2];
@@ -550,11 +551,13 @@ cudaError_t launch_pack_hilo(const double* X, int64_t N, float4* xhi, float4* xl
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* flags, cudaStream_t s) {
+cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* flags, cudaStream_t s,
+                            const int* gate) {
     if (N <= 0) return cudaSuccess;
     const int threads = 256;
     const long long blocks = (N + threads - 1) / threads;
-    pack_f64_kernel<<<(unsigned)(blocks < 65535 ? blocks : 65535), threads, 0, s>>>(X, N, x4, flags);
+    pack_f64_kernel<<<(unsigned)(blocks < 65535 ? blocks : 65535), threads, 0, s>>>(X, N, x4, flags,
+                                                                                   gate);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,95 @@
+// Points in the unit that the contractions work in, and results back from it.
+// Two passes over the points, a few microseconds each: launches, not bytes.
+#include <algorithm>
+
+#include "frame.h"
+
+namespace {
+
+constexpr int kThreads = 256;
+
+// x_0, or the origin where it is not finite.
+__device__ __forceinline__ double origin(const double* X, int c) {
+    const double x = X[c];
+    return isfinite(x) ? x : 0.0;
+}
+
+__device__ __forceinline__ int frame_exponent(const MbmFrame* frame) {
+    const double m = __longlong_as_double((long long)frame->extent);
+    return m > 0.0 ? 9 - ilogb(m) : 0;
+}
+
+// Non-negative doubles order as their bits do.
+__global__ void __launch_bounds__(kThreads)
+extent_kernel(const double* __restrict__ X, int64_t N, MbmFrame* __restrict__ frame,
+              int* __restrict__ gate) {
+    const double o[3] = {origin(X, 0), origin(X, 1), origin(X, 2)};
+    double m = 0.0;
+    bool over = false;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
+         i += (int64_t)gridDim.x * blockDim.x)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double x = X[3 * i + c], d = fabs(x - o[c]);
+            if (isfinite(d)) m = fmax(m, d);
+            else over |= isfinite(x);
+        }
+    for (int s = 16; s > 0; s >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, s));
+    if ((threadIdx.x & 31) == 0 && m > 0.0)
+        atomicMax(&frame->extent, (unsigned long long)__double_as_longlong(m));
+    if (over) *gate = 1;
+}
+
+__global__ void __launch_bounds__(kThreads)
+frame_pack_kernel(const double* __restrict__ X, int64_t N, const MbmFrame* __restrict__ frame,
+                  float4* __restrict__ xh, float4* __restrict__ xl, double4_32a* __restrict__ x4,
+                  int* __restrict__ flags) {
+    const int e = frame_exponent(frame);
+    const double o[3] = {origin(X, 0), origin(X, 1), origin(X, 2)};
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        double y[3];
+        float h[3], l[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double x = X[3 * i + c];
+            if (!isfinite(x)) atomicOr(flags, MBM_FLAG_NONFINITE);
+            y[c] = scalbn(x, e);
+            const double d = scalbn(x - o[c], e);
+            h[c] = (float)d;
+            l[c] = (float)(d - (double)h[c]);
+        }
+        xh[i] = make_float4(h[0], h[1], h[2], 0.f);
+        xl[i] = make_float4(l[0], l[1], l[2], 0.f);
+        if (x4) x4[i] = make_double4_32a(y[0], y[1], y[2], 0.0);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads)
+unframe_kernel(const MbmFrame* __restrict__ frame, int degree, const int* __restrict__ gate,
+               double* __restrict__ out, int64_t n) {
+    const int e = degree * frame_exponent(frame);
+    const bool again = *gate != 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = again ? 0.0 : scalbn(out[i], e);
+}
+
+unsigned blocks_of(int64_t n) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + kThreads - 1) / kThreads, 608));
+}
+
+}  // namespace
+
+cudaError_t launch_frame(const double* X, int64_t N, MbmFrame* frame, float4* xh, float4* xl,
+                         double4_32a* x4, int* gate, int* flags, cudaStream_t s) {
+    extent_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, frame, gate);
+    frame_pack_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, frame, xh, xl, x4, flags);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_unframe(const MbmFrame* frame, int degree, const int* gate, double* out,
+                           int64_t n, cudaStream_t s) {
+    unframe_kernel<<<blocks_of(n), kThreads, 0, s>>>(frame, degree, gate, out, n);
+    return cudaGetLastError();
+}

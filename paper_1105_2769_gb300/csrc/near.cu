@@ -22,10 +22,16 @@ namespace {
 
 constexpr int kRowWarps = 8;
 
+__device__ __noinline__ bool differ(const double* __restrict__ X, int i, int j) {
+    return X[3 * (int64_t)i] != X[3 * (int64_t)j] || X[3 * (int64_t)i + 1] != X[3 * (int64_t)j + 1] ||
+           X[3 * (int64_t)i + 2] != X[3 * (int64_t)j + 2];
+}
+
 // One warp per particle: the smallest r^2 of each lane, then of the warp.
 __global__ void __launch_bounds__(kRowWarps * 32)
 knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
-           float* __restrict__ tau, int* __restrict__ flags) {
+           const double* __restrict__ X, float min_d2, float* __restrict__ tau,
+           int* __restrict__ overflow, int* __restrict__ flags) {
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
     if (i >= N) return;
@@ -33,11 +39,14 @@ knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
     float t[kNearK];
 #pragma unroll
     for (int k = 0; k < kNearK; ++k) t[k] = INFINITY;
-    bool bad = false;
+    bool bad = false, close = false;
     for (int j = lane; j < N; j += 32) {
         float s = pair_d2_hilo(ih, il, xh[j], xl[j]);
         if (j == i) continue;
-        bad |= !(s > 0.f);
+        if (!(s > min_d2)) {
+            if (X && s >= 0.f && differ(X, i, j)) close = true;
+            else bad |= !(s > 0.f);
+        }
         if (!(s > 0.f)) continue;
 #pragma unroll
         for (int k = 0; k < kNearK; ++k) {  // insertion into the sorted list
@@ -47,6 +56,7 @@ knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
         }
     }
     if (bad) atomicOr(flags, MBM_FLAG_COINCIDENT);
+    if (close) *overflow = 1;
     float m = INFINITY;
     for (int k = 0; k < kNearK; ++k) {
         m = t[0];
@@ -397,7 +407,8 @@ cudaError_t launch_near_list(const float4* xh, const float4* xl, int64_t N, void
     const unsigned rows = (unsigned)((N + kRowWarps) / kRowWarps);
     cudaError_t e = cudaMemsetAsync(excess, 0, sizeof(*excess), s);
     if (e != cudaSuccess) return e;
-    knn_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->tau, flags);
+    knn_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->X, out->min_d2, out->tau,
+                                               overflow, flags);
     pairs_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->tau, cnt, nullptr, cap,
                                                  excess, nullptr);
     e = cudaGetLastError();

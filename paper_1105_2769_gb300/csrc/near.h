@@ -14,10 +14,16 @@ struct MbmNear {
     float* tau = nullptr;
     int2* pairs = nullptr;      // i < j, ordered by i, then j
     int* count = nullptr;       // their number on the device (0 after an overflow)
+    // What two packed points at r^2 <= min_d2 are: coincident if X holds them equal,
+    // else too close for their packed form, which sets *overflow. Without X:
+    // coincident if r^2 = 0.
+    const double* X = nullptr;
+    float min_d2 = 0.f;
 };
 
 // Thresholds and the ordered list of near pairs, in `mem` (mbm_near_bytes).
-// Sets *overflow if the list does not fit, MBM_FLAG_COINCIDENT on equal points.
+// Sets *overflow if the list does not fit or a pair is too close (in/out->X,
+// min_d2), MBM_FLAG_COINCIDENT on equal points, which are left out.
 cudaError_t launch_near_list(const float4* xh, const float4* xl, int64_t N, void* mem,
                              int* overflow, int* flags, MbmNear* out, cudaStream_t s);
 
