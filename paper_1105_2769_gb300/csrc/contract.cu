@@ -31,9 +31,14 @@
 // 2.8e-8 (9.7e-8) on mixtures; forces 1.6e-7 (3.4e-7), 1.9e-7 (3.3e-7), 2.1e-7
 // (3.8e-7). Without the split, three pieces and eight products were needed for the
 // sweep's accuracy: forces of 8 192 particles took 29 ms against 16.
-// A set with more than 16 near pairs per particle (many equal distances) is left
-// to the FP32 sweep behind, decided on the device (gate), and so is one where a
-// bounded wait ran out; that sweep returns at once otherwise.
+// Range. FP32 carries everything but the sums, down to products of three edges
+// (r^6) and of r^-10, so the points are brought to a common unit first (frame.h):
+// |x - x_0| < 2^10, and r >= 2^-10 there keeps every quantity within 2^-120 and
+// 2^110. The two FP32 parts of a point resolve such distances to 2^-28.
+//
+// A set with a closer pair, a set with more than 16 near pairs per particle (many
+// equal distances), and one where a bounded wait ran out, are left to the FP32 sweep
+// behind, decided on the device (gate); that sweep returns at once otherwise.
 //
 // Kernels: near pairs (near.cu); block maxima -> scales; piece table (stored in
 // the operand layout, so a stage is two kinds of bulk copies and no tensor map);
@@ -47,6 +52,7 @@
 #include "contract.h"
 #include "device_math.cuh"
 #include "forms.cuh"
+#include "frame.h"
 #include "near.h"
 #include "tcgen05.cuh"
 
@@ -641,13 +647,6 @@ pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
     }
 }
 
-__global__ void zero_if_kernel(const int* __restrict__ gate, double* __restrict__ out, int64_t n) {
-    if (!*gate) return;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = 0.0;
-}
-
-
 size_t up256(size_t b) { return mbm_align_up(b, 256); }
 
 // Scratch layout and slab / batch sizes for one solve.
@@ -669,7 +668,8 @@ Plan make_plan(int64_t N, bool weighted, size_t cap) {
     const size_t per_blk = (size_t)kForms * p.nb * kKbPerBlk * kPieces * kPieceB * copies;
     const size_t per_tile = (size_t)kForms * kBM * kBN * sizeof(float) * copies;
     const size_t fixed =
-        up256((size_t)p.n_pad * 32) + 8 * (size_t)p.n_pad + mbm_near_bytes(N) + 131072;
+        up256((size_t)p.n_pad * (weighted ? 40 : 32)) + 8 * (size_t)p.n_pad + mbm_near_bytes(N) +
+        131072;
     // per 256 columns of a slab: ea and f (and the weighted ones)
     const size_t per_blk_f = (size_t)p.n_pad * 8 * copies;
     if (cap < fixed) return Plan{};
@@ -691,6 +691,9 @@ Plan make_plan(int64_t N, bool weighted, size_t cap) {
 }
 
 }  // namespace
+
+// r^2 of the closest pair that the contraction takes, in the frame (see Range above).
+constexpr float kMinDist2 = 9.5367432e-7f;  // 2^-20
 
 constexpr int64_t kContractMaxN = (int64_t)1 << 20;  // tile numbers fit an int
 
@@ -731,8 +734,10 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     int* gate = head;
     int* ref = head + 1;
     auto* counter = reinterpret_cast<unsigned long long*>(head + 16);
+    auto* frame = reinterpret_cast<MbmFrame*>(head + 32);
     auto* xh = reinterpret_cast<float4*>(take((size_t)N * 16));
     auto* xl = reinterpret_cast<float4*>(take((size_t)N * 16));
+    auto* gs = weighted ? reinterpret_cast<double*>(take((size_t)N * 8)) : nullptr;
     char* near_mem = take(mbm_near_bytes(N));
     auto* row_ea = reinterpret_cast<int*>(take((size_t)n_pad * 4));
     auto* row_eag = reinterpret_cast<int*>(take((size_t)n_pad * 4));
@@ -752,13 +757,15 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     MBM_CUDA_TRY(cudaMemsetAsync(ref, 0x7f, 4, s));
     MBM_CUDA_TRY(cudaMemsetAsync(row_ea, 0x7f, up256((size_t)n_pad * 4) * 2, s));
     MBM_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)N * n_out * sizeof(double), s));
-    MBM_CUDA_TRY(launch_pack_hilo(X, N, xh, xl, ctx->d_flags, s));
+    MBM_CUDA_TRY(launch_frame(X, N, g, frame, xh, xl, nullptr, gs, gate, ctx->d_flags, s));
 
     MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)contract_kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(ContractSmem)));
     mbm_time_begin(ctx, s);
     MbmNear near;
+    near.X = X;
+    near.min_d2 = kMinDist2;
     MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
     // Row exponents come from all columns: with several slabs a first pass over
     // them finds the row exponents before any table is built.
@@ -768,7 +775,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
         scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, nullptr, n_pad, ea,
                                            row_ea);
         if (weighted)
-            scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, g, n_pad, eag,
+            scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, gs, n_pad, eag,
                                                row_eag);
     };
     if (slabs > 1)
@@ -784,7 +791,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
                                             nkb, ea, T);
         if (weighted) {
             factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(eag, row_eag, n_pad, (int)N, fg);
-            table_kernel<<<tgrid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, g, n_pad, p.nb, nkb,
+            table_kernel<<<tgrid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, gs, n_pad, p.nb, nkb,
                                                 eag, Tg);
         }
         MBM_CUDA_TRY(cudaGetLastError());
@@ -798,7 +805,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
                     Tg, T, fg, f, n_pad, p.nb, nkb, t0, nt, Cg, gate, ctx->wait_cycles);
             auto pass = [&](auto kernel) {
                 kernel<<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, p.nb, t0, near.tau,
-                                                                 C, Cg, g, row_ea, row_eag, ref,
+                                                                 C, Cg, gs, row_ea, row_eag, ref,
                                                                  sign, out);
             };
             if (what == MBM_CONTRACT_PHI) pass(pair_kernel<kPhi>);
@@ -807,12 +814,11 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
             MBM_CUDA_TRY(cudaGetLastError());
         }
     }
-    MBM_CUDA_TRY(launch_near_triples(xh, xl, nullptr, N, near, g,
+    MBM_CUDA_TRY(launch_near_triples(xh, xl, nullptr, N, near, gs,
                                      what == MBM_CONTRACT_PHI ? MBM_NEAR_PHI : MBM_NEAR_GRAD, sign,
                                      out, ctx->num_sms, s));
-    const int64_t n_val = N * n_out;
-    zero_if_kernel<<<(unsigned)((n_val + 255) / 256), 256, 0, s>>>(gate, out, n_val);
-    MBM_CUDA_TRY(cudaGetLastError());
+    MBM_CUDA_TRY(launch_unframe(frame, n_out == 1 ? 9 : 10, gate, out, N * n_out, s));
+    MBM_CUDA_TRY(launch_pack_hilo(X, N, xh, xl, ctx->d_flags, s, gate));  // the sweep's points
     gate_out->gate = gate;
     gate_out->counter = counter;
     gate_out->xh = xh;

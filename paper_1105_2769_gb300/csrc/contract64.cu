@@ -577,7 +577,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
     MBM_CUDA_TRY(cudaMemsetAsync(gate, 0, 256, s));
     MBM_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)n_val * sizeof(double), s));
-    MBM_CUDA_TRY(launch_frame(X, N, frame, xh, xl, x4, gate, ctx->d_flags, s));
+    MBM_CUDA_TRY(launch_frame(X, N, nullptr, frame, xh, xl, x4, nullptr, gate, ctx->d_flags, s));
     auto kernel = stages == 8 ? contract64_kernel<8> : contract64_kernel<16>;
     MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -19,32 +19,45 @@ __device__ __forceinline__ int frame_exponent(const MbmFrame* frame) {
     return m > 0.0 ? 9 - ilogb(m) : 0;
 }
 
+__device__ __forceinline__ int weight_exponent(const MbmFrame* frame) {
+    const double m = __longlong_as_double((long long)frame->weight);
+    return m > 0.0 ? ilogb(m) : 0;
+}
+
 // Non-negative doubles order as their bits do.
+__device__ __forceinline__ void warp_max_into(unsigned long long* dst, double m) {
+    for (int s = 16; s > 0; s >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, s));
+    if ((threadIdx.x & 31) == 0 && m > 0.0)
+        atomicMax(dst, (unsigned long long)__double_as_longlong(m));
+}
+
 __global__ void __launch_bounds__(kThreads)
-extent_kernel(const double* __restrict__ X, int64_t N, MbmFrame* __restrict__ frame,
-              int* __restrict__ gate) {
+extent_kernel(const double* __restrict__ X, int64_t N, const double* __restrict__ g,
+              MbmFrame* __restrict__ frame, int* __restrict__ gate) {
     const double o[3] = {origin(X, 0), origin(X, 1), origin(X, 2)};
-    double m = 0.0;
+    double m = 0.0, w = 0.0;
     bool over = false;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
-         i += (int64_t)gridDim.x * blockDim.x)
+         i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const double x = X[3 * i + c], d = fabs(x - o[c]);
             if (isfinite(d)) m = fmax(m, d);
             else over |= isfinite(x);
         }
-    for (int s = 16; s > 0; s >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, s));
-    if ((threadIdx.x & 31) == 0 && m > 0.0)
-        atomicMax(&frame->extent, (unsigned long long)__double_as_longlong(m));
+        if (g && isfinite(g[i])) w = fmax(w, fabs(g[i]));
+    }
+    warp_max_into(&frame->extent, m);
+    if (g) warp_max_into(&frame->weight, w);
     if (over) *gate = 1;
 }
 
 __global__ void __launch_bounds__(kThreads)
-frame_pack_kernel(const double* __restrict__ X, int64_t N, const MbmFrame* __restrict__ frame,
-                  float4* __restrict__ xh, float4* __restrict__ xl, double4_32a* __restrict__ x4,
+frame_pack_kernel(const double* __restrict__ X, int64_t N, const double* __restrict__ g,
+                  const MbmFrame* __restrict__ frame, float4* __restrict__ xh,
+                  float4* __restrict__ xl, double4_32a* __restrict__ x4, double* __restrict__ gs,
                   int* __restrict__ flags) {
-    const int e = frame_exponent(frame);
+    const int e = frame_exponent(frame), w = weight_exponent(frame);
     const double o[3] = {origin(X, 0), origin(X, 1), origin(X, 2)};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -62,13 +75,14 @@ frame_pack_kernel(const double* __restrict__ X, int64_t N, const MbmFrame* __res
         xh[i] = make_float4(h[0], h[1], h[2], 0.f);
         xl[i] = make_float4(l[0], l[1], l[2], 0.f);
         if (x4) x4[i] = make_double4_32a(y[0], y[1], y[2], 0.0);
+        if (gs) gs[i] = scalbn(g[i], -w);
     }
 }
 
 __global__ void __launch_bounds__(kThreads)
 unframe_kernel(const MbmFrame* __restrict__ frame, int degree, const int* __restrict__ gate,
                double* __restrict__ out, int64_t n) {
-    const int e = degree * frame_exponent(frame);
+    const int e = degree * frame_exponent(frame) + weight_exponent(frame);
     const bool again = *gate != 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -81,10 +95,11 @@ unsigned blocks_of(int64_t n) {
 
 }  // namespace
 
-cudaError_t launch_frame(const double* X, int64_t N, MbmFrame* frame, float4* xh, float4* xl,
-                         double4_32a* x4, int* gate, int* flags, cudaStream_t s) {
-    extent_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, frame, gate);
-    frame_pack_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, frame, xh, xl, x4, flags);
+cudaError_t launch_frame(const double* X, int64_t N, const double* g, MbmFrame* frame, float4* xh,
+                         float4* xl, double4_32a* x4, double* gs, int* gate, int* flags,
+                         cudaStream_t s) {
+    extent_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, g, frame, gate);
+    frame_pack_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, g, frame, xh, xl, x4, gs, flags);
     return cudaGetLastError();
 }
 
