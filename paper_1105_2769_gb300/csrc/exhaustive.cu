@@ -167,8 +167,8 @@ __host__ __device__ __forceinline__ long long pt_block(int A, int B, int NT) {
     return (long long)A * NT - (long long)A * (A - 1) / 2 + (B - A);
 }
 
-// The terms in FP64: distances whose square leaves the FP32 range, and what has
-// to be reported.
+// The terms in FP64: distances whose square leaves the FP32 range or that are less
+// than 2^-22 of the coordinates, and what has to be reported.
 __device__ __noinline__ int pair_terms_f64(const double* __restrict__ X, int a, int b, float v[4]) {
     const double dx = X[3 * (int64_t)b] - X[3 * (int64_t)a];
     const double dy = X[3 * (int64_t)b + 1] - X[3 * (int64_t)a + 1];
@@ -207,7 +207,10 @@ pair_table_kernel(const double* __restrict__ X, const float4* __restrict__ xh,
                 const df d[3] = {df_diff(qh.x, ql.x, ph.x, pl.x), df_diff(qh.y, ql.y, ph.y, pl.y),
                                  df_diff(qh.z, ql.z, ph.z, pl.z)};
                 const df s2 = df_dot(d, d);
-                if (s2.h > 1e-30f && s2.h < 1e30f) {
+                // (a coordinate's two parts hold it to 2^-50)
+                const float m = fmaxf(fmaxf(fmaxf(fabsf(ph.x), fabsf(ph.y)), fabsf(ph.z)),
+                                      fmaxf(fmaxf(fabsf(qh.x), fabsf(qh.y)), fabsf(qh.z)));
+                if (s2.h > 1e-30f && s2.h < 1e30f && s2.h > 5.7e-14f * (m * m)) {
                     const df y = df_rsqrt(s2);
                     v[c][0] = df_mul(d[0], y).h;
                     v[c][1] = df_mul(d[1], y).h;
