@@ -192,9 +192,9 @@ void mbm_time_end(mbm_ctx* ctx, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // Exhaustive solves (steps a1 + a2/a3).
 // ---------------------------------------------------------------------------
-// FP32 bulk from kContractMinPhi particles is a contraction (contract.cu). Below, or
-// if its scratch does not fit the context's budget or the device, the triple sweep
-// reads a pair table (NT(NT+1)/2 blocks of 16 KB: 13 MB at N = 1 279, 34 GB at
+// FP32 bulk from kContractMinPhi particles is a contraction (contract.cu). Below, if
+// its scratch does not fit the context's budget or the device, or for a set that it
+// gives back, the triple sweep reads a pair table (NT(NT+1)/2 blocks of 16 KB: 13 MB at N = 1 279, 34 GB at
 // 65 536). Larger sets, or a table that does not fit either, form pair terms in
 // the kernel instead (FP32 set-up, a few ulp per pair term).
 constexpr int64_t kPairTableMaxN = 65536;
@@ -207,8 +207,15 @@ static mbm_status run_exhaustive(mbm_ctx* ctx, const double* X, int64_t N, int m
         MbmGate g;
         MBM_TRY(mbm_contract(ctx, X, N, nullptr, MBM_CONTRACT_PHI, 1.0, phi, s, &done, &g));
         if (done) {
-            MBM_CUDA_TRY(launch_exh_fp32(g.xh, g.xl, N, phi, g.counter, ctx->d_flags, ctx->num_sms,
-                                         s, g.gate));
+            // a set that the contraction gives back
+            if (N <= kPairTableMaxN && pair_table_bytes(N) <= g.room_bytes) {
+                MBM_CUDA_TRY(launch_pair_table(X, g.xh, g.xl, N, g.room, ctx->d_flags, s, g.gate));
+                MBM_CUDA_TRY(launch_exh_fp32_table(g.room, N, phi, g.counter, ctx->d_flags,
+                                                   ctx->num_sms, s, g.gate));
+            } else {
+                MBM_CUDA_TRY(launch_exh_fp32(g.xh, g.xl, N, phi, g.counter, ctx->d_flags,
+                                             ctx->num_sms, s, g.gate));
+            }
             mbm_time_end(ctx, s);
             if (validate) return mbm_check_flags(ctx, s);
             return MBM_OK;

@@ -91,7 +91,8 @@ __device__ __forceinline__ float pow2f(int e) {  // 2^e, 0 below the normal rang
 __global__ void __launch_bounds__(kBlk)
 scale_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int b0,
              const float* __restrict__ tau, const double* __restrict__ g, int n_pad,
-             int* __restrict__ ea, int* __restrict__ row_ea) {
+             int* __restrict__ ea, int* __restrict__ row_ea, const int* __restrict__ gate) {
+    if (*gate) return;
     __shared__ float4 kh[kBlk], kl[kBlk];
     __shared__ float kg[kBlk], kt[kBlk];
     const int b = blockIdx.y, k0 = (b0 + b) * kBlk;
@@ -162,7 +163,9 @@ factor_kernel(const int* __restrict__ ea, const int* __restrict__ row_ea, int n_
 __global__ void __launch_bounds__(kBlk)
 table_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int b0,
              const float* __restrict__ tau, const double* __restrict__ g, int n_pad, int nb,
-             int nkb, const int* __restrict__ ea, unsigned char* __restrict__ T) {
+             int nkb, const int* __restrict__ ea, unsigned char* __restrict__ T,
+             const int* __restrict__ gate) {
+    if (*gate) return;
     __shared__ float coef[kForms][5];
     __shared__ float4 kh[8], kl[8];
     __shared__ float kg[8], kt[8];
@@ -314,8 +317,10 @@ __device__ __forceinline__ void drain(unsigned addr, const float* fj, float2 fi,
 __global__ void __launch_bounds__(kThreads, 1)
 contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __restrict__ TB,
                 const float* __restrict__ fA, const float* __restrict__ fB, int n_pad, int nb,
-                int nkb, int t0, int nt, float* __restrict__ C, int* __restrict__ gate,
+                int nkb, int t0, int nt, float* __restrict__ C, int* gate,
                 long long wait_limit) {
+    // (a CTA of this launch may set it meanwhile: one answer for all threads)
+    if (__syncthreads_or(*gate)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ContractSmem& sm = *reinterpret_cast<ContractSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -503,7 +508,9 @@ pair_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
             const float* __restrict__ tau, const float* __restrict__ C,
             const float* __restrict__ Cg, const double* __restrict__ g,
             const int* __restrict__ row_ea, const int* __restrict__ row_eag,
-            const int* __restrict__ ref, double sign, double* __restrict__ out) {
+            const int* __restrict__ ref, double sign, double* __restrict__ out,
+            const int* __restrict__ gate) {
+    if (*gate) return;
     constexpr int kVals = Mode == kPhi ? 1 : 3;
     __shared__ float4 jh[kBN], jl[kBN];
     __shared__ float wj[kBN], gj[kBN], tj[kBN];
@@ -659,7 +666,13 @@ struct Plan {
 // Slabs have 4 096 columns (fewer where their table would pass 16 GB), whatever
 // the room: sums over a slab are FP32 and results should not depend on what else
 // the device holds. Only a context budget that is too small for that shortens them.
-Plan make_plan(int64_t N, bool weighted, size_t cap) {
+// A potential's scratch has room for the pair table of the sweep behind, which solves
+// a set that the contraction gives back (the contraction's own buffers are free by
+// then), up to kTableRoom (N = 33 000). Beyond, that sweep forms its pair terms itself.
+constexpr size_t kTableRoom = (size_t)9 << 30;
+
+Plan make_plan(int64_t N, int what, size_t cap) {
+    const bool weighted = what == MBM_CONTRACT_VJP;
     Plan p;
     p.nb = (int)((N + kBlk - 1) / kBlk);
     p.n_pad = p.nb * kBlk;
@@ -687,6 +700,10 @@ Plan make_plan(int64_t N, bool weighted, size_t cap) {
     p.table = per_blk / copies * p.n_blk;
     p.cbuf = per_tile / copies * p.batch;
     p.total = fixed + (per_blk + per_blk_f) * p.n_blk + per_tile * p.batch;
+    if (what == MBM_CONTRACT_PHI) {
+        const size_t sweep = fixed + per_blk_f * p.n_blk + pair_table_bytes(N);
+        if (pair_table_bytes(N) <= kTableRoom && sweep <= cap) p.total = std::max(p.total, sweep);
+    }
     return p;
 }
 
@@ -697,13 +714,13 @@ constexpr float kMinDist2 = 9.5367432e-7f;  // 2^-20
 
 constexpr int64_t kContractMaxN = (int64_t)1 << 20;  // tile numbers fit an int
 
-static Plan plan_for(int64_t N, bool weighted, size_t cap) {
-    return N <= kContractMaxN ? make_plan(N, weighted, cap) : Plan{};
+static Plan plan_for(int64_t N, int what, size_t cap) {
+    return N <= kContractMaxN ? make_plan(N, what, cap) : Plan{};
 }
 
 size_t mbm_contract_bytes(int64_t N, bool forces) {
     if (N < (forces ? kContractMinForces : kContractMinPhi)) return 0;
-    return plan_for(N, false, (size_t)1 << 60).total;
+    return plan_for(N, forces ? MBM_CONTRACT_FORCES : MBM_CONTRACT_PHI, (size_t)1 << 60).total;
 }
 
 mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* g, int what,
@@ -715,7 +732,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
         cap = ctx->budget > others ? ctx->budget - others : 0;
     }
     const bool weighted = what == MBM_CONTRACT_VJP;
-    const Plan p = plan_for(N, weighted, cap);
+    const Plan p = plan_for(N, what, cap);
     if (!p.n_blk) return MBM_OK;
     const mbm_status rs = mbm_scratch_reserve(ctx, p.total);
     if (rs != MBM_OK) {
@@ -773,10 +790,10 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     auto scales = [&](int b0, int nblk) {
         const dim3 grid(p.nb, nblk);
         scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, nullptr, n_pad, ea,
-                                           row_ea);
+                                           row_ea, gate);
         if (weighted)
             scale_kernel<<<grid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, gs, n_pad, eag,
-                                               row_eag);
+                                               row_eag, gate);
     };
     if (slabs > 1)
         for (int b0 = 0; b0 < p.nb; b0 += p.n_blk) scales(b0, std::min(p.n_blk, p.nb - b0));
@@ -788,11 +805,11 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
         factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(ea, row_ea, n_pad, (int)N, f);
         const dim3 tgrid(p.nb, nkb, kBK / 8);
         table_kernel<<<tgrid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, nullptr, n_pad, p.nb,
-                                            nkb, ea, T);
+                                            nkb, ea, T, gate);
         if (weighted) {
             factor_kernel<<<dim3(p.nb, nblk), kBlk, 0, s>>>(eag, row_eag, n_pad, (int)N, fg);
             table_kernel<<<tgrid, kBlk, 0, s>>>(xh, xl, (int)N, b0, near.tau, gs, n_pad, p.nb, nkb,
-                                                eag, Tg);
+                                                eag, Tg, gate);
         }
         MBM_CUDA_TRY(cudaGetLastError());
         for (int t0 = 0; t0 < p.tiles; t0 += p.batch) {
@@ -806,7 +823,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
             auto pass = [&](auto kernel) {
                 kernel<<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, p.nb, t0, near.tau,
                                                                  C, Cg, gs, row_ea, row_eag, ref,
-                                                                 sign, out);
+                                                                 sign, out, gate);
             };
             if (what == MBM_CONTRACT_PHI) pass(pair_kernel<kPhi>);
             else if (what == MBM_CONTRACT_FORCES) pass(pair_kernel<kForce>);
@@ -816,13 +833,16 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     }
     MBM_CUDA_TRY(launch_near_triples(xh, xl, nullptr, N, near, gs,
                                      what == MBM_CONTRACT_PHI ? MBM_NEAR_PHI : MBM_NEAR_GRAD, sign,
-                                     out, ctx->num_sms, s));
+                                     out, ctx->num_sms, gate, s));
     MBM_CUDA_TRY(launch_unframe(frame, n_out == 1 ? 9 : 10, gate, out, N * n_out, s));
     MBM_CUDA_TRY(launch_pack_hilo(X, N, xh, xl, ctx->d_flags, s, gate));  // the sweep's points
     gate_out->gate = gate;
     gate_out->counter = counter;
     gate_out->xh = xh;
     gate_out->xl = xl;
+    gate_out->room = T;
+    gate_out->room_bytes =
+        p.total - (size_t)(reinterpret_cast<char*>(T) - static_cast<char*>(ctx->scratch));
     *done = true;
     return MBM_OK;
 }

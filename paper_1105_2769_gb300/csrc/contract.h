@@ -21,6 +21,8 @@ struct MbmGate {
     unsigned long long* counter = nullptr;  // zeroed
     const float4* xh = nullptr;             // packed points
     const float4* xl = nullptr;
+    void* room = nullptr;                   // scratch that is free by then
+    size_t room_bytes = 0;
 };
 
 // Enqueue the solve (FP32-bulk accuracy); *done = false if the scratch does not

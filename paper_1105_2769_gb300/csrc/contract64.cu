@@ -61,7 +61,9 @@ __device__ __forceinline__ double pow2d(int e) {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 exponent_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N, int cols,
-                const float* __restrict__ tau, int n_pad, int* __restrict__ ea) {
+                const float* __restrict__ tau, int n_pad, int* __restrict__ ea,
+                const int* __restrict__ gate) {
+    if (*gate) return;
     __shared__ float4 kh[256], kl[256];
     __shared__ float kt[256];
     const int b = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
@@ -100,7 +102,9 @@ exponent_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, in
 __global__ void __launch_bounds__(kRows)
 digit_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
              const float4* __restrict__ xl, int N, const float* __restrict__ tau, int n_pad, int nb,
-             int nkb, int stages, const int* __restrict__ ea, unsigned char* __restrict__ T) {
+             int nkb, int stages, const int* __restrict__ ea, unsigned char* __restrict__ T,
+             const int* __restrict__ gate) {
+    if (*gate) return;
     __shared__ double coef[kForms][5];
     const int rb = blockIdx.x, kb = blockIdx.y, k8 = blockIdx.z;
     const int row = threadIdx.x, i = rb * kRows + row;
@@ -246,7 +250,9 @@ __device__ __forceinline__ void read_out(unsigned addr, unsigned long long (&t)[
 template <int Stages>  // stages per block
 __global__ void __launch_bounds__(kThreads, 1)
 contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, int nt,
-                  longlong2* __restrict__ C, int* __restrict__ gate, long long wait_limit) {
+                  longlong2* __restrict__ C, int* gate, long long wait_limit) {
+    // (a CTA of this launch may set it meanwhile: one answer for all threads)
+    if (__syncthreads_or(*gate)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ContractSmem& sm = *reinterpret_cast<ContractSmem*>(smem_raw);
     constexpr int kBase = base_shift(Stages);
@@ -404,7 +410,9 @@ __global__ void __launch_bounds__(256)
 pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
               const float4* __restrict__ xl, int N, int n_pad, int n_blk, int shift, int t0,
               const float* __restrict__ tau, const int* __restrict__ ea,
-              const longlong2* __restrict__ C, double sign, double* __restrict__ out) {
+              const longlong2* __restrict__ C, double sign, double* __restrict__ out,
+              const int* __restrict__ gate) {
+    if (*gate) return;
     constexpr int kVals = Grad ? 3 : 1;
     __shared__ double coef[kForms][5];
     __shared__ double red[8][kPairCols][33];
@@ -588,9 +596,9 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     near.min_d2 = kMinDist2;
     MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
     exponent_kernel<<<dim3(n_pad / 256, n_blk), 256, 0, s>>>(xh, xl, (int)N, cols, near.tau, n_pad,
-                                                            ea);
+                                                            ea, gate);
     digit_kernel<<<dim3(nb, nkb, kBK / 8), kRows, 0, s>>>(x4, xh, xl, (int)N, near.tau, n_pad, nb,
-                                                          nkb, stages, ea, T);
+                                                          nkb, stages, ea, T, gate);
     MBM_CUDA_TRY(cudaGetLastError());
     for (int t0 = 0; t0 < tiles; t0 += batch) {
         const int nt = std::min(batch, tiles - t0);
@@ -599,12 +607,12 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
         auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
         pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(x4, xh, xl, (int)N, n_pad, n_blk,
                                                   base_shift(stages), t0, near.tau, ea, C, sign,
-                                                  out);
+                                                  out, gate);
         MBM_CUDA_TRY(cudaGetLastError());
     }
     MBM_CUDA_TRY(launch_near_triples(xh, xl, x4, N, near, nullptr,
                                      grad ? MBM_NEAR_GRAD : MBM_NEAR_PHI, sign, out, ctx->num_sms,
-                                     s));
+                                     gate, s));
     MBM_CUDA_TRY(launch_unframe(frame, grad ? 10 : 9, gate, out, n_val, s));
     MBM_CUDA_TRY(launch_pack_f64(X, N, x4, ctx->d_flags, s, gate));  // the sweep's points
     gate_out->gate = gate;

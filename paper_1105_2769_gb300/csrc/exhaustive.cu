@@ -187,7 +187,9 @@ __device__ __noinline__ int pair_terms_f64(const double* __restrict__ X, int a, 
 __global__ void __launch_bounds__(256)
 pair_table_kernel(const double* __restrict__ X, const float4* __restrict__ xh,
                   const float4* __restrict__ xl, int N, int NT,
-                  mbm_tile::PairBlock* __restrict__ pt, int* __restrict__ flags) {
+                  mbm_tile::PairBlock* __restrict__ pt, int* __restrict__ flags,
+                  const int* __restrict__ gate) {
+    if (gate && !*gate) return;
     const int A = blockIdx.y;
     const long long per_row = (long long)(NT - A) * (kTile * kTile / 2);
     mbm_tile::PairBlock* rowbase = pt + pt_block(A, A, NT);
@@ -268,7 +270,8 @@ constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz: a copy that n
 __global__ void __launch_bounds__(kWarps32 * 32, 2)
 exh_fp32_pt_kernel(const mbm_tile::PairBlock* __restrict__ pt, int N, int NT, long long n_items,
                    int n_chunk, int per, unsigned long long* __restrict__ counter, double* __restrict__ phi,
-                   int* __restrict__ flags) {
+                   int* __restrict__ flags, const int* __restrict__ gate) {
+    if (gate && !*gate) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     PtSmem& sm = *reinterpret_cast<PtSmem*>(smem_raw);
     const int lane = threadIdx.x & 31;
@@ -588,18 +591,20 @@ size_t pair_table_bytes(int64_t N) {
 }
 
 cudaError_t launch_pair_table(const double* X, const float4* xh, const float4* xl, int64_t N,
-                              void* table, int* flags, cudaStream_t s) {
+                              void* table, int* flags, cudaStream_t s, const int* gate) {
     const int NT = (int)((N + kTile - 1) / kTile);
     const long long per_row0 = (long long)NT * (kTile * kTile / 2);
-    const int gx = (int)std::min<long long>((per_row0 + 255) / 256, 1024);
+    // behind a gate few CTAs, which mostly only look at it
+    const int gx = (int)std::min<long long>((per_row0 + 255) / 256, gate ? 8 : 1024);
     pair_table_kernel<<<dim3(gx, NT), 256, 0, s>>>(X, xh, xl, (int)N, NT,
-                                                   static_cast<mbm_tile::PairBlock*>(table), flags);
+                                                   static_cast<mbm_tile::PairBlock*>(table), flags,
+                                                   gate);
     return cudaGetLastError();
 }
 
 cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
                                   unsigned long long* counter, int* flags, int num_sms,
-                                  cudaStream_t s) {
+                                  cudaStream_t s, const int* gate) {
     const int NT = (int)((N + kTile - 1) / kTile);
     // One I tile per warp and item while whole items are too few to fill two CTAs
     // per SM several times: N = 1 000 has 528 of them, of up to 32 I tiles.
@@ -615,7 +620,7 @@ cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
     const int grid = grid_for((const void*)exh_fp32_pt_kernel, threads, smem, num_sms, items);
     exh_fp32_pt_kernel<<<grid, threads, smem, s>>>(
         static_cast<const mbm_tile::PairBlock*>(table), (int)N, NT, items, n_chunk, per, counter, phi,
-        flags);
+        flags, gate);
     return cudaGetLastError();
 }
 

@@ -95,10 +95,10 @@ cudaError_t launch_exh_fp32(const float4* xhi, const float4* xlo, int64_t N, dou
 // sum that reads it.
 size_t pair_table_bytes(int64_t N);
 cudaError_t launch_pair_table(const double* X, const float4* xh, const float4* xl, int64_t N,
-                              void* table, int* flags, cudaStream_t s);
+                              void* table, int* flags, cudaStream_t s, const int* gate = nullptr);
 cudaError_t launch_exh_fp32_table(const void* table, int64_t N, double* phi,
                                   unsigned long long* counter, int* flags, int num_sms,
-                                  cudaStream_t s);
+                                  cudaStream_t s, const int* gate = nullptr);
 cudaError_t launch_exh_fp64(const double4_32a* x4, int64_t N, double* phi, unsigned long long* counter,
                             int* flags, int num_sms, cudaStream_t s, const int* gate = nullptr);
 // Exact FP32-bulk Phi of sampled particles idx[0..n_idx) (out zeroed by the caller).

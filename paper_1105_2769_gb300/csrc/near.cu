@@ -208,7 +208,9 @@ __global__ void __launch_bounds__(kNearWarps * 32)
 near_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
             const double4_32a* __restrict__ x64, int N, const float* __restrict__ tau,
             const int2* __restrict__ pairs, const int* __restrict__ count,
-            const double* __restrict__ g, double sign, double* __restrict__ out) {
+            const double* __restrict__ g, double sign, double* __restrict__ out,
+            const int* __restrict__ gate) {
+    if (*gate) return;
     constexpr int kRow = Grad ? 6 : 1;   // shares of a and b
     constexpr int kCol = Grad ? 3 : 1;
     __shared__ NearPair<R> np[kChunk];
@@ -423,7 +425,8 @@ cudaError_t launch_near_list(const float4* xh, const float4* xl, int64_t N, void
 
 cudaError_t launch_near_triples(const float4* xh, const float4* xl, const double4_32a* X64,
                                 int64_t N, const MbmNear& near, const double* g, int what,
-                                double sign, double* out, int num_sms, cudaStream_t s) {
+                                double sign, double* out, int num_sms, const int* gate,
+                                cudaStream_t s) {
     const unsigned bx = (unsigned)((N + kNearWarps * 32 - 1) / (kNearWarps * 32));
     // about 2 N pairs; enough CTAs for eight per SM, at least one chunk each
     const int64_t chunks = (2 * N + kChunk - 1) / kChunk;
@@ -434,17 +437,17 @@ cudaError_t launch_near_triples(const float4* xh, const float4* xl, const double
     if (what == MBM_NEAR_PHI) {
         if (X64)
             near_kernel<double, false><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
         else
             near_kernel<float, false><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
     } else {
         if (X64)
             near_kernel<double, true><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
         else
             near_kernel<float, true><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
     }
     return cudaGetLastError();
 }
