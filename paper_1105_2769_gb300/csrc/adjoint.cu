@@ -323,8 +323,11 @@ mbm_status run_adjoint(mbm_ctx* ctx, const double* X, int64_t N, const double* g
                        double* out, double sign, cudaStream_t s) {
     if (mode != MBM_EXH_FP32 && mode != MBM_EXH_FP64)
         return mbm_fail(MBM_ENOTSUP, "forces and VJP support MBM_EXH_FP32 and MBM_EXH_FP64");
-    MBM_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)N * 3 * sizeof(double), s));
-    if (N < 3) return MBM_OK;
+    const size_t out_bytes = (size_t)N * 3 * sizeof(double);
+    if (N < 3) {
+        MBM_CUDA_TRY(cudaMemsetAsync(out, 0, out_bytes, s));
+        return MBM_OK;
+    }
     if (mode == MBM_EXH_FP32 && N >= kContractMinForces && N <= INT_MAX) {
         bool done = false;
         MbmGate gt;
@@ -352,6 +355,7 @@ mbm_status run_adjoint(mbm_ctx* ctx, const double* X, int64_t N, const double* g
                                              : (size_t)N * sizeof(double4_32a);
     MBM_TRY(mbm_scratch_reserve(ctx, 256 + pack));
     char* base = static_cast<char*>(ctx->scratch) + 256;
+    MBM_CUDA_TRY(cudaMemsetAsync(out, 0, out_bytes, s));
     MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
     mbm_time_begin(ctx, s);
     if (mode == MBM_EXH_FP32) {

@@ -33,8 +33,8 @@
 // sweep's accuracy: forces of 8 192 particles took 29 ms against 16.
 // Range. FP32 carries everything but the sums, down to products of three edges
 // (r^6) and of r^-10, so the points are brought to a common unit first (frame.h):
-// |x - x_0| < 2^10, and r >= 2^-10 there keeps every quantity within 2^-120 and
-// 2^110. The two FP32 parts of a point resolve such distances to 2^-28.
+// |x - x_0| < 2^11, and r >= 2^-11.5 there keeps a triple's r^-10 within 2^-128 and
+// 2^115. The two FP32 parts of a point resolve such distances to 2^-25.
 //
 // A set with a closer pair, a set with more than 16 near pairs per particle (many
 // equal distances), and one where a bounded wait ran out, are left to the FP32 sweep
@@ -710,7 +710,7 @@ Plan make_plan(int64_t N, int what, size_t cap) {
 }  // namespace
 
 // r^2 of the closest pair that the contraction takes, in the frame (see Range above).
-constexpr float kMinDist2 = 9.5367432e-7f;  // 2^-20
+constexpr float kMinDist2 = 1.1920929e-7f;  // 2^-23
 
 constexpr int64_t kContractMaxN = (int64_t)1 << 20;  // tile numbers fit an int
 
@@ -773,8 +773,8 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     MBM_CUDA_TRY(cudaMemsetAsync(head, 0, 256, s));
     MBM_CUDA_TRY(cudaMemsetAsync(ref, 0x7f, 4, s));
     MBM_CUDA_TRY(cudaMemsetAsync(row_ea, 0x7f, up256((size_t)n_pad * 4) * 2, s));
-    MBM_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)N * n_out * sizeof(double), s));
-    MBM_CUDA_TRY(launch_frame(X, N, g, frame, xh, xl, nullptr, gs, gate, ctx->d_flags, s));
+    const MbmOut res{out, N * n_out, n_out == 1 ? 9 : 10};
+    MBM_CUDA_TRY(launch_frame(X, N, g, frame, xh, xl, nullptr, gs, res, gate, ctx->d_flags, s));
 
     MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)contract_kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -783,6 +783,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     MbmNear near;
     near.X = X;
     near.min_d2 = kMinDist2;
+    near.excess = counter + 1;
     MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
     // Row exponents come from all columns: with several slabs a first pass over
     // them finds the row exponents before any table is built.
@@ -834,8 +835,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     MBM_CUDA_TRY(launch_near_triples(xh, xl, nullptr, N, near, gs,
                                      what == MBM_CONTRACT_PHI ? MBM_NEAR_PHI : MBM_NEAR_GRAD, sign,
                                      out, ctx->num_sms, gate, s));
-    MBM_CUDA_TRY(launch_unframe(frame, n_out == 1 ? 9 : 10, gate, out, N * n_out, s));
-    MBM_CUDA_TRY(launch_pack_hilo(X, N, xh, xl, ctx->d_flags, s, gate));  // the sweep's points
+    MBM_CUDA_TRY(launch_unframe(X, N, frame, xh, xl, nullptr, res, gate, s));
     gate_out->gate = gate;
     gate_out->counter = counter;
     gate_out->xh = xh;

@@ -14,7 +14,7 @@
 // with the near triples the result is as close to 64 bits as the FP64 sweep's.
 //
 // Range. FP32 carries the near test and the exponents, so the points are brought to
-// a common unit first (frame.h): |x - x_0| < 2^10. With r >= 2^-20 there, every FP32
+// a common unit first (frame.h): |x - x_0| < 2^11. With r >= 2^-19 there, every FP32
 // quantity is in range, and r^2 from the two FP32 parts of a point (2^-49 of it) is
 // within 2^-17: inside the exponents' margin. A set with a closer pair goes to the
 // FP64 sweep, decided on the device (gate); so does one with more than 16 near
@@ -529,7 +529,7 @@ size_t up256(size_t b) { return mbm_align_up(b, 256); }
 }  // namespace
 
 // r^2 of the closest pair that the two FP32 parts of a point resolve, in the frame.
-constexpr float kMinDist2 = 9.094947e-13f;  // 2^-40
+constexpr float kMinDist2 = 3.637979e-12f;  // 2^-38
 
 // Largest N: its digit table (140 N^2 bytes) has to fit the device.
 constexpr int64_t kMaxN64 = 24576;
@@ -581,11 +581,11 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     auto* C = reinterpret_cast<longlong2*>(take(per_tile * batch));
 
     const bool grad = what != MBM_CONTRACT_PHI;
-    const int64_t n_val = N * (grad ? 3 : 1);
     MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
     MBM_CUDA_TRY(cudaMemsetAsync(gate, 0, 256, s));
-    MBM_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)n_val * sizeof(double), s));
-    MBM_CUDA_TRY(launch_frame(X, N, nullptr, frame, xh, xl, x4, nullptr, gate, ctx->d_flags, s));
+    const MbmOut res{out, N * (grad ? 3 : 1), grad ? 10 : 9};
+    MBM_CUDA_TRY(launch_frame(X, N, nullptr, frame, xh, xl, x4, nullptr, res, gate, ctx->d_flags,
+                              s));
     auto kernel = stages == 8 ? contract64_kernel<8> : contract64_kernel<16>;
     MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -594,6 +594,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     MbmNear near;
     near.X = X;
     near.min_d2 = kMinDist2;
+    near.excess = counter + 1;
     MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
     exponent_kernel<<<dim3(n_pad / 256, n_blk), 256, 0, s>>>(xh, xl, (int)N, cols, near.tau, n_pad,
                                                             ea, gate);
@@ -613,8 +614,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     MBM_CUDA_TRY(launch_near_triples(xh, xl, x4, N, near, nullptr,
                                      grad ? MBM_NEAR_GRAD : MBM_NEAR_PHI, sign, out, ctx->num_sms,
                                      gate, s));
-    MBM_CUDA_TRY(launch_unframe(frame, grad ? 10 : 9, gate, out, n_val, s));
-    MBM_CUDA_TRY(launch_pack_f64(X, N, x4, ctx->d_flags, s, gate));  // the sweep's points
+    MBM_CUDA_TRY(launch_unframe(X, N, frame, xh, xl, x4, res, gate, s));
     gate_out->gate = gate;
     gate_out->counter = counter;
     gate_out->x4 = x4;

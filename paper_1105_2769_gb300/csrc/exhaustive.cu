@@ -43,9 +43,7 @@ constexpr int kWarps64 = 4;   // FP64 kernel: 4 warps per CTA
 // Step a1: input pack.
 // ---------------------------------------------------------------------------
 __global__ void pack_hilo_kernel(const double* __restrict__ X, int64_t N, float4* __restrict__ xh,
-                                 float4* __restrict__ xl, int* __restrict__ flags,
-                                 const int* __restrict__ gate) {
-    if (gate && !*gate) return;
+                                 float4* __restrict__ xl, int* __restrict__ flags) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double x = X[3 * i], y = X[3 * i + 1], z = X[3 * i + 2];
@@ -58,8 +56,7 @@ __global__ void pack_hilo_kernel(const double* __restrict__ X, int64_t N, float4
 }
 
 __global__ void pack_f64_kernel(const double* __restrict__ X, int64_t N, double4_32a* __restrict__ x4,
-                                int* __restrict__ flags, const int* __restrict__ gate) {
-    if (gate && !*gate) return;
+                                int* __restrict__ flags) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double x = X[3 * i], y = X[3 * i + 1], z = X[3 * i + 2];
@@ -550,22 +547,20 @@ int grid_for(const void* kernel, int threads, size_t smem, int num_sms, long lon
 }  // namespace
 
 cudaError_t launch_pack_hilo(const double* X, int64_t N, float4* xhi, float4* xlo, int* flags,
-                             cudaStream_t s, const int* gate) {
+                             cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     const int threads = 256;
     const long long blocks = (N + threads - 1) / threads;
     pack_hilo_kernel<<<(unsigned)(blocks < 65535 ? blocks : 65535), threads, 0, s>>>(X, N, xhi, xlo,
-                                                                                    flags, gate);
+                                                                                    flags);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* flags, cudaStream_t s,
-                            const int* gate) {
+cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* flags, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     const int threads = 256;
     const long long blocks = (N + threads - 1) / threads;
-    pack_f64_kernel<<<(unsigned)(blocks < 65535 ? blocks : 65535), threads, 0, s>>>(X, N, x4, flags,
-                                                                                   gate);
+    pack_f64_kernel<<<(unsigned)(blocks < 65535 ? blocks : 65535), threads, 0, s>>>(X, N, x4, flags);
     return cudaGetLastError();
 }
 

@@ -16,7 +16,7 @@ __device__ __forceinline__ double origin(const double* X, int c) {
 
 __device__ __forceinline__ int frame_exponent(const MbmFrame* frame) {
     const double m = __longlong_as_double((long long)frame->extent);
-    return m > 0.0 ? 9 - ilogb(m) : 0;
+    return m > 0.0 ? 10 - ilogb(m) : 0;
 }
 
 __device__ __forceinline__ int weight_exponent(const MbmFrame* frame) {
@@ -52,15 +52,21 @@ extent_kernel(const double* __restrict__ X, int64_t N, const double* __restrict_
     if (over) *gate = 1;
 }
 
+__device__ __forceinline__ void split(double x, float& h, float& l) {
+    h = (float)x;
+    l = (float)(x - (double)h);
+}
+
 __global__ void __launch_bounds__(kThreads)
-frame_pack_kernel(const double* __restrict__ X, int64_t N, const double* __restrict__ g,
-                  const MbmFrame* __restrict__ frame, float4* __restrict__ xh,
-                  float4* __restrict__ xl, double4_32a* __restrict__ x4, double* __restrict__ gs,
-                  int* __restrict__ flags) {
+frame_kernel(const double* __restrict__ X, int64_t N, const double* __restrict__ g,
+             const MbmFrame* __restrict__ frame, float4* __restrict__ xh, float4* __restrict__ xl,
+             double4_32a* __restrict__ x4, double* __restrict__ gs, MbmOut out,
+             int* __restrict__ flags) {
     const int e = frame_exponent(frame), w = weight_exponent(frame);
     const double o[3] = {origin(X, 0), origin(X, 1), origin(X, 2)};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
-         i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = first; i < N; i += step) {
         double y[3];
         float h[3], l[3];
 #pragma unroll
@@ -68,25 +74,41 @@ frame_pack_kernel(const double* __restrict__ X, int64_t N, const double* __restr
             const double x = X[3 * i + c];
             if (!isfinite(x)) atomicOr(flags, MBM_FLAG_NONFINITE);
             y[c] = scalbn(x, e);
-            const double d = scalbn(x - o[c], e);
-            h[c] = (float)d;
-            l[c] = (float)(d - (double)h[c]);
+            split(scalbn(x - o[c], e), h[c], l[c]);
         }
         xh[i] = make_float4(h[0], h[1], h[2], 0.f);
         xl[i] = make_float4(l[0], l[1], l[2], 0.f);
         if (x4) x4[i] = make_double4_32a(y[0], y[1], y[2], 0.0);
         if (gs) gs[i] = scalbn(g[i], -w);
     }
+    for (int64_t i = first; i < out.n; i += step) out.v[i] = 0.0;
 }
 
 __global__ void __launch_bounds__(kThreads)
-unframe_kernel(const MbmFrame* __restrict__ frame, int degree, const int* __restrict__ gate,
-               double* __restrict__ out, int64_t n) {
-    const int e = degree * frame_exponent(frame) + weight_exponent(frame);
-    const bool again = *gate != 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = again ? 0.0 : scalbn(out[i], e);
+unframe_kernel(const double* __restrict__ X, int64_t N, const MbmFrame* __restrict__ frame,
+               float4* __restrict__ xh, float4* __restrict__ xl, double4_32a* __restrict__ x4,
+               MbmOut out, const int* __restrict__ gate) {
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    if (!*gate) {
+        const int e = out.degree * frame_exponent(frame) + weight_exponent(frame);
+        for (int64_t i = first; i < out.n; i += step) out.v[i] = scalbn(out.v[i], e);
+        return;
+    }
+    for (int64_t i = first; i < out.n; i += step) out.v[i] = 0.0;
+    for (int64_t i = first; i < N; i += step) {
+        const double x = X[3 * i], y = X[3 * i + 1], z = X[3 * i + 2];
+        if (x4) {
+            x4[i] = make_double4_32a(x, y, z, 0.0);
+        } else {
+            float h[3], l[3];
+            split(x, h[0], l[0]);
+            split(y, h[1], l[1]);
+            split(z, h[2], l[2]);
+            xh[i] = make_float4(h[0], h[1], h[2], 0.f);
+            xl[i] = make_float4(l[0], l[1], l[2], 0.f);
+        }
+    }
 }
 
 unsigned blocks_of(int64_t n) {
@@ -96,15 +118,15 @@ unsigned blocks_of(int64_t n) {
 }  // namespace
 
 cudaError_t launch_frame(const double* X, int64_t N, const double* g, MbmFrame* frame, float4* xh,
-                         float4* xl, double4_32a* x4, double* gs, int* gate, int* flags,
-                         cudaStream_t s) {
+                         float4* xl, double4_32a* x4, double* gs, const MbmOut& out, int* gate,
+                         int* flags, cudaStream_t s) {
     extent_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, g, frame, gate);
-    frame_pack_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, g, frame, xh, xl, x4, gs, flags);
+    frame_kernel<<<blocks_of(N), kThreads, 0, s>>>(X, N, g, frame, xh, xl, x4, gs, out, flags);
     return cudaGetLastError();
 }
 
-cudaError_t launch_unframe(const MbmFrame* frame, int degree, const int* gate, double* out,
-                           int64_t n, cudaStream_t s) {
-    unframe_kernel<<<blocks_of(n), kThreads, 0, s>>>(frame, degree, gate, out, n);
+cudaError_t launch_unframe(const double* X, int64_t N, const MbmFrame* frame, float4* xh, float4* xl,
+                           double4_32a* x4, const MbmOut& out, const int* gate, cudaStream_t s) {
+    unframe_kernel<<<blocks_of(out.n), kThreads, 0, s>>>(X, N, frame, xh, xl, x4, out, gate);
     return cudaGetLastError();
 }

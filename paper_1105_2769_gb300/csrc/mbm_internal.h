@@ -76,13 +76,11 @@ static inline size_t mbm_align_up(size_t x, size_t a) { return (x + a - 1) / a *
 // ---------------------------------------------------------------------------
 // Launchers (each .cu file owns its kernels).
 // ---------------------------------------------------------------------------
-// Input pack (step a1): FP64 AoS -> FP32 hi/lo float4 pairs, finite check (gate: as
-// below).
+// Input pack (step a1): FP64 AoS -> FP32 hi/lo float4 pairs, finite check.
 cudaError_t launch_pack_hilo(const double* X, int64_t N, float4* xhi, float4* xlo, int* flags,
-                             cudaStream_t s, const int* gate = nullptr);
-// Input pack to FP64 float4-like (x, y, z, 0) double quads (gate: as below).
-cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* flags, cudaStream_t s,
-                            const int* gate = nullptr);
+                             cudaStream_t s);
+// Input pack to FP64 float4-like (x, y, z, 0) double quads.
+cudaError_t launch_pack_f64(const double* X, int64_t N, double4_32a* x4, int* flags, cudaStream_t s);
 
 // Exhaustive sums (steps a2/a3). phi must be zeroed by the caller.
 // counter: one zeroed unsigned long long of scratch for dynamic scheduling.

@@ -22,9 +22,23 @@ namespace {
 
 constexpr int kRowWarps = 8;
 
-__device__ __noinline__ bool differ(const double* __restrict__ X, int i, int j) {
-    return X[3 * (int64_t)i] != X[3 * (int64_t)j] || X[3 * (int64_t)i + 1] != X[3 * (int64_t)j + 1] ||
-           X[3 * (int64_t)i + 2] != X[3 * (int64_t)j + 2];
+// What the pairs of particle i at r^2 <= min_d2 are (rare): MBM_FLAG_COINCIDENT, or
+// too close for the packed points, which *overflow takes.
+__device__ __noinline__ void sort_out_close(const float4* __restrict__ xh,
+                                            const float4* __restrict__ xl, int N, int i, int lane,
+                                            const double* __restrict__ X, float min_d2,
+                                            int* __restrict__ overflow, int* __restrict__ flags) {
+    for (int j = lane; j < N; j += 32) {
+        const float s = pair_d2_hilo(xh[i], xl[i], xh[j], xl[j]);
+        if (j == i || s > min_d2) continue;
+        bool same = !(s > 0.f);
+        if (X && s >= 0.f) {
+            same = true;
+            for (int c = 0; c < 3; ++c) same &= X[3 * (int64_t)i + c] == X[3 * (int64_t)j + c];
+            if (!same) *overflow = 1;
+        }
+        if (same) atomicOr(flags, MBM_FLAG_COINCIDENT);
+    }
 }
 
 // One warp per particle: the smallest r^2 of each lane, then of the warp.
@@ -39,14 +53,11 @@ knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
     float t[kNearK];
 #pragma unroll
     for (int k = 0; k < kNearK; ++k) t[k] = INFINITY;
-    bool bad = false, close = false;
+    bool close = false;
     for (int j = lane; j < N; j += 32) {
         float s = pair_d2_hilo(ih, il, xh[j], xl[j]);
         if (j == i) continue;
-        if (!(s > min_d2)) {
-            if (X && s >= 0.f && differ(X, i, j)) close = true;
-            else bad |= !(s > 0.f);
-        }
+        close |= !(s > min_d2);
         if (!(s > 0.f)) continue;
 #pragma unroll
         for (int k = 0; k < kNearK; ++k) {  // insertion into the sorted list
@@ -55,8 +66,8 @@ knn_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, int N,
             t[k] = lo;
         }
     }
-    if (bad) atomicOr(flags, MBM_FLAG_COINCIDENT);
-    if (close) *overflow = 1;
+    if (__any_sync(0xffffffffu, close))
+        sort_out_close(xh, xl, N, i, lane, X, min_d2, overflow, flags);
     float m = INFINITY;
     for (int k = 0; k < kNearK; ++k) {
         m = t[0];
@@ -402,13 +413,17 @@ cudaError_t launch_near_list(const float4* xh, const float4* xl, int64_t N, void
     int* cnt = reinterpret_cast<int*>(take((size_t)(N + 1) * 4));
     int* off = reinterpret_cast<int*>(take((size_t)(N + 1) * 4));
     out->count = reinterpret_cast<int*>(take(256));
-    auto* excess = reinterpret_cast<unsigned long long*>(out->count + 16);
+    auto* excess = out->excess;
     out->pairs = reinterpret_cast<int2*>(take((size_t)N * kNearMax * sizeof(int2)));
     void* tmp = take(mbm_scan_temp_bytes_i32(N + 1));
     const int cap = (int)(N * kNearMax);
     const unsigned rows = (unsigned)((N + kRowWarps) / kRowWarps);
-    cudaError_t e = cudaMemsetAsync(excess, 0, sizeof(*excess), s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
+    if (!excess) {
+        excess = reinterpret_cast<unsigned long long*>(out->count + 16);
+        e = cudaMemsetAsync(excess, 0, sizeof(*excess), s);
+        if (e != cudaSuccess) return e;
+    }
     knn_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->X, out->min_d2, out->tau,
                                                overflow, flags);
     pairs_kernel<<<rows, kRowWarps * 32, 0, s>>>(xh, xl, (int)N, out->tau, cnt, nullptr, cap,

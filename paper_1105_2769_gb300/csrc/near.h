@@ -19,6 +19,7 @@ struct MbmNear {
     // coincident if r^2 = 0.
     const double* X = nullptr;
     float min_d2 = 0.f;
+    unsigned long long* excess = nullptr;  // zeroed word for the count, or NULL
 };
 
 // Thresholds and the ordered list of near pairs, in `mem` (mbm_near_bytes).
