@@ -120,11 +120,11 @@ mbm_status mbm_ctx_destroy(mbm_ctx* ctx);
 /* Library-owned device bytes currently held by the context. */
 size_t mbm_ctx_bytes_in_use(const mbm_ctx* ctx);
 
-/* Clock cycles after which a wait inside the tensor-core kernels gives up
- * (default 4e9, about 2 s; 0 = at once, which makes the wait run out on purpose).
- * No wait of a healthy solve comes near the default. A solve whose wait ran out is
- * done again on the device by the triple sweep: its result is right, and late. */
-mbm_status mbm_ctx_set_wait_cycles(mbm_ctx* ctx, int64_t cycles);
+/* Waits inside the tensor-core kernels are bounded (about 2 s, which no healthy solve
+ * comes near); a solve whose wait ran out is done again on the device by the triple
+ * sweep, so its result is right, and late. For tests: 1 makes a wait of every such
+ * kernel run out, with work of its own in flight; 0 (the default) ends that. */
+mbm_status mbm_ctx_expire_waits(mbm_ctx* ctx, int enable);
 
 /* Enable (1) or disable (0) CUDA-event timing of each solve's dominant
  * kernel (the exhaustive kernel, or the tree path's base-case kernels).

@@ -82,7 +82,7 @@ SIGNATURES = {
     "mbm_ctx_create": (_int, [_int, ctypes.c_size_t, ctypes.POINTER(_vp)]),
     "mbm_ctx_destroy": (_int, [_vp]),
     "mbm_ctx_bytes_in_use": (ctypes.c_size_t, [_vp]),
-    "mbm_ctx_set_wait_cycles": (_int, [_vp, _i64]),
+    "mbm_ctx_expire_waits": (_int, [_vp, _int]),
     "mbm_ctx_set_timing": (_int, [_vp, _int]),
     "mbm_ctx_last_kernel_ms": (ctypes.c_double, [_vp]),
     "mbm_potential": (_int, [_vp, _vp, _i64, _dbl, _dbl, _int, _vp, _vp]),

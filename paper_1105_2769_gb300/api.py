@@ -46,9 +46,9 @@ class Context:
         """Dominant-kernel time of the last timed solve (waits for it)."""
         return float(_lib.load().mbm_ctx_last_kernel_ms(self.handle))
 
-    def set_wait_cycles(self, cycles: int):
-        """Bound of the waits inside the tensor-core kernels (0: they run out at once)."""
-        _lib.check(_lib.load().mbm_ctx_set_wait_cycles(self.handle, int(cycles)))
+    def expire_waits(self, enable: bool = True):
+        """For tests: a wait of every tensor-core kernel runs out (the triple sweep solves)."""
+        _lib.check(_lib.load().mbm_ctx_expire_waits(self.handle, int(bool(enable))))
 
     def bytes_in_use(self) -> int:
         return int(_lib.load().mbm_ctx_bytes_in_use(self.handle))

@@ -139,11 +139,10 @@ extern "C" mbm_status mbm_ctx_destroy(mbm_ctx* ctx) {
 
 extern "C" size_t mbm_ctx_bytes_in_use(const mbm_ctx* ctx) { return ctx ? ctx->in_use : 0; }
 
-extern "C" mbm_status mbm_ctx_set_wait_cycles(mbm_ctx* ctx, int64_t cycles) {
+extern "C" mbm_status mbm_ctx_expire_waits(mbm_ctx* ctx, int enable) {
     if (!ctx) return mbm_fail(MBM_EINVAL, "ctx is NULL");
-    if (cycles < 0) return mbm_fail(MBM_EINVAL, "cycles < 0");
     std::lock_guard<std::mutex> lock(ctx->mu);
-    ctx->wait_cycles = cycles;
+    ctx->expire_waits = enable != 0;
     return MBM_OK;
 }
 

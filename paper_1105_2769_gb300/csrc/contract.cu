@@ -77,7 +77,7 @@ constexpr float kLowScale = 1.0f / 2048.0f;
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 2) * 32;
 constexpr int kGroup = 8;  // J tiles walked together: their rows and 19 I tiles stay in L2
-constexpr long long kDrainLimit = 4000000000LL;  // for work in flight after an expired wait
+constexpr long long kWaitLimit = 4000000000LL;
 
 __device__ __forceinline__ float pow2f(int e) {  // 2^e, 0 below the normal range
     return e < -126 ? 0.f : __int_as_float((min(e, 127) + 127) << 23);
@@ -268,7 +268,6 @@ struct ContractSmem {
     unsigned long long full[kStages], empty[kStages];
     unsigned long long acc_full[2], acc_empty[2];
     unsigned long long done;  // the MMAs have ended
-    long long wait_limit;
     unsigned tmem;
     volatile int abort;
 };
@@ -276,12 +275,12 @@ struct ContractSmem {
 // Bounded wait; the first one to give up tells every role to stop.
 __device__ __forceinline__ bool wait_phase(ContractSmem& sm, unsigned long long* bar,
                                            unsigned parity) {
-    if (mbar_test_wait(bar, parity)) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     for (;;) {
-        if (sm.wait_limit > 0 && mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait(bar, parity)) return true;
         if (sm.abort) return false;
-        if (clock64() - t0 > sm.wait_limit) {
+        if (clock64() - t0 > kWaitLimit) {
             sm.abort = 1;
             return false;
         }
@@ -317,8 +316,7 @@ __device__ __forceinline__ void drain(unsigned addr, const float* fj, float2 fi,
 __global__ void __launch_bounds__(kThreads, 1)
 contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __restrict__ TB,
                 const float* __restrict__ fA, const float* __restrict__ fB, int n_pad, int nb,
-                int nkb, int t0, int nt, float* __restrict__ C, int* gate,
-                long long wait_limit) {
+                int nkb, int t0, int nt, float* __restrict__ C, int* gate, int expire) {
     // (a CTA of this launch may set it meanwhile: one answer for all threads)
     if (__syncthreads_or(*gate)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -335,7 +333,6 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
             mbar_init(&sm.acc_empty[a], kEpiWarps);
         }
         mbar_init(&sm.done, 1);
-        sm.wait_limit = wait_limit;
         sm.abort = 0;
         mbar_fence_init();
     }
@@ -382,17 +379,20 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
             }
             // copies in flight land before shared memory is released
             for (unsigned q = it > kStages ? it - kStages : 0; q < it; ++q)
-                mbar_wait_bounded(&sm.full[q % kStages], (q / kStages) & 1, kDrainLimit);
+                mbar_wait_bounded(&sm.full[q % kStages], (q / kStages) & 1, kWaitLimit);
             for (unsigned q = win > kFactorSlots ? win - kFactorSlots : 0; q < win; ++q)
-                mbar_wait_bounded(&sm.factors[q % kFactorSlots], (q / kFactorSlots) & 1, kDrainLimit);
+                mbar_wait_bounded(&sm.factors[q % kFactorSlots], (q / kFactorSlots) & 1, kWaitLimit);
         }
     } else if (warp == kEpiWarps + 1) {
         if (lane == 0) {
             constexpr unsigned idesc = tc_idesc_f16(kBM, kBN);
             unsigned it = 0, win = 0, blk = 0;  // stages, windows and blocks handed over
             bool ok = true;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                for (int kb = 0; kb < nkb; kb += kKbPerWin, ++win) {
+            // (expire, a switch of tests: this role gives up after its first window)
+            const int items = expire ? 0 : n_items, kbs = expire ? kKbPerWin : nkb;
+            int item = blockIdx.x;
+            do {
+                for (int kb = 0; kb < kbs; kb += kKbPerWin, ++win) {
                     const bool first = kb % kKbPerBlk == 0;
                     const bool last = kb % kKbPerBlk == kKbPerBlk - kKbPerWin;
                     if (win && !wait_phase(sm, &sm.acc_empty[0], (win - 1) & 1)) {
@@ -438,11 +438,13 @@ contract_kernel(const unsigned char* __restrict__ TA, const unsigned char* __res
                         tc_commit(smem_u32(&sm.empty[it % kStages]));
                     }
                 }
-            }
+                item += gridDim.x;
+            } while (item < items && ok);
+            if (expire) sm.abort = 1;
             // MMAs in flight end before TMEM and shared memory are released, also those
             // that an expired wait left without a commit
             tc_commit(smem_u32(&sm.done));
-            mbar_wait_bounded(&sm.done, 0, kDrainLimit);
+            mbar_wait_bounded(&sm.done, 0, kWaitLimit);
         }
     } else {
         // rows 32 (warp % 4) + lane of the tile, columns 64 (warp / 4) + 0..63
@@ -817,10 +819,10 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
             const int nt = std::min(p.batch, p.tiles - t0);
             const int grid = std::min(nt * kForms, std::max(1, ctx->num_sms));
             contract_kernel<<<grid, kThreads, sizeof(ContractSmem), s>>>(
-                T, T, f, f, n_pad, p.nb, nkb, t0, nt, C, gate, ctx->wait_cycles);
+                T, T, f, f, n_pad, p.nb, nkb, t0, nt, C, gate, ctx->expire_waits);
             if (weighted)
                 contract_kernel<<<grid, kThreads, sizeof(ContractSmem), s>>>(
-                    Tg, T, fg, f, n_pad, p.nb, nkb, t0, nt, Cg, gate, ctx->wait_cycles);
+                    Tg, T, fg, f, n_pad, p.nb, nkb, t0, nt, Cg, gate, ctx->expire_waits);
             auto pass = [&](auto kernel) {
                 kernel<<<dim3(nt, kBN / kPairCols), 256, 0, s>>>(xh, xl, (int)N, p.nb, t0, near.tau,
                                                                  C, Cg, gs, row_ea, row_eag, ref,

@@ -45,7 +45,7 @@ constexpr int kStages = 2;
 constexpr int kBufs = 4;     // TMEM accumulators of 128 columns
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 2) * 32;
-constexpr long long kDrainLimit = 4000000000LL;  // for work in flight after an expired wait
+constexpr long long kWaitLimit = 4000000000LL;
 
 // Block of S stages: its 64-bit sums hold the weight-0 products, below 2^19 a
 // stage, at 2^base: 2^62 at most.
@@ -184,7 +184,6 @@ struct ContractSmem {
     unsigned long long full[kStages], empty[kStages];
     unsigned long long acc_full[kBufs], acc_empty[kBufs];
     unsigned long long done;  // the MMAs have ended
-    long long wait_limit;
     unsigned tmem;
     volatile int abort;
 };
@@ -192,12 +191,12 @@ struct ContractSmem {
 // Bounded wait; the first one to give up tells every role to stop.
 __device__ __forceinline__ bool wait_phase(ContractSmem& sm, unsigned long long* bar,
                                            unsigned parity) {
-    if (mbar_test_wait(bar, parity)) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     for (;;) {
-        if (sm.wait_limit > 0 && mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait(bar, parity)) return true;
         if (sm.abort) return false;
-        if (clock64() - t0 > sm.wait_limit) {
+        if (clock64() - t0 > kWaitLimit) {
             sm.abort = 1;
             return false;
         }
@@ -250,7 +249,7 @@ __device__ __forceinline__ void read_out(unsigned addr, unsigned long long (&t)[
 template <int Stages>  // stages per block
 __global__ void __launch_bounds__(kThreads, 1)
 contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, int nt,
-                  longlong2* __restrict__ C, int* gate, long long wait_limit) {
+                  longlong2* __restrict__ C, int* gate, int expire) {
     // (a CTA of this launch may set it meanwhile: one answer for all threads)
     if (__syncthreads_or(*gate)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -267,7 +266,6 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
             mbar_init(&sm.acc_empty[a], kEpiWarps);
         }
         mbar_init(&sm.done, 1);
-        sm.wait_limit = wait_limit;
         sm.abort = 0;
         mbar_fence_init();
     }
@@ -301,7 +299,7 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
             }
             // copies in flight land before shared memory is released
             for (unsigned q = it > kStages ? it - kStages : 0; q < it; ++q)
-                mbar_wait_bounded(&sm.full[q % kStages], (q / kStages) & 1, kDrainLimit);
+                mbar_wait_bounded(&sm.full[q % kStages], (q / kStages) & 1, kWaitLimit);
         }
     } else if (warp == kEpiWarps + 1) {
         if (lane == 0) {
@@ -336,13 +334,17 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
                                            idesc, p + k > 0);
                         tc_commit(smem_u32(&sm.acc_full[buf]));
                     }
+                    if (expire) {  // a switch of tests: run out with MMAs under way
+                        sm.abort = 1;
+                        ok = false;
+                    }
                     if (ok) tc_commit(smem_u32(&sm.empty[s]));
                 }
             }
             // MMAs in flight end before TMEM and shared memory are released, also those
             // that an expired wait left without a commit
             tc_commit(smem_u32(&sm.done));
-            mbar_wait_bounded(&sm.done, 0, kDrainLimit);
+            mbar_wait_bounded(&sm.done, 0, kWaitLimit);
         }
     } else {
         // rows 32 (warp % 4) + lane of the tile, columns 32 (warp / 4) + 0..31
@@ -604,7 +606,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     for (int t0 = 0; t0 < tiles; t0 += batch) {
         const int nt = std::min(batch, tiles - t0);
         kernel<<<std::min(nt * kForms, std::max(1, ctx->num_sms)), kThreads, sizeof(ContractSmem),
-                 s>>>(T, nb, nkb, t0, nt, C, gate, ctx->wait_cycles);
+                 s>>>(T, nb, nkb, t0, nt, C, gate, ctx->expire_waits);
         auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
         pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(x4, xh, xl, (int)N, n_pad, n_blk,
                                                   base_shift(stages), t0, near.tau, ea, C, sign,

@@ -49,7 +49,7 @@ struct mbm_ctx {
     size_t scratch_bytes = 0;
     int* d_flags = nullptr;  // device status word (+ padding)
     int* h_flags = nullptr;  // pinned host mirror
-    long long wait_cycles = 4000000000LL;  // bound of the contractions' device waits (about 2 s)
+    int expire_waits = 0;    // test switch: a wait of every contraction runs out
     std::mutex mu;           // one solve at a time per context
     bool timing = false;     // record events around the dominant kernel
     bool timed = false;      // the last solve recorded events
