@@ -102,8 +102,8 @@ exponent_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, in
 __global__ void __launch_bounds__(kRows)
 digit_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
              const float4* __restrict__ xl, int N, const float* __restrict__ tau, int n_pad, int nb,
-             int nkb, int stages, const int* __restrict__ ea, unsigned char* __restrict__ T,
-             const int* __restrict__ gate) {
+             int kb0, int nkb, int stages, const int* __restrict__ ea,
+             unsigned char* __restrict__ T, const int* __restrict__ gate) {
     if (*gate) return;
     __shared__ double coef[kForms][5];
     const int rb = blockIdx.x, kb = blockIdx.y, k8 = blockIdx.z;
@@ -116,12 +116,12 @@ digit_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
     const float ti = i < N ? tau[i] : 0.f;
     const double4_32a xi = i < N ? x4[i] : make_double4_32a(0, 0, 0, 0);
     // terms in units of 2^-48 of |2^ea l| < 2^7
-    const double a = i < N ? pow2d(ea[(size_t)(kb / stages) * n_pad + i] + 48) : 0.0;
+    const double a = i < N ? pow2d(ea[(size_t)((kb0 + kb) / stages) * n_pad + i] + 48) : 0.0;
     const size_t off = (size_t)(row >> 3) * 512 + k8 * 128 + (row & 7) * 16;
     double v[8][5];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-        const int k = kb * kBK + k8 * 8 + q;
+        const int k = (kb0 + kb) * kBK + k8 * 8 + q;
 #pragma unroll
         for (int m = 0; m < 5; ++m) v[q][m] = 0.0;
         if (i < N && k < N && k != i) {
@@ -402,8 +402,8 @@ contract64_kernel(const unsigned char* __restrict__ T, int nb, int nkb, int t0, 
 
 // ---------------------------------------------------------------------------
 // Pair pass in FP64: 16 CTAs per tile, a thread per row and 4 columns, two at a
-// time (ten tiles at N = 512 need that many to fill the chip): C^r = sum over blocks of the scaled 64-bit sums, G = sum_r C^r A_r, then
-// rho e.G e or (rho / r)(2 G e - 5 (e.G e) e).
+// time (ten tiles at N = 512 need that many to fill the chip): C^r = sum over the
+// slab's blocks of the scaled 64-bit sums, G = sum_r C^r A_r, then rho e.G e or (rho / r)(2 G e - 5 (e.G e) e).
 // ---------------------------------------------------------------------------
 constexpr int kPairCols = 4;  // columns per thread
 
@@ -533,33 +533,62 @@ size_t up256(size_t b) { return mbm_align_up(b, 256); }
 // r^2 of the closest pair that the two FP32 parts of a point resolve, in the frame.
 constexpr float kMinDist2 = 3.637979e-12f;  // 2^-38
 
-// Largest N: its digit table (140 N^2 bytes) has to fit the device.
+// Largest N that was measured (7 s a solve).
 constexpr int64_t kMaxN64 = 24576;
+
+// Scratch layout of one solve. The digit table takes 140 bytes per pair of
+// particles (58 GB at N = 20 000), so the columns k go in slabs whose table stays
+// below kTableMost: C^r is a sum over k and so is all that follows. A slab more is one
+// more pair pass (46 ms of FP64 at N = 20 000, against 0.6 s of its contraction).
+constexpr size_t kTableMost = (size_t)6 << 30, kSumsMost = (size_t)3 << 30;
+
+struct Plan64 {
+    int stages = 8, cols = 0;               // of a block
+    int nb = 0, n_blk = 0, n_pad = 0;       // row blocks; column blocks in all
+    int slab = 0, tiles = 0, batch = 0;     // column blocks per slab; tiles per pair pass
+    size_t table = 0, per_tile = 0, total = 0;
+};
+
+static Plan64 plan64(int64_t N, size_t cap) {
+    Plan64 p;
+    // blocks of 512 columns halve the 64-bit sums to convert; 256 waste less at small N
+    p.stages = N > 2048 ? 16 : 8;
+    p.cols = p.stages * kBK;
+    p.nb = (int)((N + kRows - 1) / kRows);
+    p.n_blk = (int)((N + p.cols - 1) / p.cols);
+    p.n_pad = (int)mbm_align_up((size_t)p.nb * kRows, 256);
+    p.tiles = p.nb * (p.nb + 1) / 2;
+    const size_t blk_table = (size_t)kForms * p.nb * p.stages * kStageBytes;
+    const size_t blk_sums = (size_t)kForms * kRows * kRows * 8;
+    const size_t fixed = 256 + up256((size_t)N * 16) * 2 + up256((size_t)N * 32) +
+                         mbm_near_bytes(N) + up256((size_t)p.n_pad * 4 * p.n_blk) + 4096;
+    if (cap < fixed + blk_table + blk_sums) return Plan64{};
+    const size_t room = cap - fixed;
+    const size_t most = std::min<size_t>(
+        p.n_blk, std::min(std::max<size_t>(1, kTableMost / blk_table), room / (blk_table + blk_sums)));
+    const int slabs = (int)((p.n_blk + most - 1) / most);
+    p.slab = (p.n_blk + slabs - 1) / slabs;  // even slabs
+    p.table = blk_table * p.slab;
+    p.per_tile = blk_sums * p.slab;
+    const size_t sums = std::min(kSumsMost, room - p.table);
+    p.batch = (int)std::max<size_t>(1, std::min<size_t>(p.tiles, sums / p.per_tile));
+    p.total = fixed + p.table + p.per_tile * p.batch;
+    return p;
+}
 
 mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, double sign,
                           double* out, cudaStream_t s, bool* done, MbmGate64* gate_out) {
     *done = false;
     if (N > kMaxN64) return MBM_OK;
-    // blocks of 512 columns halve the 64-bit sums to convert; 256 waste less at small N
-    const int stages = N > 2048 ? 16 : 8;
-    const int cols = stages * kBK;
-    const int nb = (int)((N + kRows - 1) / kRows);
-    const int n_blk = (int)((N + cols - 1) / cols), nkb = n_blk * stages;
-    const int n_pad = (int)mbm_align_up((size_t)nb * kRows, 256);
-    const int tiles = nb * (nb + 1) / 2;
-    const size_t table = (size_t)kForms * nb * nkb * kStageBytes;
-    const size_t per_tile = (size_t)kForms * n_blk * kRows * kRows * 8;
-    const size_t fixed = 256 + up256((size_t)N * 16) * 2 + up256((size_t)N * 32) +
-                         mbm_near_bytes(N) + up256((size_t)n_pad * 4 * n_blk) + 4096;
     size_t cap = (size_t)1 << 60;
     if (ctx->budget) {
         const size_t others = ctx->in_use - ctx->scratch_bytes;
         cap = ctx->budget > others ? ctx->budget - others : 0;
     }
-    if (cap < fixed + table + per_tile) return MBM_OK;
-    const size_t most = std::min<size_t>((size_t)3 << 30, cap - fixed - table);
-    const int batch = (int)std::max<size_t>(1, std::min<size_t>(tiles, most / per_tile));
-    const mbm_status rs = mbm_scratch_reserve(ctx, fixed + up256(table) + per_tile * batch);
+    const Plan64 p = plan64(N, cap);
+    if (!p.slab) return MBM_OK;
+    const int nb = p.nb, n_pad = p.n_pad;
+    const mbm_status rs = mbm_scratch_reserve(ctx, p.total);
     if (rs != MBM_OK) {
         if (rs != MBM_EBUDGET && rs != MBM_ENOMEM) return rs;
         cudaGetLastError();  // no room: the FP64 sweep needs less
@@ -578,9 +607,9 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     auto* xh = reinterpret_cast<float4*>(take((size_t)N * 16));
     auto* xl = reinterpret_cast<float4*>(take((size_t)N * 16));
     char* near_mem = take(mbm_near_bytes(N));
-    int* ea = reinterpret_cast<int*>(take((size_t)n_pad * 4 * n_blk));
-    auto* T = reinterpret_cast<unsigned char*>(take(table));
-    auto* C = reinterpret_cast<longlong2*>(take(per_tile * batch));
+    int* ea = reinterpret_cast<int*>(take((size_t)n_pad * 4 * p.n_blk));
+    auto* T = reinterpret_cast<unsigned char*>(take(p.table));
+    auto* C = reinterpret_cast<longlong2*>(take(p.per_tile * p.batch));
 
     const bool grad = what != MBM_CONTRACT_PHI;
     MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
@@ -588,7 +617,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     const MbmOut res{out, N * (grad ? 3 : 1), grad ? 10 : 9};
     MBM_CUDA_TRY(launch_frame(X, N, nullptr, frame, xh, xl, x4, nullptr, res, gate, ctx->d_flags,
                               s));
-    auto kernel = stages == 8 ? contract64_kernel<8> : contract64_kernel<16>;
+    auto kernel = p.stages == 8 ? contract64_kernel<8> : contract64_kernel<16>;
     MBM_CUDA_TRY(cudaFuncSetAttribute((const void*)kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(ContractSmem)));
@@ -598,20 +627,24 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     near.min_d2 = kMinDist2;
     near.excess = counter + 1;
     MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
-    exponent_kernel<<<dim3(n_pad / 256, n_blk), 256, 0, s>>>(xh, xl, (int)N, cols, near.tau, n_pad,
-                                                            ea, gate);
-    digit_kernel<<<dim3(nb, nkb, kBK / 8), kRows, 0, s>>>(x4, xh, xl, (int)N, near.tau, n_pad, nb,
-                                                          nkb, stages, ea, T, gate);
-    MBM_CUDA_TRY(cudaGetLastError());
-    for (int t0 = 0; t0 < tiles; t0 += batch) {
-        const int nt = std::min(batch, tiles - t0);
-        kernel<<<std::min(nt * kForms, std::max(1, ctx->num_sms)), kThreads, sizeof(ContractSmem),
-                 s>>>(T, nb, nkb, t0, nt, C, gate, ctx->expire_waits);
-        auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
-        pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(x4, xh, xl, (int)N, n_pad, n_blk,
-                                                  base_shift(stages), t0, near.tau, ea, C, sign,
-                                                  out, gate);
+    exponent_kernel<<<dim3(n_pad / 256, p.n_blk), 256, 0, s>>>(xh, xl, (int)N, p.cols, near.tau,
+                                                              n_pad, ea, gate);
+    for (int b0 = 0; b0 < p.n_blk; b0 += p.slab) {
+        const int n_blk = std::min(p.slab, p.n_blk - b0), nkb = n_blk * p.stages;
+        digit_kernel<<<dim3(nb, nkb, kBK / 8), kRows, 0, s>>>(x4, xh, xl, (int)N, near.tau, n_pad,
+                                                              nb, b0 * p.stages, nkb, p.stages, ea,
+                                                              T, gate);
         MBM_CUDA_TRY(cudaGetLastError());
+        for (int t0 = 0; t0 < p.tiles; t0 += p.batch) {
+            const int nt = std::min(p.batch, p.tiles - t0);
+            kernel<<<std::min(nt * kForms, std::max(1, ctx->num_sms)), kThreads,
+                     sizeof(ContractSmem), s>>>(T, nb, nkb, t0, nt, C, gate, ctx->expire_waits);
+            auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
+            pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(
+                x4, xh, xl, (int)N, n_pad, n_blk, base_shift(p.stages), t0, near.tau,
+                ea + (size_t)b0 * n_pad, C, sign, out, gate);
+            MBM_CUDA_TRY(cudaGetLastError());
+        }
     }
     MBM_CUDA_TRY(launch_near_triples(xh, xl, x4, N, near, nullptr,
                                      grad ? MBM_NEAR_GRAD : MBM_NEAR_PHI, sign, out, ctx->num_sms,
