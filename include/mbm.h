@@ -356,7 +356,8 @@ mbm_status mbm_submit(mbm_server* server, const mbm_request* req, uint64_t* tick
  * for an unknown or already collected ticket. */
 mbm_status mbm_poll(mbm_server* server, uint64_t ticket, mbm_result* res, int64_t timeout_us);
 
-/* Counters: requests admitted, waiting, rejected, completed; bytes held. */
+/* Counters: requests admitted, waiting, rejected, completed; bytes held (running
+ * requests' estimates, resident systems, and the buffers that idle slots keep). */
 mbm_status mbm_server_stats(mbm_server* server, int64_t* admitted, int64_t* pending,
                             int64_t* rejected, int64_t* completed, size_t* reserved);
 

@@ -85,6 +85,24 @@ mbm_status mbm_scratch_reserve(mbm_ctx* ctx, size_t bytes) {
     return MBM_OK;
 }
 
+void mbm_ctx_set_room(mbm_ctx* ctx, size_t bytes) {
+    std::lock_guard<std::mutex> lock(ctx->mu);
+    ctx->budget = bytes ? bytes + (ctx->in_use - ctx->scratch_bytes) : 0;
+}
+
+void mbm_scratch_release(mbm_ctx* ctx) {
+    std::lock_guard<std::mutex> lock(ctx->mu);
+    if (ctx->scratch) cudaFree(ctx->scratch);  // (waits for work in flight)
+    ctx->scratch = nullptr;
+    mbm_budget_release(ctx, ctx->scratch_bytes);
+    ctx->scratch_bytes = 0;
+}
+
+size_t mbm_scratch_held(mbm_ctx* ctx) {
+    std::lock_guard<std::mutex> lock(ctx->mu);
+    return ctx->scratch_bytes;
+}
+
 mbm_status mbm_check_flags(mbm_ctx* ctx, cudaStream_t stream) {
     MBM_CUDA_TRY(cudaMemcpyAsync(ctx->h_flags, ctx->d_flags, sizeof(int), cudaMemcpyDeviceToHost,
                                  stream));

@@ -42,5 +42,7 @@ struct MbmGate64 {
 // N = 100 took 3 ms in gather form and take 0.5.)
 constexpr int64_t kContract64MinPhi = 192;
 constexpr int64_t kContract64MinForces = 96;
+// Scratch of a potential or force solve of N particles (0: not a contraction).
+size_t mbm_contract64_bytes(int64_t N, bool forces);
 mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, double sign,
                           double* out, cudaStream_t s, bool* done, MbmGate64* gate);

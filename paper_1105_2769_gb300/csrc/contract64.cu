@@ -576,6 +576,11 @@ static Plan64 plan64(int64_t N, size_t cap) {
     return p;
 }
 
+size_t mbm_contract64_bytes(int64_t N, bool forces) {
+    if (N < (forces ? kContract64MinForces : kContract64MinPhi) || N > kMaxN64) return 0;
+    return plan64(N, (size_t)1 << 60).total;
+}
+
 mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, double sign,
                           double* out, cudaStream_t s, bool* done, MbmGate64* gate_out) {
     *done = false;

@@ -65,6 +65,11 @@ void mbm_time_set_ms(mbm_ctx* ctx, double ms);
 
 // Make sure the arena holds at least `bytes`; may reallocate (synchronous).
 mbm_status mbm_scratch_reserve(mbm_ctx* ctx, size_t bytes);
+// Bound what the next solves may take as scratch (0 = the device): the plans shrink to
+// it or leave the solve to a path that needs less. / Free the arena. / Its size.
+void mbm_ctx_set_room(mbm_ctx* ctx, size_t bytes);
+void mbm_scratch_release(mbm_ctx* ctx);
+size_t mbm_scratch_held(mbm_ctx* ctx);
 // Charge/uncharge library-owned bytes against the budget.
 mbm_status mbm_budget_charge(mbm_ctx* ctx, size_t bytes);
 void mbm_budget_release(mbm_ctx* ctx, size_t bytes);

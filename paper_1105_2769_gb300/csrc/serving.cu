@@ -46,6 +46,7 @@ struct Job {
     mbm_request req{};
     mbm_config cfg{};
     size_t est = 0;
+    size_t room = 0;  // scratch that the solve may take (0 = not bounded)
     clk::time_point submitted;
 };
 
@@ -73,21 +74,36 @@ struct Worker {
     size_t capX = 0, capOut = 0;
     unsigned long long* d_stamp = nullptr;  // device clock at a request's start and end
     unsigned long long* h_stamp = nullptr;  // pinned host copy
+    // Buffers outlive a request and stay counted in `reserved` (with a budget) while the
+    // slot is idle; `trim` asks the slot to give them back.
+    size_t held = 0;     // bytes counted
+    bool busy = false, trim = false;
 };
 
-// The contraction's scratch counts where the budget can hold it; a smaller
-// budget admits the request as before and the solve finds its own room.
-size_t estimate_bytes(const mbm_request& r, const mbm_config& c, size_t budget) {
+// Device footprint of a request, and the scratch its solve may take within it. An
+// exhaustive solve counts what its fastest path takes (the contraction's tables, or the
+// pair table) where the budget can hold that, and else the triple sweep's packed points,
+// and its context is held to it. One exception, as old as the server: an FP32 potential
+// that the budget cannot hold in full is admitted at its packed points and not bounded,
+// so that its result is the one it has alone.
+void estimate(Job& job, size_t budget) {
+    const mbm_request& r = job.req;
     const size_t N = (size_t)r.N;
-    const size_t io = N * 24 + N * (r.kind == MBM_REQ_FORCES ? 24 : 8);
+    const bool forces = r.kind == MBM_REQ_FORCES;
+    const size_t io = N * 24 + N * (forces ? 24 : 8);
     const int base = r.mode & 0xff;
-    if (base != MBM_TREE) {
-        const size_t least = io + N * 32 + 4096;
-        const size_t more =
-            base == MBM_EXH_FP32 ? mbm_contract_bytes(r.N, r.kind == MBM_REQ_FORCES) : 0;
-        return budget && least + more > budget ? least : least + more;
+    job.room = 0;
+    if (base == MBM_TREE) {
+        job.est = io + mbm_tree_solve_bytes(r.N, job.cfg, forces) + (1 << 20);
+        return;
     }
-    return io + mbm_tree_solve_bytes(r.N, c, r.kind == MBM_REQ_FORCES) + (1 << 20);
+    const size_t least = N * 32 + 4096;
+    size_t more = base == MBM_EXH_FP32 ? mbm_contract_bytes(r.N, forces)
+                                       : mbm_contract64_bytes(r.N, forces);
+    if (base == MBM_EXH_FP32 && !forces && !more) more = pair_table_bytes(r.N);
+    const bool whole = !budget || io + least + more <= budget;
+    job.room = whole || forces || base != MBM_EXH_FP32 ? least + (whole ? more : 0) : 0;
+    job.est = io + least + (whole ? more : 0);
 }
 
 }  // namespace
@@ -95,7 +111,7 @@ size_t estimate_bytes(const mbm_request& r, const mbm_config& c, size_t budget) 
 struct mbm_server {
     int device = 0;
     size_t budget = 0;
-    size_t reserved = 0;        // admitted estimates + resident systems
+    size_t reserved = 0;        // admitted estimates, resident systems, idle slots' buffers
     std::vector<Worker> workers;
     std::deque<Job> pending;
     std::unordered_map<uint64_t, Done> done;
@@ -117,9 +133,9 @@ void free_resident(Resident& r) {
     r = Resident{};
 }
 
-// Take resident systems nobody uses off the table until `need` more bytes
-// fit (LRU); the caller holds the lock, and they are freed after it is
-// released (s->evicted).
+// Make room for `need` more bytes: take resident systems nobody uses off the table
+// (LRU), then ask idle slots for their buffers. The caller holds the lock; systems are
+// freed after it is released (s->evicted), slots wake up and free their own.
 void evict_for(mbm_server* s, size_t need) {
     while (s->budget && s->reserved + need > s->budget) {
         auto victim = s->resident.end();
@@ -127,33 +143,78 @@ void evict_for(mbm_server* s, size_t need) {
             if (it->second.users == 0 &&
                 (victim == s->resident.end() || it->second.last_use < victim->second.last_use))
                 victim = it;
-        if (victim == s->resident.end()) return;
+        if (victim == s->resident.end()) break;
         s->reserved -= victim->second.bytes;
         s->evicted.push_back(victim->second);
         s->resident.erase(victim);
     }
+    if (!s->budget || s->reserved + need <= s->budget) return;
+    bool any = false;
+    for (auto& w : s->workers)
+        if (!w.busy && w.held && !w.trim) w.trim = any = true;
+    if (any) s->cv_work.notify_all();
+}
+
+// Bytes that a request adds to what the slot holds already.
+size_t added(const Worker& w, size_t est) { return est > w.held ? est - w.held : 0; }
+
+void start_job(mbm_server* s, Worker& w, const Job& job) {
+    s->reserved += added(w, job.est);
+    w.held = std::max(w.held, job.est);
+    w.busy = true;
 }
 
 // Pick the next job this worker may start (caller holds the lock).
-bool take_job(mbm_server* s, Job& out) {
-    if (s->pending.empty()) return false;
+bool take_job(mbm_server* s, Worker& w, Job& out) {
+    if (s->pending.empty() || w.trim) return false;
     const size_t room_head = s->pending.front().est;
-    evict_for(s, room_head);
-    if (!s->budget || s->reserved + room_head <= s->budget) {
+    evict_for(s, added(w, room_head));
+    if (w.trim) return false;  // its own buffers first
+    if (!s->budget || s->reserved + added(w, room_head) <= s->budget) {
         out = s->pending.front();
         s->pending.pop_front();
-        s->reserved += out.est;
+        start_job(s, w, out);
         return true;
     }
     for (auto it = s->pending.begin() + 1; it != s->pending.end(); ++it) {
         if (s->reserved + room_head + it->est <= s->budget) {
             out = *it;
             s->pending.erase(it);
-            s->reserved += out.est;
+            start_job(s, w, out);
             return true;
         }
     }
     return false;
+}
+
+void drop_buffers(Worker& w) {
+    if (w.dX) cudaFree(w.dX);
+    if (w.dOut) cudaFree(w.dOut);
+    w.dX = w.dOut = nullptr;
+    w.capX = w.capOut = 0;
+    mbm_scratch_release(w.ctx);
+}
+
+// After a request: what the slot holds from here on is counted, and given back if the
+// budget has no room for it.
+void end_job(mbm_server* s, Worker& w) {
+    const size_t now = mbm_scratch_held(w.ctx) + w.capX + w.capOut;
+    bool keep = true;
+    {
+        std::unique_lock<std::mutex> lock(s->mu);
+        keep = !s->budget || s->reserved - w.held + now <= s->budget;
+        if (keep) {
+            s->reserved = s->reserved - w.held + now;
+            w.held = now;
+            w.busy = false;
+        }
+    }
+    if (keep) return;
+    drop_buffers(w);
+    std::unique_lock<std::mutex> lock(s->mu);
+    s->reserved -= w.held;
+    w.held = 0;
+    w.busy = false;
 }
 
 mbm_status grow(double** p, size_t* cap, size_t bytes) {
@@ -198,6 +259,7 @@ mbm_status run_job(mbm_server* s, Worker& w, const Job& job, int slot, mbm_resul
     const bool tree_mode = (r.mode & 0xff) == MBM_TREE;
     res.slot = slot;
     w.h_stamp[0] = w.h_stamp[1] = 0;
+    mbm_ctx_set_room(w.ctx, job.room);
     Resident* res_entry = nullptr;
     if (r.system_id) {
         std::unique_lock<std::mutex> lock(s->mu);
@@ -288,15 +350,26 @@ void worker_main(mbm_server* s, int slot) {
     cudaSetDevice(s->device);
     for (;;) {
         Job job;
+        bool trim = false;
         std::vector<Resident> dead;
         {
             std::unique_lock<std::mutex> lock(s->mu);
-            s->cv_work.wait(lock,
-                            [&] { return s->stop || !s->evicted.empty() || take_job(s, job); });
+            s->cv_work.wait(lock, [&] {
+                return s->stop || !s->evicted.empty() || take_job(s, w, job) || w.trim;
+            });
             dead.swap(s->evicted);
+            trim = w.trim && !w.busy;
             if (job.ticket != 0) s->n_admitted++;
         }
         for (auto& d : dead) free_resident(d);  // outside the lock
+        if (trim) {
+            drop_buffers(w);
+            std::unique_lock<std::mutex> lock(s->mu);
+            s->reserved -= w.held;
+            w.held = 0;
+            w.trim = false;
+            s->cv_work.notify_all();
+        }
         if (job.ticket == 0) {
             if (s->stop) return;
             continue;
@@ -309,9 +382,9 @@ void worker_main(mbm_server* s, int slot) {
         res.compute_ms = ms_between(t0, t1);
         res.latency_ms = ms_between(job.submitted, t1);
         res.bytes_reserved = (int64_t)job.est;
+        end_job(s, w);
         {
             std::unique_lock<std::mutex> lock(s->mu);
-            s->reserved -= job.est;
             Done& d = s->done[job.ticket];
             d.res = res;
             d.ready = true;
@@ -396,7 +469,7 @@ extern "C" mbm_status mbm_submit(mbm_server* s, const mbm_request* req, uint64_t
     if (req->cfg) job.cfg = *req->cfg;
     else mbm_config_default(&job.cfg);
     job.req.cfg = nullptr;
-    job.est = estimate_bytes(job.req, job.cfg, s->budget);
+    estimate(job, s->budget);
     job.submitted = clk::now();
     std::unique_lock<std::mutex> lock(s->mu);
     if (s->budget && job.est > s->budget) {
