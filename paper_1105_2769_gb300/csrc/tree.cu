@@ -1758,10 +1758,14 @@ seed_scale_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl, 
 // warp's shared table; a's terms to 8 columns c are held in registers and
 // its term to row b is formed once per row, so the inner loop is the gradient
 // alone: 29 packed operations per two columns, the e_ab and e_ac terms summed
-// per row and column before the vectors, FP64 sums per leaf and 8 columns (per
+// per row and column before the vectors, FP64 sums per 4 rows and 8 columns (per
 // row they kept the FP64 pipe half busy). Masked pairs have zero terms and contribute exactly 0.
 constexpr int kForceWarps = 4;
 constexpr int kForceCols = 8;
+// Rows whose sums are FP32 (errors of forces at eps = 0 against 64 bits, ten kinds of
+// sets: 32 rows 2.5 % above those of one row, 8 rows 1.1 %, 4 rows 0.2 %; 39.6, 39.9 and
+// 40.4 ms at N = 3 000).
+constexpr int kForceRows = 4;
 // Largest seed level of the force criterion's A^l: the seed pass costs the
 // seed node's size squared per particle and, for gradients, outweighs the
 // base cases it saves beyond 2 048-point seed nodes (N = 65 536, eps = 1e-2:
@@ -1837,56 +1841,62 @@ base_forces_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
                     vz[q] = make_float2(p0.ez, p1.ez);
                     rv[q] = make_float2(p0.rho, p1.rho);
                     iv[q] = make_float2(p0.y, p1.y);
-                    a2[q] = make_float2(0.f, 0.f);
                 }
                 // -grad = sum c1 e_ab + sum c2 e_ac - sum c3 e_bc: the first summed per
-                // row, the second per column, before the vectors come in
-                float g1x = 0.f, g1y = 0.f, g1z = 0.f;
-                float2 g3x = make_float2(0.f, 0.f), g3y = g3x, g3z = g3x;
+                // row, the second per column, before the vectors come in; kForceRows
+                // rows at a time, then on in FP64
 #pragma unroll 1
-                for (int bi = 0; bi < n[o1]; ++bi) {
-                    const PairFY ab = pair_sample_y_or_zero(ah, al, sm.ph[o1][bi], sm.pl[o1][bi],
-                                                            act && !(ex1 && bi == lane));
-                    const float2 ux = f2_splat(ab.ex), uy = f2_splat(ab.ey), uz = f2_splat(ab.ez);
-                    const float2 r3 = f2_splat(3.0f * ab.rho), iu = f2_splat(ab.y);
-                    float2 a1 = make_float2(0.f, 0.f);
-                    const mbm_tile::TabPair* tr = sm.tab[bi] + ((cb - h0) >> 1);
+                for (int r0 = 0; r0 < n[o1]; r0 += kForceRows) {
+                    const int r1 = min(n[o1], r0 + kForceRows);
+                    float g1x = 0.f, g1y = 0.f, g1z = 0.f;
+                    float2 g3x = make_float2(0.f, 0.f), g3y = g3x, g3z = g3x;
+#pragma unroll
+                    for (int q = 0; q < kP; ++q) a2[q] = make_float2(0.f, 0.f);
+#pragma unroll 1
+                    for (int bi = r0; bi < r1; ++bi) {
+                        const PairFY ab = pair_sample_y_or_zero(ah, al, sm.ph[o1][bi], sm.pl[o1][bi],
+                                                                act && !(ex1 && bi == lane));
+                        const float2 ux = f2_splat(ab.ex), uy = f2_splat(ab.ey), uz = f2_splat(ab.ez);
+                        const float2 r3 = f2_splat(3.0f * ab.rho), iu = f2_splat(ab.y);
+                        float2 a1 = make_float2(0.f, 0.f);
+                        const mbm_tile::TabPair* tr = sm.tab[bi] + ((cb - h0) >> 1);
+#pragma unroll
+                        for (int q = 0; q < kP; ++q) {
+                            const float4 t0 = tr[q].xy, t1 = tr[q].zr;
+                            const float2 wx = make_float2(t0.x, t0.y), wy = make_float2(t0.z, t0.w);
+                            const float2 wz = make_float2(t1.x, t1.y), rw = make_float2(t1.z, t1.w);
+                            const float2 p1 = f2_fma(uz, vz[q], f2_fma(uy, vy[q], f2_mul(ux, vx[q])));
+                            const float2 p2 = f2_fma(uz, wz, f2_fma(uy, wy, f2_mul(ux, wx)));
+                            const float2 p3 = f2_fma(vz[q], wz, f2_fma(vy[q], wy, f2_mul(vx[q], wx)));
+                            const float2 p12 = f2_mul(p1, p2), p13 = f2_mul(p1, p3);
+                            const float2 p23 = f2_mul(p2, p3);
+                            const float2 qf = f2_fma(f2_splat(5.f), f2_mul(p12, p3), f2_splat(-1.f));
+                            const float2 R3 = f2_mul(f2_mul(r3, rv[q]), rw);
+                            const float2 su = f2_mul(R3, iu), sv = f2_mul(R3, iv[q]);
+                            const float2 np23 = f2_mul(p23, f2_splat(-1.f));
+                            a1 = f2_add(a1, f2_fma(su, qf, f2_mul(sv, np23)));
+                            a2[q] = f2_add(a2[q], f2_fma(sv, qf, f2_mul(su, np23)));
+                            const float2 c3 = f2_fma(su, p13, f2_mul(sv, p12));
+                            g3x = f2_fma(c3, wx, g3x);
+                            g3y = f2_fma(c3, wy, g3y);
+                            g3z = f2_fma(c3, wz, g3z);
+                        }
+                        const float c1 = a1.x + a1.y;
+                        g1x = fmaf(c1, ab.ex, g1x);
+                        g1y = fmaf(c1, ab.ey, g1y);
+                        g1z = fmaf(c1, ab.ez, g1z);
+                    }
+                    float2 g2x = make_float2(0.f, 0.f), g2y = g2x, g2z = g2x;
 #pragma unroll
                     for (int q = 0; q < kP; ++q) {
-                        const float4 t0 = tr[q].xy, t1 = tr[q].zr;
-                        const float2 wx = make_float2(t0.x, t0.y), wy = make_float2(t0.z, t0.w);
-                        const float2 wz = make_float2(t1.x, t1.y), rw = make_float2(t1.z, t1.w);
-                        const float2 p1 = f2_fma(uz, vz[q], f2_fma(uy, vy[q], f2_mul(ux, vx[q])));
-                        const float2 p2 = f2_fma(uz, wz, f2_fma(uy, wy, f2_mul(ux, wx)));
-                        const float2 p3 = f2_fma(vz[q], wz, f2_fma(vy[q], wy, f2_mul(vx[q], wx)));
-                        const float2 p12 = f2_mul(p1, p2), p13 = f2_mul(p1, p3);
-                        const float2 p23 = f2_mul(p2, p3);
-                        const float2 qf = f2_fma(f2_splat(5.f), f2_mul(p12, p3), f2_splat(-1.f));
-                        const float2 R3 = f2_mul(f2_mul(r3, rv[q]), rw);
-                        const float2 su = f2_mul(R3, iu), sv = f2_mul(R3, iv[q]);
-                        const float2 np23 = f2_mul(p23, f2_splat(-1.f));
-                        a1 = f2_add(a1, f2_fma(su, qf, f2_mul(sv, np23)));
-                        a2[q] = f2_add(a2[q], f2_fma(sv, qf, f2_mul(su, np23)));
-                        const float2 c3 = f2_fma(su, p13, f2_mul(sv, p12));
-                        g3x = f2_fma(c3, wx, g3x);
-                        g3y = f2_fma(c3, wy, g3y);
-                        g3z = f2_fma(c3, wz, g3z);
+                        g2x = f2_fma(a2[q], vx[q], g2x);
+                        g2y = f2_fma(a2[q], vy[q], g2y);
+                        g2z = f2_fma(a2[q], vz[q], g2z);
                     }
-                    const float c1 = a1.x + a1.y;
-                    g1x = fmaf(c1, ab.ex, g1x);
-                    g1y = fmaf(c1, ab.ey, g1y);
-                    g1z = fmaf(c1, ab.ez, g1z);
+                    gx += (double)((g3x.x + g3x.y) - g1x - (g2x.x + g2x.y));
+                    gy += (double)((g3y.x + g3y.y) - g1y - (g2y.x + g2y.y));
+                    gz += (double)((g3z.x + g3z.y) - g1z - (g2z.x + g2z.y));
                 }
-                float2 g2x = make_float2(0.f, 0.f), g2y = g2x, g2z = g2x;
-#pragma unroll
-                for (int q = 0; q < kP; ++q) {
-                    g2x = f2_fma(a2[q], vx[q], g2x);
-                    g2y = f2_fma(a2[q], vy[q], g2y);
-                    g2z = f2_fma(a2[q], vz[q], g2z);
-                }
-                gx += (double)((g3x.x + g3x.y) - g1x - (g2x.x + g2x.y));
-                gy += (double)((g3y.x + g3y.y) - g1y - (g2y.x + g2y.y));
-                gz += (double)((g3z.x + g3z.y) - g1z - (g2z.x + g2z.y));
             }
         }
         if (act) {
