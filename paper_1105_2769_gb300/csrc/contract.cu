@@ -836,7 +836,7 @@ mbm_status mbm_contract(mbm_ctx* ctx, const double* X, int64_t N, const double* 
     }
     MBM_CUDA_TRY(launch_near_triples(xh, xl, nullptr, N, near, gs,
                                      what == MBM_CONTRACT_PHI ? MBM_NEAR_PHI : MBM_NEAR_GRAD, sign,
-                                     out, ctx->num_sms, gate, s));
+                                     out, nullptr, ctx->num_sms, gate, s));
     MBM_CUDA_TRY(launch_unframe(X, N, frame, xh, xl, nullptr, res, gate, s));
     gate_out->gate = gate;
     gate_out->counter = counter;

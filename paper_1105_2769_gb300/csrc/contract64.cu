@@ -413,7 +413,7 @@ pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
               const float4* __restrict__ xl, int N, int n_pad, int n_blk, int shift, int t0,
               const float* __restrict__ tau, const int* __restrict__ ea,
               const longlong2* __restrict__ C, double sign, double* __restrict__ out,
-              const int* __restrict__ gate) {
+              double* __restrict__ lo, const int* __restrict__ gate) {
     if (*gate) return;
     constexpr int kVals = Grad ? 3 : 1;
     __shared__ double coef[kForms][5];
@@ -517,11 +517,11 @@ pair64_kernel(const double4_32a* __restrict__ x4, const float4* __restrict__ xh,
         for (int o = 16; o >= 4; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane < 4 && j < N && t != 0.0) {
             if constexpr (Grad) atomicAdd(&out[3 * (size_t)j + d], sign * t);
-            else atomicAdd(&out[j], t);
+            else atomic_add_carried(&out[j], &lo[j], t);
         }
         if (iv && sum[d] != 0.0) {
             if constexpr (Grad) atomicAdd(&out[3 * (size_t)i + d], -sign * sum[d]);
-            else atomicAdd(&out[i], sum[d]);
+            else atomic_add_carried(&out[i], &lo[i], sum[d]);
         }
     }
 }
@@ -561,7 +561,8 @@ static Plan64 plan64(int64_t N, size_t cap) {
     const size_t blk_table = (size_t)kForms * p.nb * p.stages * kStageBytes;
     const size_t blk_sums = (size_t)kForms * kRows * kRows * 8;
     const size_t fixed = 256 + up256((size_t)N * 16) * 2 + up256((size_t)N * 32) +
-                         mbm_near_bytes(N) + up256((size_t)p.n_pad * 4 * p.n_blk) + 4096;
+                         up256((size_t)N * 8) + mbm_near_bytes(N) +
+                         up256((size_t)p.n_pad * 4 * p.n_blk) + 4096;
     if (cap < fixed + blk_table + blk_sums) return Plan64{};
     const size_t room = cap - fixed;
     const size_t most = std::min<size_t>(
@@ -611,6 +612,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     auto* x4 = reinterpret_cast<double4_32a*>(take((size_t)N * 32));
     auto* xh = reinterpret_cast<float4*>(take((size_t)N * 16));
     auto* xl = reinterpret_cast<float4*>(take((size_t)N * 16));
+    auto* lo = reinterpret_cast<double*>(take((size_t)N * 8));
     char* near_mem = take(mbm_near_bytes(N));
     int* ea = reinterpret_cast<int*>(take((size_t)n_pad * 4 * p.n_blk));
     auto* T = reinterpret_cast<unsigned char*>(take(p.table));
@@ -619,7 +621,8 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     const bool grad = what != MBM_CONTRACT_PHI;
     MBM_CUDA_TRY(cudaMemsetAsync(ctx->d_flags, 0, sizeof(int), s));
     MBM_CUDA_TRY(cudaMemsetAsync(gate, 0, 256, s));
-    const MbmOut res{out, N * (grad ? 3 : 1), grad ? 10 : 9};
+    // potentials, whose terms cancel, carry what their additions round off
+    const MbmOut res{out, N * (grad ? 3 : 1), grad ? 10 : 9, grad ? nullptr : lo};
     MBM_CUDA_TRY(launch_frame(X, N, nullptr, frame, xh, xl, x4, nullptr, res, gate, ctx->d_flags,
                               s));
     auto kernel = p.stages == 8 ? contract64_kernel<8> : contract64_kernel<16>;
@@ -647,13 +650,13 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
             auto pass = grad ? pair64_kernel<true> : pair64_kernel<false>;
             pass<<<dim3(nt, kRows / (2 * kPairCols)), 256, 0, s>>>(
                 x4, xh, xl, (int)N, n_pad, n_blk, base_shift(p.stages), t0, near.tau,
-                ea + (size_t)b0 * n_pad, C, sign, out, gate);
+                ea + (size_t)b0 * n_pad, C, sign, out, lo, gate);
             MBM_CUDA_TRY(cudaGetLastError());
         }
     }
     MBM_CUDA_TRY(launch_near_triples(xh, xl, x4, N, near, nullptr,
-                                     grad ? MBM_NEAR_GRAD : MBM_NEAR_PHI, sign, out, ctx->num_sms,
-                                     gate, s));
+                                     grad ? MBM_NEAR_GRAD : MBM_NEAR_PHI, sign, out, lo,
+                                     ctx->num_sms, gate, s));
     MBM_CUDA_TRY(launch_unframe(X, N, frame, xh, xl, x4, res, gate, s));
     gate_out->gate = gate;
     gate_out->counter = counter;

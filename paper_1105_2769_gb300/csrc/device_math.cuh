@@ -73,6 +73,15 @@ __device__ __forceinline__ double inv_pow52d(double s) {
     return y2 * y2 * y;
 }
 
+// *v += x with what the addition rounds off going to *lo: v + lo does not depend on the
+// order of the additions (to eps^2).
+__device__ __forceinline__ void atomic_add_carried(double* v, double* lo, double x) {
+    const double a = atomicAdd(v, x);
+    const double s = __dadd_rn(a, x), b = __dsub_rn(s, a);
+    const double e = __dadd_rn(__dsub_rn(a, __dsub_rn(s, b)), __dsub_rn(x, b));
+    if (e != 0.0) atomicAdd(lo, e);
+}
+
 // Tile-pair item index t -> (J, K), J <= K, ordered by J descending so the
 // items with the most I tiles (I <= J) come first. Items with J' > J number
 // M(M+1)/2 with M = NT-1-J.

@@ -81,7 +81,10 @@ frame_kernel(const double* __restrict__ X, int64_t N, const double* __restrict__
         if (x4) x4[i] = make_double4_32a(y[0], y[1], y[2], 0.0);
         if (gs) gs[i] = scalbn(g[i], -w);
     }
-    for (int64_t i = first; i < out.n; i += step) out.v[i] = 0.0;
+    for (int64_t i = first; i < out.n; i += step) {
+        out.v[i] = 0.0;
+        if (out.lo) out.lo[i] = 0.0;
+    }
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -92,7 +95,8 @@ unframe_kernel(const double* __restrict__ X, int64_t N, const MbmFrame* __restri
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     if (!*gate) {
         const int e = out.degree * frame_exponent(frame) + weight_exponent(frame);
-        for (int64_t i = first; i < out.n; i += step) out.v[i] = scalbn(out.v[i], e);
+        for (int64_t i = first; i < out.n; i += step)
+            out.v[i] = scalbn(out.lo ? out.v[i] + out.lo[i] : out.v[i], e);
         return;
     }
     for (int64_t i = first; i < out.n; i += step) out.v[i] = 0.0;

@@ -18,6 +18,7 @@ struct MbmOut {
     double* v;
     int64_t n;    // numbers
     int degree;   // 9 for potentials, 10 for gradients
+    double* lo = nullptr;  // what the additions to v rounded off (NULL: not carried)
 };
 
 // The frame of X and the packed points in it: x4 = 2^e x (FP64), and xh + xl =
@@ -28,7 +29,7 @@ cudaError_t launch_frame(const double* X, int64_t N, const double* g, MbmFrame* 
                          float4* xl, double4_32a* x4, double* gs, const MbmOut& out, int* gate,
                          int* flags, cudaStream_t s);
 
-// Out of the frame: out times 2^(degree e) and the weights' unit. If *gate is set, zero
+// Out of the frame: out (with lo) times 2^(degree e) and the weights' unit. If *gate is set, zero
 // instead, and the points packed as they are (x4, or xh and xl), for the sweep behind.
 cudaError_t launch_unframe(const double* X, int64_t N, const MbmFrame* frame, float4* xh, float4* xl,
                            double4_32a* x4, const MbmOut& out, const int* gate, cudaStream_t s);

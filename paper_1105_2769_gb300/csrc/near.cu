@@ -220,7 +220,7 @@ near_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
             const double4_32a* __restrict__ x64, int N, const float* __restrict__ tau,
             const int2* __restrict__ pairs, const int* __restrict__ count,
             const double* __restrict__ g, double sign, double* __restrict__ out,
-            const int* __restrict__ gate) {
+            double* __restrict__ out_lo, const int* __restrict__ gate) {
     if (*gate) return;
     constexpr int kRow = Grad ? 6 : 1;   // shares of a and b
     constexpr int kCol = Grad ? 3 : 1;
@@ -377,6 +377,10 @@ near_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
                 if constexpr (Grad) {
                     const int o = d < 3 ? np[threadIdx.x].i : np[threadIdx.x].j;
                     atomicAdd(&out[3 * (size_t)o + d % 3], sign * t);
+                } else if constexpr (sizeof(R) == 8) {
+                    const int i = np[threadIdx.x].i, j = np[threadIdx.x].j;
+                    atomic_add_carried(&out[i], &out_lo[i], t);
+                    atomic_add_carried(&out[j], &out_lo[j], t);
                 } else {
                     atomicAdd(&out[np[threadIdx.x].i], t);
                     atomicAdd(&out[np[threadIdx.x].j], t);
@@ -388,6 +392,7 @@ near_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
 #pragma unroll
         for (int d = 0; d < kCol; ++d)
             if constexpr (Grad) atomicAdd(&out[3 * (size_t)k + d], sign * col[d]);
+            else if constexpr (sizeof(R) == 8) atomic_add_carried(&out[k], &out_lo[k], col[d]);
             else atomicAdd(&out[k], col[d]);
     }
 }
@@ -440,8 +445,8 @@ cudaError_t launch_near_list(const float4* xh, const float4* xl, int64_t N, void
 
 cudaError_t launch_near_triples(const float4* xh, const float4* xl, const double4_32a* X64,
                                 int64_t N, const MbmNear& near, const double* g, int what,
-                                double sign, double* out, int num_sms, const int* gate,
-                                cudaStream_t s) {
+                                double sign, double* out, double* out_lo, int num_sms,
+                                const int* gate, cudaStream_t s) {
     const unsigned bx = (unsigned)((N + kNearWarps * 32 - 1) / (kNearWarps * 32));
     // about 2 N pairs; enough CTAs for eight per SM, at least one chunk each
     const int64_t chunks = (2 * N + kChunk - 1) / kChunk;
@@ -452,17 +457,17 @@ cudaError_t launch_near_triples(const float4* xh, const float4* xl, const double
     if (what == MBM_NEAR_PHI) {
         if (X64)
             near_kernel<double, false><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, out_lo, gate);
         else
             near_kernel<float, false><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, out_lo, gate);
     } else {
         if (X64)
             near_kernel<double, true><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, out_lo, gate);
         else
             near_kernel<float, true><<<grid, threads, 0, s>>>(
-                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, gate);
+                xh, xl, X64, (int)N, near.tau, near.pairs, near.count, g, sign, out, out_lo, gate);
     }
     return cudaGetLastError();
 }

@@ -32,11 +32,11 @@ enum : int { MBM_NEAR_PHI = 0, MBM_NEAR_GRAD = 1 };
 
 // Adds the triples with at least one near pair: potentials to out[N], or
 // sign * w_t grad phi to out[3 N] (w_t = g_a + g_b + g_c, 1 without g).
-// Nothing if *gate is set. X64: NULL = FP32 terms from xh/xl, else FP64 from these points.
+// Nothing if *gate is set. out_lo: carries of FP64 potentials. X64: NULL = FP32 terms from xh/xl, else FP64 from these points.
 cudaError_t launch_near_triples(const float4* xh, const float4* xl, const double4_32a* X64,
                                 int64_t N, const MbmNear& near, const double* g, int what,
-                                double sign, double* out, int num_sms, const int* gate,
-                                cudaStream_t s);
+                                double sign, double* out, double* out_lo, int num_sms,
+                                const int* gate, cudaStream_t s);
 
 // The test itself, on the device.
 __device__ __forceinline__ bool mbm_is_near(float s, float tau_a, float tau_b) {
