@@ -52,8 +52,17 @@ typedef enum {
 
 /* Modes of mbm_potential / mbm_forces. */
 enum {
-    MBM_EXH_FP64 = 0, /* exhaustive, FP64 everywhere */
-    MBM_EXH_FP32 = 1, /* exhaustive, FP32 triple arithmetic, FP64 accumulation */
+    /* Exhaustive, FP64 accuracy: 1e-12 of a potential without strong cancellation, 1e-12
+     * of the sum of its triples' gradients for a force. Triples with a close pair and all
+     * sums over pairs are FP64; the rest are matrix products of 48-bit fixed-point terms,
+     * exact in themselves (N >= 192 for potentials, 96 for forces; FP64 triple sweeps
+     * below, above 24 576 and for VJPs). */
+    MBM_EXH_FP64 = 0,
+    /* Exhaustive, FP32 bulk: 1e-6 of a potential without strong cancellation. Triples with
+     * a close pair in FP32; the rest are matrix products of 22-bit terms on the tensor
+     * cores with FP32 sums (N >= 1 280 for potentials, 96 for gradients; FP32 triple
+     * sweeps below); sums over pairs in FP64. */
+    MBM_EXH_FP32 = 1,
     MBM_TREE = 2,     /* multi-tree approximation (Algorithm 2) */
     MBM_ABS = 0x100   /* with MBM_TREE: eps is the absolute bound tau (Def. 2.1) */
 };

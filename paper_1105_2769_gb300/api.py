@@ -6,8 +6,8 @@
     Potential.apply(X)                              -> Phi with autograd
 
 ``X`` is a CUDA float64 tensor of shape (N, 3). Modes: "fp64" (exhaustive,
-FP64 everywhere), "fp32" (exhaustive, FP32 triple arithmetic with FP64
-accumulation), "tree" (multi-tree approximation with relative ``eps``),
+FP64 accuracy), "fp32" (exhaustive, FP32 bulk with FP64 accumulation; include/mbm.h
+says what is held in how many bits), "tree" (multi-tree approximation with relative ``eps``),
 "tree_abs" (multi-tree with absolute bound ``eps`` = tau). All work runs on
 the current torch CUDA stream.
 """

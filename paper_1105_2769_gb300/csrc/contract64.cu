@@ -11,7 +11,11 @@
 // 1.5 2^23 and adds it to a 64-bit fixed-point sum at its weight; products below
 // 2^-48 are left out. The 64-bit sums of a block are converted, scaled and added in FP64 by
 // the pair pass. Error of the contraction: 4e-17 of a potential (norm, N = 300);
-// with the near triples the result is as close to 64 bits as the FP64 sweep's.
+// with the near triples the result is as close to 64 bits as the FP64 sweep's (norm
+// and median at or below it for N = 100 to 3 001, unit, uniform and mixture sets). An
+// entry far below its row's largest within a block keeps fewer bits than FP64 would:
+// beside a group of six at 1e-3 of the spacing of 3 000 others, forces lose to 3e-14
+// (median; 7e-13 at worst), potentials stay below the sweep's 1e-12.
 //
 // Range. FP32 carries the near test and the exponents, so the points are brought to
 // a common unit first (frame.h): |x - x_0| < 2^11. With r >= 2^-19 there, every FP32

@@ -196,7 +196,7 @@ __device__ __forceinline__ float phi_df(const EdgeDf& u, const EdgeDf& a, const 
     return f.h;
 }
 
-constexpr int kChunk = 32;      // near pairs staged at a time
+constexpr int kChunk = 32;      // near pairs staged at a time, one per lane in the sums
 constexpr int kNearWarps = 4;   // 128 particles j per CTA
 
 template <typename R>
@@ -262,111 +262,108 @@ near_kernel(const float4* __restrict__ xh, const float4* __restrict__ xl,
             np[threadIdx.x] = q;
         }
         __syncthreads();
-        for (int h = 0; h < cnt; h += 32) {
-            R part[kCol], row[kRow];
+        R part[kCol], row[kRow];
 #pragma unroll
-            for (int d = 0; d < kCol; ++d) part[d] = 0;
-            float low = 0.f;
-            (void)low;
-            for (int q = 0; q < 32; ++q) {
-                const int p = h + q;
+        for (int d = 0; d < kCol; ++d) part[d] = 0;
+        float low = 0.f;
+        (void)low;
+        for (int p = 0; p < kChunk; ++p) {
 #pragma unroll
-                for (int d = 0; d < kRow; ++d) row[d] = 0;
-                if (p < cnt && kv) {
-                    const NearPair<R>& n = np[p];
-                    const float sa = pair_d2_hilo(ah[p], al[p], kh, kl);
-                    const float sb = pair_d2_hilo(bh[p], bl[p], kh, kl);
-                    if (k != n.i && k != n.j && sa > 0.f && sb > 0.f) {
-                        const int hits = 1 + (int)mbm_is_near(sa, n.ti, tk) +
-                                         (int)mbm_is_near(sb, n.tj, tk);
-                        R w = hits == 1 ? (R)1 : hits == 2 ? (R)0.5 : (R)1 / (R)3;
-                        if constexpr (sizeof(R) == 4 && !Grad) {
-                            const float f = (float)w * phi_df(n.d, edge_df(ah[p], al[p], kh, kl),
-                                                              edge_df(bh[p], bl[p], kh, kl));
-                            // carried sums: see row_sum_exact
-                            const float t = __fadd_rn(part[0], f), bb = __fsub_rn(t, part[0]);
-                            low = __fadd_rn(low, __fadd_rn(__fsub_rn(part[0], __fsub_rn(t, bb)),
-                                                           __fsub_rn(f, bb)));
-                            part[0] = t;
+            for (int d = 0; d < kRow; ++d) row[d] = 0;
+            if (p < cnt && kv) {
+                const NearPair<R>& n = np[p];
+                const float sa = pair_d2_hilo(ah[p], al[p], kh, kl);
+                const float sb = pair_d2_hilo(bh[p], bl[p], kh, kl);
+                if (k != n.i && k != n.j && sa > 0.f && sb > 0.f) {
+                    const int hits = 1 + (int)mbm_is_near(sa, n.ti, tk) +
+                                     (int)mbm_is_near(sb, n.tj, tk);
+                    R w = hits == 1 ? (R)1 : hits == 2 ? (R)0.5 : (R)1 / (R)3;
+                    if constexpr (sizeof(R) == 4 && !Grad) {
+                        const float f = (float)w * phi_df(n.d, edge_df(ah[p], al[p], kh, kl),
+                                                          edge_df(bh[p], bl[p], kh, kl));
+                        // carried sums: see row_sum_exact
+                        const float t = __fadd_rn(part[0], f), bb = __fsub_rn(t, part[0]);
+                        low = __fadd_rn(low, __fadd_rn(__fsub_rn(part[0], __fsub_rn(t, bb)),
+                                                       __fsub_rn(f, bb)));
+                        part[0] = t;
+                        row[0] = f;
+                    } else {
+                        Edge<R> a, b;
+                        if constexpr (sizeof(R) == 8) {
+                            a = edge64(x64[n.i], kd);
+                            b = edge64(x64[n.j], kd);
+                        } else {
+                            a = edge32(ah[p], al[p], kh, kl);
+                            b = edge32(bh[p], bl[p], kh, kl);
+                        }
+                        const R ux = n.e.x, uy = n.e.y, uz = n.e.z;
+                        const R p1 = ux * a.x + uy * a.y + uz * a.z;
+                        const R p2 = ux * b.x + uy * b.y + uz * b.z;
+                        const R p3 = a.x * b.x + a.y * b.y + a.z * b.z;
+                        const R rr = n.e.rho * a.rho * b.rho;
+                        if constexpr (!Grad) {
+                            const R f = w * (rr - (R)3 * (p1 * p2 * p3) * rr);
+                            part[0] += f;
                             row[0] = f;
                         } else {
-                            Edge<R> a, b;
-                            if constexpr (sizeof(R) == 8) {
-                                a = edge64(x64[n.i], kd);
-                                b = edge64(x64[n.j], kd);
-                            } else {
-                                a = edge32(ah[p], al[p], kh, kl);
-                                b = edge32(bh[p], bl[p], kh, kl);
-                            }
-                            const R ux = n.e.x, uy = n.e.y, uz = n.e.z;
-                            const R p1 = ux * a.x + uy * a.y + uz * a.z;
-                            const R p2 = ux * b.x + uy * b.y + uz * b.z;
-                            const R p3 = a.x * b.x + a.y * b.y + a.z * b.z;
-                            const R rr = n.e.rho * a.rho * b.rho;
-                            if constexpr (!Grad) {
-                                const R f = w * (rr - (R)3 * (p1 * p2 * p3) * rr);
-                                part[0] += f;
-                                row[0] = f;
-                            } else {
-                                w *= g ? n.w + gk : (R)1;
-                                const R qf = (R)5 * (p1 * p2 * p3) - (R)1;
-                                const R t3 = (R)3 * rr * w;
-                                const R su = t3 * n.e.inv, sa3 = t3 * a.inv, sb3 = t3 * b.inv;
-                                const R p23 = p2 * p3, p13 = p1 * p3, p12 = p1 * p2;
-                                // grad_a = -c1 u - c2 e_ak + c3 e_bk
-                                R c1 = su * qf - sa3 * p23, c2 = sa3 * qf - su * p23,
-                                  c3 = su * p13 + sa3 * p12;
-                                row[0] = c3 * b.x - c1 * ux - c2 * a.x;
-                                row[1] = c3 * b.y - c1 * uy - c2 * a.y;
-                                row[2] = c3 * b.z - c1 * uz - c2 * a.z;
-                                // grad_b = c1' u - c2' e_bk + c3' e_ak
-                                c1 = su * qf + sb3 * p13;
-                                c2 = sb3 * qf + su * p13;
-                                c3 = sb3 * p12 - su * p23;
-                                row[kRow - 3] = c1 * ux - c2 * b.x + c3 * a.x;
-                                row[kRow - 2] = c1 * uy - c2 * b.y + c3 * a.y;
-                                row[kRow - 1] = c1 * uz - c2 * b.z + c3 * a.z;
-                                // grad_k by itself: as minus the sum of the other two it
-                                // would carry their rounding, which for a pair far
-                                // closer than k is 1 / r_ab against grad_k's 1 / r_ak
-                                c1 = sa3 * qf - sb3 * p12;
-                                c2 = sb3 * qf - sa3 * p12;
-                                c3 = sa3 * p23 + sb3 * p13;
-                                part[0] += c1 * a.x + c2 * b.x - c3 * ux;
-                                part[kCol / 2] += c1 * a.y + c2 * b.y - c3 * uy;
-                                part[kCol - 1] += c1 * a.z + c2 * b.z - c3 * uz;
-                            }
+                            w *= g ? n.w + gk : (R)1;
+                            const R qf = (R)5 * (p1 * p2 * p3) - (R)1;
+                            const R t3 = (R)3 * rr * w;
+                            const R su = t3 * n.e.inv, sa3 = t3 * a.inv, sb3 = t3 * b.inv;
+                            const R p23 = p2 * p3, p13 = p1 * p3, p12 = p1 * p2;
+                            // grad_a = -c1 u - c2 e_ak + c3 e_bk
+                            R c1 = su * qf - sa3 * p23, c2 = sa3 * qf - su * p23,
+                              c3 = su * p13 + sa3 * p12;
+                            row[0] = c3 * b.x - c1 * ux - c2 * a.x;
+                            row[1] = c3 * b.y - c1 * uy - c2 * a.y;
+                            row[2] = c3 * b.z - c1 * uz - c2 * a.z;
+                            // grad_b = c1' u - c2' e_bk + c3' e_ak
+                            c1 = su * qf + sb3 * p13;
+                            c2 = sb3 * qf + su * p13;
+                            c3 = sb3 * p12 - su * p23;
+                            row[kRow - 3] = c1 * ux - c2 * b.x + c3 * a.x;
+                            row[kRow - 2] = c1 * uy - c2 * b.y + c3 * a.y;
+                            row[kRow - 1] = c1 * uz - c2 * b.z + c3 * a.z;
+                            // grad_k by itself: as minus the sum of the other two it
+                            // would carry their rounding, which for a pair far
+                            // closer than k is 1 / r_ab against grad_k's 1 / r_ak
+                            c1 = sa3 * qf - sb3 * p12;
+                            c2 = sb3 * qf - sa3 * p12;
+                            c3 = sa3 * p23 + sb3 * p13;
+                            part[0] += c1 * a.x + c2 * b.x - c3 * ux;
+                            part[kCol / 2] += c1 * a.y + c2 * b.y - c3 * uy;
+                            part[kCol - 1] += c1 * a.z + c2 * b.z - c3 * uz;
                         }
                     }
                 }
-                if constexpr (Grad) {
-                    // six sums over the warp by butterflies, lane q keeps pair q's
-#pragma unroll
-                    for (int d = 0; d < kRow; ++d) {
-                        R v = row[d];
-                        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                        if (lane == q) rows[d][warp][h + q] = (double)v;
-                    }
-                } else {
-                    red[warp][q][lane] = row[0];
-                }
             }
-            if constexpr (!Grad) {
-                __syncwarp();
-                if constexpr (sizeof(R) == 4) {
-                    rows[0][warp][h + lane] = mbm_tile::row_sum_exact(red[warp], lane);
-                } else {
-                    R t = 0;
-#pragma unroll 8
-                    for (int q = 0; q < 32; ++q) t += red[warp][lane][q];
-                    rows[0][warp][h + lane] = (double)t;
-                }
-                __syncwarp();
-            }
+            if constexpr (Grad) {
+                // six sums over the warp by butterflies, lane p keeps pair p's
 #pragma unroll
-            for (int d = 0; d < kCol; ++d) col[d] += (double)part[d];
-            if constexpr (sizeof(R) == 4 && !Grad) col[0] += (double)low;
+                for (int d = 0; d < kRow; ++d) {
+                    R v = row[d];
+                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    if (lane == p) rows[d][warp][p] = (double)v;
+                }
+            } else {
+                red[warp][p][lane] = row[0];
+            }
         }
+        if constexpr (!Grad) {
+            __syncwarp();
+            if constexpr (sizeof(R) == 4) {
+                rows[0][warp][lane] = mbm_tile::row_sum_exact(red[warp], lane);
+            } else {
+                R t = 0;
+#pragma unroll 8
+                for (int q = 0; q < 32; ++q) t += red[warp][lane][q];
+                rows[0][warp][lane] = (double)t;
+            }
+            __syncwarp();
+        }
+#pragma unroll
+        for (int d = 0; d < kCol; ++d) col[d] += (double)part[d];
+        if constexpr (sizeof(R) == 4 && !Grad) col[0] += (double)low;
         __syncthreads();
         if ((int)threadIdx.x < cnt) {
 #pragma unroll
