@@ -45,9 +45,10 @@ N_MAIN = 32768
 # same for potentials and forces.
 FLOPS_PER_TRIPLE_CONTRACT = 180
 FP32_LANES_PER_SM = 128
-# Kernels of one FP32-bulk solve of N_MAIN particles (launch list in
-# profiles/contract_n32768_launches.md).
-LAUNCHES_PER_STEP = 220
+# Kernels of one FP32-bulk solve of N_MAIN particles, counted in the launch list of
+# profiles/contract_n32768_launches.md (they depend on N alone: 2 of the frame, 7 of the
+# near list, 8 slabs of 4 and of 11 batches of 2 each, 1 reference, 4 at the end).
+LAUNCHES_PER_STEP = 222
 N_CONFIG3 = 1 << 20
 
 
@@ -264,6 +265,8 @@ def contract_roofline(rate):
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if peak else None, "kernel": "contract_kernel",
             "flops_per_triple": FLOPS_PER_TRIPLE_CONTRACT, "traffic": None,
+            "traffic_note": "5.8 GB of DRAM per contraction launch (4 096 columns) at N = 8 192, "
+                            "12 % of its throughput (profiles/contract_n8192_full.md)",
             "peak_note": "measured cuBLAS bf16 GEMM, sustained; time is the whole solve's kernels "
                          "(near triples, tables, contraction, pair pass)"}
 
