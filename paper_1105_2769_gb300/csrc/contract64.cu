@@ -13,9 +13,10 @@
 // the pair pass. Error of the contraction: 4e-17 of a potential (norm, N = 300);
 // with the near triples the result is as close to 64 bits as the FP64 sweep's (norm
 // and median at or below it for N = 100 to 3 001, unit, uniform and mixture sets). An
-// entry far below its row's largest within a block keeps fewer bits than FP64 would:
-// beside a group of six at 1e-3 of the spacing of 3 000 others, forces lose to 3e-14
-// (median; 7e-13 at worst), potentials stay below the sweep's 1e-12.
+// entry far below its row's largest within a block keeps fewer bits than FP64 would,
+// so pairs of a tight group are near pairs (near.cu): beside 30 points within 1e-3 of
+// the spacing of 8 000 others, potentials were off by 2.1e-12 of sum|phi| and forces by
+// 1.2e-12 of sum|grad phi|, and are by 5e-16.
 //
 // Range. FP32 carries the near test and the exponents, so the points are brought to
 // a common unit first (frame.h): |x - x_0| < 2^11. With r >= 2^-19 there, every FP32
@@ -539,6 +540,10 @@ constexpr float kMinDist2 = 3.637979e-12f;  // 2^-38
 
 // Largest N that was measured (7 s a solve).
 constexpr int64_t kMaxN64 = 24576;
+// Smallest N whose near list looks for tight groups: what a group costs the others grows
+// with N (1.3e-13 of sum|grad phi| at N = 3 000, 1.2e-12 at 8 000), the search takes three
+// launches.
+constexpr int64_t kGroupsMinN = 2048;
 
 // Scratch layout of one solve. The digit table takes 140 bytes per pair of
 // particles (58 GB at N = 20 000), so the columns k go in slabs whose table stays
@@ -638,6 +643,7 @@ mbm_status mbm_contract64(mbm_ctx* ctx, const double* X, int64_t N, int what, do
     near.X = X;
     near.min_d2 = kMinDist2;
     near.excess = counter + 1;
+    near.groups = N > kGroupsMinN;
     MBM_CUDA_TRY(launch_near_list(xh, xl, N, near_mem, gate, ctx->d_flags, &near, s));
     exponent_kernel<<<dim3(n_pad / 256, p.n_blk), 256, 0, s>>>(xh, xl, (int)N, p.cols, near.tau,
                                                               n_pad, ea, gate);

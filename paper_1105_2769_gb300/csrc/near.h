@@ -20,6 +20,8 @@ struct MbmNear {
     const double* X = nullptr;
     float min_d2 = 0.f;
     unsigned long long* excess = nullptr;  // zeroed word for the count, or NULL
+    // Pairs far closer than the usual third neighbour are near too (raises tau).
+    bool groups = false;
 };
 
 // Thresholds and the ordered list of near pairs, in `mem` (mbm_near_bytes).
