@@ -61,7 +61,9 @@ enum {
     /* Exhaustive, FP32 bulk: 1e-6 of a potential without strong cancellation. Triples with
      * a close pair in FP32; the rest are matrix products of 22-bit terms on the tensor
      * cores with FP32 sums (N >= 1 280 for potentials, 96 for gradients; FP32 triple
-     * sweeps below); sums over pairs in FP64. */
+     * sweeps below); sums over pairs in FP64. A set whose closest pair is less than about
+     * 3e-7 of its extent is solved by those sweeps too, whose terms (r^-9, r^-10, and r^-6
+     * of a pair) are in the caller's unit and have to stay in FP32's range. */
     MBM_EXH_FP32 = 1,
     MBM_TREE = 2,     /* multi-tree approximation (Algorithm 2) */
     MBM_ABS = 0x100   /* with MBM_TREE: eps is the absolute bound tau (Def. 2.1) */

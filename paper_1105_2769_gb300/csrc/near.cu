@@ -259,8 +259,8 @@ struct NearPair {
 // A CTA owns 128 particles k, one per lane, and every gridDim.y-th chunk of near
 // pairs (a, b). k's share stays in registers; the shares of a and b are summed
 // over the lanes through a transposed buffer, 32 pairs at a time. Bound by FP32
-// instructions (FMA pipe 73 %, issue 83 %, 1.7 ms at N = 8 192) or, in FP64, by that
-// pipe. Chunks of 32 pairs, not 64 or more: N = 700 has only 1 400 pairs for the
+// instructions (FMA pipe 71 %, issue 82 %, 1.7 ms at N = 8 192) or, in FP64, by that
+// pipe; FP32 gradients by the conversions of their sums to FP64 (pipe 82 %, 1.6 ms). Chunks of 32 pairs, not 64 or more: N = 700 has only 1 400 pairs for the
 // whole chip.
 template <typename R, bool Grad>
 __global__ void __launch_bounds__(kNearWarps * 32)
